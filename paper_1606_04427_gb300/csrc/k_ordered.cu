@@ -40,15 +40,6 @@ struct __align__(16) OWarpSmem {
     uint64_t bar[2];
 };
 
-__device__ __forceinline__ int find_tile_o(const int *__restrict__ item_off, int N, int item) {
-    int a = 0, b = N - 1;  // last gt with item_off[gt] <= item
-    while (a < b) {
-        const int m = (a + b + 1) >> 1;
-        if (__ldg(&item_off[m]) <= item) a = m; else b = m - 1;
-    }
-    return a;
-}
-
 // A record whose largest x = s E w (w <= 1) is small takes a series path: with
 // phi(x) = (1 - exp(-x)) / x = sum_k (-x)^k / (k + 1)!, a = 1 - x phi and b = E w phi, no
 // exponential per channel.  phi to degree 2 where x <= kSeries2Max (next term x^3 / 24
@@ -133,7 +124,6 @@ __global__ void __launch_bounds__(kOWarps * 32, 4)
     OWarpSmem *ws = reinterpret_cast<OWarpSmem *>(s_raw) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     const int nt = fr.n_tiles;
-    const int N = fr.V * nt;
     const int S2 = split * split;
     const int total_items = (int)fr.sizes[kSizeItems] * S2;
     const int64_t K = fr.sizes[kSizeK];
@@ -157,10 +147,9 @@ __global__ void __launch_bounds__(kOWarps * 32, 4)
         if (item >= total_items) break;
 
         const int qs = item / S2, q = item - qs * S2;
-        const int slice = fr.order ? __ldg(&fr.order[qs]) : qs;  // largest slices first
-        const int gt = find_tile_o(fr.item_off, N, slice);
+        const int2 ord = __ldg(&fr.order[qs]);  // largest slices first
+        const int gt = ord.x, chunk = ord.y, slice = fr.item_off[gt] + chunk;
         const int v = gt / nt, t = gt - v * nt;
-        const int chunk = slice - fr.item_off[gt];
         const int arrivals = (fr.item_off[gt + 1] - fr.item_off[gt]) * S2;
         const int slot = fr.split_slot[gt];
         const float kexp = fr.views[v].kexp;

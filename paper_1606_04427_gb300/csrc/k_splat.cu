@@ -5,40 +5,44 @@
 // draw adds particle colour x scalar weight to the pixel.  Section 2.1: the weight is
 // a Gaussian of the distance to the particle centre over the radius-dependent area.
 //
-// GB300 layout: persistent CTAs pull work items from a queue.  A work item is a tile,
-// or a K-record slice of a crowded tile (so dense clusters do not serialise on one
-// worker); slices of a split tile add their partial sums into a scratch tile and the
-// last slice to finish writes the result.  Records are staged from HBM into shared
-// memory by bulk copies (cp.async.bulk, double buffered, mbarrier completion with a
-// bounded wait).  The paper's worker is a thread; here pixels are owned by lanes, each
-// accumulating its pixels in registers (no atomics: a pixel has exactly one owner), in
-// blocks of 8 x 4 pixels, one pixel of each block per lane.  Two kernels:
-//   k_splat_warp  tiles up to 32 px: one warp owns a square of up to 16 x 16 pixels (a
-//                 tile, or a quarter of a larger one) and runs its records grouped by
-//                 the rectangle of blocks they cover (below);
-//   k_splat       tiles above 32 px: the 8 warps of a CTA share a tile by block rows,
-//                 each record queued to the warps whose rows it meets.
-// In clustered data most pixels receive hundreds of contributions per frame, where a
-// shared-memory scatter would serialise on atomic conflicts.
+// GB300 layout: persistent warps pull work items from a queue.  A work item is a region of
+// up to 16 x 16 pixels (a tile, or one of the split x split regions of a tile above 16 px)
+// and a tile list, or a K-record slice of a crowded tile's list; slices of a split tile add
+// their partial sums into an exact scratch tile and the last one to finish writes the
+// result.  Warps never wait on one another.
+//
+// What a warp does with an item.  The kernel is bound by instruction issue and the latency
+// between its phases (the records are read once, DRAM is nearly idle), so the layout is
+// chosen for few instructions per covered pixel and per record:
+//   1. fill: records are read 32 at a time from the list (kAhead copies ahead, through a ring
+//      in shared memory); those whose support meets the region are appended to a batch;
+//   2. decode, one record per lane: the 4 x 4-pixel squares (16 of them) its box meets, its
+//      colour (colormap, or the particle's emission) and Gaussian scale.  Ballots give every
+//      square a word of records per 32;
+//   3. lists: per square, the batch positions of its records, unpacked from the words by two
+//      lanes per square;
+//   4. passes: a square is evaluated by a pair of lanes, 2 x 4 pixels each in packed FP32x2
+//      arithmetic, so 16 records are in flight per warp instruction.  The squares are taken
+//      longest list first, 16 at a time, or fewer with 2^a lane pairs each where the lists are
+//      unequal (the pairs of a square then split its list and their sums are added by
+//      shuffles).  Sums stay in registers for a pass and are added to the region's accumulator
+//      in shared memory.
+// Squares of a pass are distinct and passes are in order, so no pixel is ever updated by two
+// lanes at once and the summation order depends only on the list's order.
+//
+// Why 4 x 4 squares and two lanes each: a particle of the two-species benchmark set covers 50
+// pixels in 6.7 such squares (107 lane evaluations, against 142 in 8 x 4 blocks with a warp per
+// record), a step of the pass loop serves 16 records instead of one, and the small records,
+// most of a list, no longer cost a whole warp each.  The 10 M-particle frame at 2048^2 takes
+// 500 M warp instructions (792 M with a warp per record), the 100 M-particle frame 5.75 ms
+// (7.35), 10 M close particles at 4096^2 4.5 ms (5.2), 1 M at 637 x 483 119 us (195), 100 k at
+// 256^2 48 us (107).  Batches of 192: 128 balance worse (6.2 ms), 224 leave 14 warps per SM
+// instead of 16 (6.7 ms); scalar instead of packed arithmetic: 18 more instructions per step
+// (6.5 ms against 6.1 before the loop was unrolled); unrolling by 3 drops the copies of the
+// prefetched record (6.1 -> 5.75 ms).
 #include "splotch_internal.cuh"
 
 namespace spl {
-
-// ---------------------------------------------------------------------------------------
-// CTA-per-item splat for tiles above 32 px.  Per stage of kStage records:
-//   1. decode: one thread per record computes the record's pixel box inside the tile, its
-//      colour (brightness x colormap, or the particle's emission) and Gaussian scale, and
-//      appends the record to the list of every warp owning a block row the box meets
-//      (block row r: warp r mod 8);
-//   2. gather: each warp walks its list; for every block of its own that the box
-//      overlaps, each lane tests its pixel with the FP32 coverage rule and adds e * w
-//      to its registers.
-
-struct __align__(16) Rec {
-    int ilo, ihi, jlo, jhi;  // tile-local box
-    float X, Y, R2, kr;
-    float er, eg, eb, pad;
-};
 
 __device__ __forceinline__ int find_tile(const int *__restrict__ item_off, int N, int item) {
     int a = 0, b = N - 1;  // last gt with item_off[gt] <= item
@@ -49,414 +53,58 @@ __device__ __forceinline__ int find_tile(const int *__restrict__ item_off, int N
     return a;
 }
 
-// blocks of 8 x 4 pixels; warp w owns block rows w, w + 8, ...: NR block rows of NC
-// blocks each (NC = ceil(T / 8), NR = ceil(ceil(T / 4) / 8))
-__host__ __device__ __forceinline__ int block_cols(int T) { return (T + 7) >> 3; }
-__host__ __device__ __forceinline__ int block_rows_per_warp(int T) {
-    return (((T + 3) >> 2) + kSplatWarps - 1) / kSplatWarps;
-}
-
-size_t splat_smem_bytes(int) {
-    return sizeof(float4) * 2 * kStage + sizeof(Rec) * kStage + sizeof(short) * kSplatWarps * kStage;
-}
-
-// pixel centre coordinate that no support reaches (its square overflows to +inf)
-constexpr float kFar = 1e30f;
-
 // Output of a pixel's accumulation a: mode 0 writes 1 - exp(-a) (final transform),
 // 1 writes a, 2 adds a to what the pixel holds (several renders summed in one image).
 __device__ __forceinline__ void put_pixel(float *p, float a, int mode) {
     *p = mode == 2 ? *p + a : (mode ? a : -expm1f(-a));
 }
 
-template <int NR, int NC>
-__global__ void __launch_bounds__(kSplatThreads, 3) k_splat(SceneDev sc, FrameDev fr, int *queue, float *out,
-                                                         int out_accum) {
-    if (fr.status[kStatOverflow] || fr.status[kStatTimeout]) return;  // no complete tile lists
-    extern __shared__ __align__(16) unsigned char s_raw[];
-    __shared__ uint64_t s_bar[2];
-    __shared__ int s_item, s_last;
-
-    float4 *s_buf = reinterpret_cast<float4 *>(s_raw);             // [2][kStage]
-    Rec *s_rec = reinterpret_cast<Rec *>(s_buf + 2 * kStage);       // [kStage]
-    short *s_wl = reinterpret_cast<short *>(s_rec + kStage);        // [warps][kStage]
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nt = fr.n_tiles;
-    const int N = fr.V * nt;
-    const int total_items = (int)fr.sizes[kSizeItems];
-    const int64_t K = fr.sizes[kSizeK];
-    const ViewParams g0 = fr.views[0];
-    const int T = g0.T, W = g0.W, H = g0.H, ntx = g0.ntx;
-    const int lc = lane & 7, lr = lane >> 3;
-
-    if (tid == 0) {
-        mbar_init(&s_bar[0], 1);
-        mbar_init(&s_bar[1], 1);
-        mbar_fence_init();
-    }
-    __syncthreads();
-    uint32_t phase0 = 0, phase1 = 0;
-
-    for (;;) {
-        if (tid == 0) s_item = atomicAdd(queue, 1);
-        __syncthreads();
-        const int qi = s_item;
-        if (qi >= total_items) break;
-        const int item = fr.order ? __ldg(&fr.order[qi]) : qi;
-
-        const int gt = find_tile(fr.item_off, N, item);
-        const int v = gt / nt, t = gt - v * nt;
-        const int chunk = item - fr.item_off[gt];
-        const int n_it = fr.item_off[gt + 1] - fr.item_off[gt];
-        const int slot = fr.split_slot[gt];
-        const float kexp = fr.views[v].kexp;
-        const int tx = t % ntx, ty = t / ntx;
-        const int px0 = tx * T, py0 = ty * T;
-        const int tw = min(T, W - px0), th = min(T, H - py0);
-        const int64_t seg1 = fr.offsets[gt + 1];
-        const int64_t e0 = fr.offsets[gt] + (int64_t)chunk * K;
-        const int nrec = (int)(min(seg1, e0 + K) - e0);
-        const int nst = (nrec + kStage - 1) / kStage;
-
-        // this lane's pixels: column c * 8 + lc of block row warp + 8 rr (tile rows
-        // 4 (warp + 8 rr) + lr); pixels outside the tile get a centre no support reaches
-        float fx[NC], fy[NR], ar[NR][NC], ag[NR][NC], ab[NR][NC];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fx[c] = c * 8 + lc < tw ? (float)(px0 + c * 8 + lc) + 0.5f : kFar;
-#pragma unroll
-        for (int rr = 0; rr < NR; ++rr) {
-            const int row = 4 * (warp + kSplatWarps * rr) + lr;
-            fy[rr] = row < th ? (float)(py0 + row) + 0.5f : kFar;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) ar[rr][c] = ag[rr][c] = ab[rr][c] = 0.0f;
-        }
-
-        if (tid == 0 && nrec > 0) {
-            const int c0 = min(kStage, nrec);
-            fence_proxy_async_smem();
-            mbar_arrive_expect_tx(&s_bar[0], (uint32_t)c0 * 16u);
-            bulk_g2s(s_buf, fr.lists + e0, (uint32_t)c0 * 16u, &s_bar[0]);
-        }
-
-        for (int si = 0; si < nst; ++si) {
-            const int cb = si & 1;
-            if (tid == 0 && si + 1 < nst) {
-                const int nb = (si + 1) & 1;
-                const int cn = min(kStage, nrec - (si + 1) * kStage);
-                fence_proxy_async_smem();
-                mbar_arrive_expect_tx(&s_bar[nb], (uint32_t)cn * 16u);
-                bulk_g2s(s_buf + nb * kStage, fr.lists + e0 + (int64_t)(si + 1) * kStage,
-                         (uint32_t)cn * 16u, &s_bar[nb]);
-            }
-            const bool ok = mbar_wait_bounded(&s_bar[cb], cb ? phase1 : phase0, kWaitCycles);
-            if (cb) phase1 ^= 1u; else phase0 ^= 1u;
-            if (__syncthreads_or(!ok)) {
-                if (tid == 0) atomicExch(&fr.status[kStatTimeout], 1);
-                return;
-            }
-            const int cnt = min(kStage, nrec - si * kStage);
-            const float4 *recs = s_buf + cb * kStage;
-
-            // ---- 1. decode; queue each record to the warps owning the block rows it meets
-            for (int idx = tid; idx < cnt; idx += kSplatThreads) {
-                const float4 rec = recs[idx];
-                const float X = rec.x, Y = rec.y, R = rec.z;
-                const uint32_t code = __float_as_uint(rec.w);
-                // tight pixel range of the support inside the tile; eps exceeds the FP32
-                // rounding of X +- R at any position, so no covered pixel is left out
-                const float eps = 1e-3f + 2e-6f * (fabsf(X) + fabsf(Y) + R);
-                const int ilo = max(px0, (int)ceilf(clampf(X - R - 0.5f - eps, px0 - 1.0f, (float)(px0 + tw))));
-                const int ihi = min(px0 + tw - 1, (int)floorf(clampf(X + R - 0.5f + eps, px0 - 1.0f, (float)(px0 + tw))));
-                const int jlo = max(py0, (int)ceilf(clampf(Y - R - 0.5f - eps, py0 - 1.0f, (float)(py0 + th))));
-                const int jhi = min(py0 + th - 1, (int)floorf(clampf(Y + R - 0.5f + eps, py0 - 1.0f, (float)(py0 + th))));
-                if (ilo > ihi || jlo > jhi) {
-                    s_rec[idx].jlo = 1;  // no pixel of the tile: no warp takes it
-                    s_rec[idx].jhi = 0;
-                    continue;
-                }
-                int type;
-                float3 e;
-                if (sc.emit) {
-                    const float4 em = __ldg(&sc.emit[code]);  // the code is the particle index
-                    type = __float_as_int(em.w);
-                    e = make_float3(em.x, em.y, em.z);
-                } else {
-                    type = (int)(code >> 24);
-                    const float It = fminf((float)(code & kCodeMax) * (1.0f / (float)kCodeMax), 1.0f);
-                    const bool per_view = fr.vlut != nullptr;  // the view's colormap in a plan
-                    const int vi = v * sc.n_types + type;
-                    const float4 *lut = per_view ? fr.vlut : sc.lut;
-                    const int len = per_view ? __ldg(&fr.vlut_len[vi]) : __ldg(&sc.lut_len[type]);
-                    const int off = per_view ? __ldg(&fr.vlut_off[vi]) : __ldg(&sc.lut_off[type]);
-                    const float f = It * (float)(len - 1);
-                    const int kk = min((int)f, len - 2);
-                    const float tau = f - (float)kk;
-                    const float4 c0 = __ldg(&lut[off + kk]);
-                    const float4 c1 = __ldg(&lut[off + kk + 1]);
-                    e = make_float3((1.0f - tau) * c0.x + tau * c1.x, (1.0f - tau) * c0.y + tau * c1.y,
-                                    (1.0f - tau) * c0.z + tau * c1.z);
-                }
-                Rec q;
-                q.ilo = ilo - px0;
-                q.ihi = ihi - px0;
-                q.jlo = jlo - py0;
-                q.jhi = jhi - py0;
-                q.X = X;
-                q.Y = Y;
-                q.R2 = __fmul_rn(R, R);
-                q.kr = __fdividef(kexp, q.R2);
-                const float vs = fr.vscale ? __ldg(&fr.vscale[v * sc.n_types + type]) : 1.0f;
-                q.er = e.x * vs;
-                q.eg = e.y * vs;
-                q.eb = e.z * vs;
-                q.pad = 0.0f;
-                s_rec[idx] = q;
-            }
-            __syncthreads();
-            // this warp's list: the records whose box meets one of its block rows, in
-            // record order (so every pixel sums its records in list order)
-            int nmine = 0;
-            short *mine = s_wl + warp * kStage;
-            for (int j0 = 0; j0 < cnt; j0 += 32) {
-                const int idx = j0 + lane;
-                bool meets = false;
-                if (idx < cnt) {
-                    const int jl = s_rec[idx].jlo, jh = s_rec[idx].jhi;
-                    if (jl <= jh) {
-                        const int br0 = jl >> 2, nbr = (jh >> 2) - br0 + 1;
-                        meets = nbr >= kSplatWarps || ((warp - br0) & (kSplatWarps - 1)) < nbr;
-                    }
-                }
-                const uint32_t bal = __ballot_sync(0xffffffffu, meets);
-                if (meets) mine[nmine + __popc(bal & ((1u << lane) - 1u))] = (short)idx;
-                nmine += __popc(bal);
-            }
-            __syncwarp();
-
-            // ---- 2. gather: this warp's list over this warp's blocks ---------------------
-            for (int k = 0; k < nmine; ++k) {
-                const Rec *q = &s_rec[mine[k]];
-                const int4 box = *reinterpret_cast<const int4 *>(&q->ilo);
-                const float4 pa = *reinterpret_cast<const float4 *>(&q->X);
-                const float4 pb = *reinterpret_cast<const float4 *>(&q->er);
-                // block columns the box overlaps, as a bit mask (uniform over the warp)
-                const uint32_t cm = (2u << (box.y >> 3)) - (1u << (box.x >> 3));
-#pragma unroll
-                for (int rr = 0; rr < NR; ++rr) {
-                    const int r0 = 4 * (warp + kSplatWarps * rr);
-                    if (NR > 1 && (r0 > box.w || r0 + 3 < box.z)) continue;
-                    const float dy = __fsub_rn(fy[rr], pa.y);
-                    const float dy2 = __fmul_rn(dy, dy);
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        if (!(cm & (1u << c))) continue;
-                        const float dx = __fsub_rn(fx[c], pa.x);
-                        const float d2 = __fadd_rn(__fmul_rn(dx, dx), dy2);
-                        if (d2 < pa.z) {
-                            const float w = ex2_fast(d2 * pa.w);
-                            ar[rr][c] += pb.x * w;
-                            ag[rr][c] += pb.y * w;
-                            ab[rr][c] += pb.z * w;
-                        }
-                    }
-                }
-            }
-            __syncthreads();
-        }
-
-        // epilogue: final transform of this lane's pixels, or merge of a split tile
-        float *o = out + (int64_t)v * H * W * 3;
-        if (slot < 0) {
-#pragma unroll
-            for (int rr = 0; rr < NR; ++rr) {
-                const int row = 4 * (warp + kSplatWarps * rr) + lr;
-                if (row >= th) continue;
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    if (c * 8 + lc >= tw) continue;
-                    float *p = o + ((int64_t)(py0 + row) * W + px0 + c * 8 + lc) * 3;
-                    put_pixel(p, ar[rr][c], out_accum);
-                    put_pixel(p + 1, ag[rr][c], out_accum);
-                    put_pixel(p + 2, ab[rr][c], out_accum);
-                }
-            }
-        } else {
-            unsigned long long *scr = fr.scratch + (int64_t)slot * 6 * T * T;
-#pragma unroll
-            for (int rr = 0; rr < NR; ++rr) {
-                const int row = 4 * (warp + kSplatWarps * rr) + lr;
-                if (row >= th) continue;
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    if (c * 8 + lc >= tw) continue;
-                    const int pix = row * T + c * 8 + lc;
-                    fix_add(&scr[2 * pix], ar[rr][c]);
-                    fix_add(&scr[2 * (T * T + pix)], ag[rr][c]);
-                    fix_add(&scr[2 * (2 * T * T + pix)], ab[rr][c]);
-                }
-            }
-            __threadfence();
-            __syncthreads();
-            if (tid == 0) s_last = (atomicAdd(&fr.tickets[slot], 1) == n_it - 1);
-            __syncthreads();
-            if (s_last) {
-                __threadfence();
-                const int rowlen = 3 * tw;
-                for (int k = tid; k < th * rowlen; k += kSplatThreads) {
-                    const int r = k / rowlen, cc = k - r * rowlen;
-                    const int col = cc / 3, ch = cc - col * 3;
-                    const float a = fix_value(&scr[2 * (ch * T * T + r * T + col)]);
-                    put_pixel(&o[((int64_t)(py0 + r) * W + px0) * 3 + cc], a, out_accum);
-                }
-                __syncthreads();
-                for (int k = tid; k < 6 * T * T; k += kSplatThreads) scr[k] = 0ull;
-                if (tid == 0) fr.tickets[slot] = 0;
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// ---------------------------------------------------------------------------------------
-// Warp-per-item splat for tiles up to 32 px.  One warp owns every pixel of a square of at
-// most 16 x 16 pixels (NR x NC blocks of 8 x 4 pixels, all in registers): a tile of up
-// to 16 px, or one of the four quadrants of a larger tile, which are four separate work
-// items over the same record list (binning with the larger tile keeps the scatter's
-// open list slices within L2).  The warps of a CTA never wait on one another: in
-// clustered data the density inside a tile is far from uniform, and with a tile's pixel
-// rows shared out among several warps the busiest one set the pace.
-// Per stage of 128 records (bulk copy into the warp's own double buffer, mbarrier
-// completion with a bounded wait):
-//   1. each lane takes 4 records: pixel box inside the square, and the rectangle of
-//      blocks it covers; live records are counted per rectangle;
-//   2. the live records are grouped by rectangle (warp-local counting sort), and their
-//      colour (colormap, or the particle's emission in vector-colour scenes) and Gaussian
-//      scale are computed, one record per lane;
-//   3. for every rectangle present, one jump to straight-line code for that rectangle,
-//      which runs over its records: each lane evaluates its pixel of every covered block
-//      with the FP32 coverage rule and adds e * w to its registers.
-// No atomics on pixels: a pixel has one owner.  Slices of a split tile add their partial
-// sums into a scratch tile and the last one to finish writes the tile.
-
-constexpr int kWarpsPerCta = 4;
-constexpr int kWStage = 128;  // records per bulk copy, per warp
-
-struct __align__(16) WRec {
-    float X, Y, R2, kr;
-    float er, eg, eb, pad;
-};
+constexpr int kRegion = 16;     // edge of the region a warp owns, in pixels
+constexpr int kWarpsPerCta = 2;
+constexpr int kBatch = 192;     // records per batch (list entries are 8-bit batch positions)
+constexpr int kAhead = 3;       // 32-record loads in flight
+constexpr int kRounds = kBatch / 32;            // records per lane of a full batch
+constexpr int kWords = (kBatch / 32 + 1) / 2;   // 32-record words per lane (two lanes share a square's words)
+static_assert(kBatch < 256 && kBatch % 32 == 0, "8-bit list entries; entry kBatch covers nothing");
 
 struct __align__(16) WarpSmem {
-    float4 buf[2][kWStage];      // staged records
-    WRec dec[kWStage];           // decoded live records, grouped by rectangle
-    int cnt[32];                 // live records per block rectangle
-    unsigned char ord[kWStage];  // live records grouped by rectangle
-    uint64_t bar[2];
+    float4 pa[kBatch + 1];           // raw record, then (-X, -Y, R^2, Gaussian scale); the last
+    float4 pb[kBatch + 1];           // entry covers nothing.  pb: emission r, g, b
+    float acc[3][kRegion][kRegion];  // the region's accumulator
+    // per square: batch positions of the records that meet it (a word of padding per square
+    // keeps equal places of the 16 lists in different banks)
+    unsigned char list[16][kBatch + 4];
+    float4 ring[kAhead][32];  // records on their way from the list
 };
 
-template <int NR, int NC>
-struct WarpShape {
-    static constexpr int kRects = (NR * (NR + 1) / 2) * (NC * (NC + 1) / 2);
-    static_assert(kRects <= 32, "one lane per block rectangle");
-    // resident CTAs per SM, which caps the registers: below about 80 per thread the
-    // compiler reloads record fields from shared memory instead of keeping them
-    static constexpr int kMinCtas = NR * NC <= 2 ? 8 : 6;
-};
+// 16 bytes from global to shared memory, asynchronously (LDGSTS)
+__device__ __forceinline__ void copy16_async(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void copy_wait() {  // all but the newest N groups done
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void copy_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Index of the block range [a, b] among the n (n + 1) / 2 ranges of n blocks.
-__host__ __device__ constexpr int range_id(int a, int b, int n) { return a * n - a * (a - 1) / 2 + (b - a); }
-
-// Straight-line splat of one record over the block rectangle rows [R0, R1] x columns
-// [C0, C1]: every lane evaluates its pixel of each block, uncovered pixels add zero.
-template <int NR, int NC, int R0, int R1, int C0, int C1>
-__device__ __forceinline__ void rect_splat(const float (&fx)[NC], const float (&fy)[NR], float (&ar)[NR][NC],
-                                           float (&ag)[NR][NC], float (&ab)[NR][NC], const float4 &pa,
-                                           const float4 &pb) {
-    // dx^2 once per block column, dy^2 once per block row (same rounding as per pixel)
-    float dx2[NC];
-#pragma unroll
-    for (int c = C0; c <= C1; ++c) {
-        const float dx = __fsub_rn(fx[c], pa.x);
-        dx2[c] = __fmul_rn(dx, dx);
-    }
-#pragma unroll
-    for (int r = R0; r <= R1; ++r) {
-        const float dy = __fsub_rn(fy[r], pa.y);
-        const float dy2 = __fmul_rn(dy, dy);
-#pragma unroll
-        for (int c = C0; c <= C1; ++c) {
-            const float d2 = __fadd_rn(dx2[c], dy2);
-            const float w = ex2_fast(d2 * pa.w);
-            // a += e * w only where d2 < R^2 (predicated: uncovered pixels add nothing)
-            asm("{\n\t.reg .pred p;\n\t"
-                "setp.lt.f32 p, %3, %4;\n\t"
-                "@p fma.rn.f32 %0, %5, %8, %0;\n\t"
-                "@p fma.rn.f32 %1, %6, %8, %1;\n\t"
-                "@p fma.rn.f32 %2, %7, %8, %2;\n\t}"
-                : "+f"(ar[r][c]), "+f"(ag[r][c]), "+f"(ab[r][c])
-                : "f"(d2), "f"(pa.z), "f"(pb.x), "f"(pb.y), "f"(pb.z), "f"(w));
-        }
-    }
+__device__ __forceinline__ uint32_t leading_zeros(uint32_t v) {  // v != 0
+    uint32_t z;
+    asm("bfind.shiftamt.u32 %0, %1;" : "=r"(z) : "r"(v));
+    return z;
 }
 
-// All records of one block rectangle, taken from the grouped order: the jump to the
-// rectangle's code is made once for the group.
-template <int NR, int NC, int R0, int R1, int C0, int C1>
-__device__ __forceinline__ void rect_run(const WarpSmem *ws, int j0, int n, const float (&fx)[NC],
-                                         const float (&fy)[NR], float (&ar)[NR][NC], float (&ag)[NR][NC],
-                                         float (&ab)[NR][NC]) {
-    // not unrolled: 30 copies of an unrolled loop overflow the instruction cache
-#pragma unroll 1
-    for (int j = j0; j < j0 + n; ++j) {
-        const float4 pa = *reinterpret_cast<const float4 *>(&ws->dec[j].X);
-        const float4 pb = *reinterpret_cast<const float4 *>(&ws->dec[j].er);
-        rect_splat<NR, NC, R0, R1, C0, C1>(fx, fy, ar, ag, ab, pa, pb);
-    }
-}
-
-#define SPL_RUN(R0, R1, C0, C1)                                                               \
-    case range_id(R0, R1, NR) * (NC * (NC + 1) / 2) + range_id(C0, C1, NC):                  \
-        rect_run<NR, NC, R0, R1, C0, C1>(ws, j0, n, fx, fy, ar, ag, ab);                      \
-        break;
-#define SPL_RUNS4(C0, C1)                                                                      \
-    SPL_RUN(0, 0, C0, C1) SPL_RUN(0, 1, C0, C1) SPL_RUN(0, 2, C0, C1) SPL_RUN(0, 3, C0, C1)     \
-    SPL_RUN(1, 1, C0, C1) SPL_RUN(1, 2, C0, C1) SPL_RUN(1, 3, C0, C1) SPL_RUN(2, 2, C0, C1)     \
-    SPL_RUN(2, 3, C0, C1) SPL_RUN(3, 3, C0, C1)
-
-template <int NR, int NC>
-__device__ __forceinline__ void run_dispatch(int id, const WarpSmem *ws, int j0, int n, const float (&fx)[NC],
-                                             const float (&fy)[NR], float (&ar)[NR][NC], float (&ag)[NR][NC],
-                                             float (&ab)[NR][NC]) {
-    if constexpr (NR == 2 && NC == 1) {
-        switch (id) {
-            SPL_RUN(0, 0, 0, 0)
-            SPL_RUN(0, 1, 0, 0)
-            SPL_RUN(1, 1, 0, 0)
-            default: break;
-        }
-    } else {
-        static_assert(NR == 4 && NC == 2, "shapes: 8 x 8 and 16 x 16 pixels");
-        switch (id) {
-            SPL_RUNS4(0, 0)
-            SPL_RUNS4(0, 1)
-            SPL_RUNS4(1, 1)
-            default: break;
-        }
-    }
-}
-#undef SPL_RUNS4
-#undef SPL_RUN
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 
 // kViewScale: multiply every record's emission by a per-view, per-species scale (plans
 // with a brightness sequence); a separate instance, so plain renders carry no extra code.
-template <int NR, int NC, bool kViewScale, bool kEmit>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, (WarpShape<NR, NC>::kMinCtas))
-    k_splat_warp(SceneDev sc, FrameDev fr, int *queue, float *out, int out_accum, int split) {
-    if (fr.status[kStatOverflow] || fr.status[kStatTimeout]) return;  // no complete tile lists
+template <bool kViewScale, bool kEmit>
+__global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
+    k_splat(SceneDev sc, FrameDev fr, int *queue, float *out, int out_accum, int split) {
+    if (fr.status[kStatOverflow]) return;  // no complete tile lists
     extern __shared__ __align__(16) unsigned char s_raw[];
     WarpSmem *ws = reinterpret_cast<WarpSmem *>(s_raw) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
+    const uint32_t lt_mask = (1u << lane) - 1u;
     const int nt = fr.n_tiles;
     const int N = fr.V * nt;
     const int S2 = split * split;
@@ -464,30 +112,34 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, (WarpShape<NR, NC>::kMinCta
     const int64_t K = fr.sizes[kSizeK];
     const ViewParams g0 = fr.views[0];
     const int T = g0.T, W = g0.W, H = g0.H, ntx = g0.ntx;
-    const int sub = (T + split - 1) / split;  // edge of the square a warp owns
-    const int lc = lane & 7, lr = lane >> 3;
-
+    const int sub = (T + split - 1) / split;  // edge of the region a warp owns
+    const int pair = lane >> 1;               // lane pair: the unit that evaluates a square
+    const bool vec_rows = (W & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;  // 16-byte rows of 4 pixels
     if (lane == 0) {
-        mbar_init(&ws->bar[0], 1);
-        mbar_init(&ws->bar[1], 1);
-        mbar_fence_init();
+        ws->pa[kBatch] = make_float4(0.0f, 0.0f, -1.0f, -1.0f);
+        ws->pb[kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
-    __syncwarp();
-    uint32_t phase0 = 0, phase1 = 0;
 
+    // the next item is taken from the queue while the current one is rendered
+    int next = 0;
+    if (lane == 0) next = atomicAdd(queue, 1);
     for (;;) {
-        int item = 0;
-        if (lane == 0) item = atomicAdd(queue, 1);
-        item = __shfl_sync(0xffffffffu, item, 0);
+        const int item = __shfl_sync(0xffffffffu, next, 0);
         if (item >= total_items) break;
+        if (lane == 0) next = atomicAdd(queue, 1);
 
-        // item = (slice of a tile list, square of the tile); the squares of a slice are
+        // item = (slice of a tile list, region of the tile); the regions of a slice are
         // consecutive items, so they run at once and share the slice's records in L2
         const int qs = item / S2, q = item - qs * S2;
-        const int slice = fr.order ? __ldg(&fr.order[qs]) : qs;
-        const int gt = find_tile(fr.item_off, N, slice);
+        int gt, chunk;  // the slice's tile and its place in the tile's list
+        if (fr.order) {
+            const int2 o = __ldg(&fr.order[qs]);
+            gt = o.x, chunk = o.y;
+        } else {
+            gt = find_tile(fr.item_off, N, qs);
+            chunk = qs - fr.item_off[gt];
+        }
         const int v = gt / nt, t = gt - v * nt;
-        const int chunk = slice - fr.item_off[gt];
         const int arrivals = (fr.item_off[gt + 1] - fr.item_off[gt]) * S2;
         const int slot = fr.split_slot[gt];
         const float kexp = fr.views[v].kexp;
@@ -499,184 +151,345 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, (WarpShape<NR, NC>::kMinCta
         const int64_t seg1 = fr.offsets[gt + 1];
         const int64_t e0 = fr.offsets[gt] + (int64_t)chunk * K;
         const int nrec = (tw > 0 && th > 0) ? (int)(min(seg1, e0 + K) - e0) : 0;
-        const int nst = (nrec + kWStage - 1) / kWStage;
+        const float4 *recs = fr.lists + e0;
 
-        // this lane's pixels: (c * 8 + lc, r * 4 + lr) of the square; pixels outside it
-        // get a centre no support reaches
-        float fx[NC], fy[NR], ar[NR][NC], ag[NR][NC], ab[NR][NC];
+        float *acc = &ws->acc[0][0][0];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) fx[c] = c * 8 + lc < tw ? (float)(px0 + c * 8 + lc) + 0.5f : kFar;
+        for (int k = 0; k < 3 * kRegion * kRegion / 128; ++k)
+            reinterpret_cast<float4 *>(acc)[k * 32 + lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+
+        // A support that covers a pixel centre of the region lies within R of its centres' box:
+        // max(|X - xc|, |Y - yc|) < R + half; the widening exceeds the FP32 rounding at any
+        // position, so no covered pixel is left out
+        const float hx = 0.5f * (float)(tw - 1), hy = 0.5f * (float)(th - 1);
+        const float xc = (float)px0 + 0.5f + hx, yc = (float)py0 + 0.5f + hy;
+        const float half = fmaxf(hx, hy) + 1e-3f + 4e-6f * (xc + yc);
+        const float widen = 2.5e-4f + 1e-6f * (xc + yc);  // the same in squares
+        const uint32_t ex = (tw + 3) >> 2, ey = (th + 3) >> 2;  // square columns and rows
+        const float cx = -0.25f * ((float)px0 + 0.5f), cy = -0.25f * ((float)py0 + 0.5f);
+
+        // kAhead loads of 32 records ahead, through shared memory; a lane reads what it copied
+        // itself, so waiting for its own copies is enough
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            fy[r] = r * 4 + lr < th ? (float)(py0 + r * 4 + lr) + 0.5f : kFar;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) ar[r][c] = ag[r][c] = ab[r][c] = 0.0f;
+        for (int g = 0; g < kAhead; ++g) {
+            if (g * 32 + lane < nrec) copy16_async(&ws->ring[g][lane], recs + g * 32 + lane);
+            copy_commit();
         }
-
-        if (lane == 0 && nrec > 0) {
-            const int c0 = min(kWStage, nrec);
-            fence_proxy_async_smem();
-            mbar_arrive_expect_tx(&ws->bar[0], (uint32_t)c0 * 16u);
-            bulk_g2s(ws->buf[0], fr.lists + e0, (uint32_t)c0 * 16u, &ws->bar[0]);
-        }
-        for (int si = 0; si < nst; ++si) {
-            const int cb = si & 1;
-            if (lane == 0 && si + 1 < nst) {
-                const int nb = (si + 1) & 1;
-                const int cn = min(kWStage, nrec - (si + 1) * kWStage);
-                fence_proxy_async_smem();
-                mbar_arrive_expect_tx(&ws->bar[nb], (uint32_t)cn * 16u);
-                bulk_g2s(ws->buf[nb], fr.lists + e0 + (int64_t)(si + 1) * kWStage, (uint32_t)cn * 16u,
-                         &ws->bar[nb]);
-            }
-            const bool ok = mbar_wait_bounded(&ws->bar[cb], cb ? phase1 : phase0, kWaitCycles);
-            if (cb) phase1 ^= 1u; else phase0 ^= 1u;
-            if (!__all_sync(0xffffffffu, ok)) {
-                if (lane == 0) atomicExch(&fr.status[kStatTimeout], 1);
-                return;
-            }
-            const int cnt = min(kWStage, nrec - si * kWStage);
-            const float4 *recs = ws->buf[cb];
-
-            // ---- 1. pixel box and block rectangle of every record; count per rectangle
-            ws->cnt[lane] = 0;
+        int at = 0;  // ring row of the next 32 records
+        int base = 0;
+        while (base < nrec) {
+            // ---- 1. fill the batch with records that meet the region
+            int nbuf = 0;
             __syncwarp();
-            int rid[kWStage / 32], rrank[kWStage / 32];
+            while (base < nrec && nbuf <= kBatch - 32) {
+                copy_wait<kAhead - 1>();
+                const float4 rec = ws->ring[at][lane];
+                const bool live = base + lane < nrec && fmaxf(fabsf(rec.x - xc), fabsf(rec.y - yc)) <
+                                                            fmaf(rec.z, 1.000004f, half);
+                const uint32_t bal = __ballot_sync(0xffffffffu, live);
+                if (live) {
+                    const int j = nbuf + __popc(bal & lt_mask);
+                    ws->pa[j] = rec;
+                    if constexpr (kEmit)  // the record's last word is the particle index
+                        copy16_async(&ws->pb[j], &sc.emit[__float_as_uint(rec.w)]);
+                }
+                nbuf += __popc(bal);
+                // the ballot has consumed these records: their row takes the next copy
+                const int nx = base + 32 * kAhead + lane;
+                if (nx < nrec) copy16_async(&ws->ring[at][lane], recs + nx);
+                copy_commit();
+                at = at + 1 == kAhead ? 0 : at + 1;
+                base += 32;
+            }
+            if (nbuf == 0) continue;
+            __syncwarp();
+
+            // ---- 2. the squares a record's box meets, its colour and Gaussian scale, one record
+            // per lane.  The loads of all the batch's records go out together, stage by stage;
+            // lanes past the end repeat the last record.
+            uint32_t word[kWords];
+            int cnt = 0;
 #pragma unroll
-            for (int q4 = 0; q4 < kWStage / 32; ++q4) {
-                const int idx = q4 * 32 + lane;
-                rid[q4] = -1;
-                rrank[q4] = 0;
-                if (idx < cnt) {
-                    const float4 rec = recs[idx];
-                    const float X = rec.x, Y = rec.y, R = rec.z;
-                    // tight pixel range of the support inside the square; eps exceeds the
-                    // FP32 rounding of X +- R at any position, so no covered pixel is lost
-                    const float eps = 1e-3f + 2e-6f * (fabsf(X) + fabsf(Y) + R);
-                    const int ilo = max(0, (int)ceilf(clampf(X - R - 0.5f - eps, px0 - 1.0f, (float)(px0 + tw))) - px0);
-                    const int ihi = min(tw - 1, (int)floorf(clampf(X + R - 0.5f + eps, px0 - 1.0f, (float)(px0 + tw))) - px0);
-                    const int jlo = max(0, (int)ceilf(clampf(Y - R - 0.5f - eps, py0 - 1.0f, (float)(py0 + th))) - py0);
-                    const int jhi = min(th - 1, (int)floorf(clampf(Y + R - 0.5f + eps, py0 - 1.0f, (float)(py0 + th))) - py0);
-                    if (ilo <= ihi && jlo <= jhi)
-                        rid[q4] = range_id(jlo >> 2, jhi >> 2, NR) * (NC * (NC + 1) / 2) +
-                                  range_id(ilo >> 3, ihi >> 3, NC);
+            for (int g = 0; g < kWords; ++g) word[g] = 0;
+            {
+                float4 rec[kRounds];
+#pragma unroll
+                for (int g = 0; g < kRounds; ++g) rec[g] = ws->pa[min(g * 32 + lane, nbuf - 1)];
+                // Pixel p of the region (centre p0 + p + 0.5) lies in square p / 4, so the support
+                // [X - R, X + R] meets squares ceil((X - p0 - 0.5) / 4 - 3 / 4 - R / 4) up to
+                // floor((X - p0 - 0.5) / 4 + R / 4).  (A record that meets no column or row of the
+                // region gets an empty or a meaningless mask; its pixels are tested one by one, so
+                // it adds nothing either way.)  Ballots over the four columns and rows give each
+                // square its word of 32 records; lane s keeps the even words of square s, lane
+                // 16 + s the odd ones.
+#pragma unroll
+                for (int g = 0; g < kRounds; ++g) {
+                    const float rq = fmaf(rec[g].z, 0.250001f, widen);
+                    const float qx = fmaf(rec[g].x, 0.25f, cx), qy = fmaf(rec[g].y, 0.25f, cy);
+                    // first square and one past the last (conversions below 0 give 0)
+                    const uint32_t x0 = __float2uint_ru(qx - (rq + 0.75f)), y0 = __float2uint_ru(qy - (rq + 0.75f));
+                    const uint32_t x1 = min(ex, __float2uint_rd(qx + (rq + 1.0f)));
+                    const uint32_t y1 = min(ey, __float2uint_rd(qy + (rq + 1.0f)));
+                    const uint32_t m =
+                        g * 32 + lane < nbuf ? ((1u << x1) - (1u << x0)) + (((1u << y1) - (1u << y0)) << 4) : 0u;
+                    uint32_t b[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) b[k] = __ballot_sync(0xffffffffu, m & (1u << k));
+                    const uint32_t c = (lane & 2) ? ((lane & 1) ? b[3] : b[2]) : ((lane & 1) ? b[1] : b[0]);
+                    const uint32_t r = (lane & 8) ? ((lane & 4) ? b[7] : b[6]) : ((lane & 4) ? b[5] : b[4]);
+                    if ((lane >> 4) == (g & 1)) {
+                        word[g >> 1] = c & r;
+                        cnt += __popc(c & r);
+                    }
                 }
-                // rank among the stage's records of the same rectangle, in record order
-                // (lanes with equal rectangle ids, found bit by bit with ballots)
-                const uint32_t peers = warp_peers<6>((uint32_t)(rid[q4] + 1));
-                const int leader = __ffs(peers) - 1;
-                int before = 0;
-                if (rid[q4] >= 0 && lane == leader) {
-                    before = ws->cnt[rid[q4]];
-                    ws->cnt[rid[q4]] = before + __popc(peers);
+                float3 e[kRounds];
+                float vs[kRounds];
+                if constexpr (kEmit) {
+                    copy_wait_all();
+                    __syncwarp();
+                    if constexpr (kViewScale)
+#pragma unroll
+                        for (int g = 0; g < kRounds; ++g) {
+                            const float4 em = ws->pb[min(g * 32 + lane, nbuf - 1)];
+                            e[g] = make_float3(em.x, em.y, em.z);
+                            vs[g] = __ldg(&fr.vscale[v * sc.n_types + __float_as_int(em.w)]);
+                        }
+                } else {
+                    // the view's colormap in a plan with per-view sequences, else the scene's
+                    const float4 *lut = kViewScale ? fr.vlut : sc.lut;
+                    const int *lut_len = kViewScale ? fr.vlut_len + v * sc.n_types : sc.lut_len;
+                    const int *lut_off = kViewScale ? fr.vlut_off + v * sc.n_types : sc.lut_off;
+                    int len[kRounds], off[kRounds];
+#pragma unroll
+                    for (int g = 0; g < kRounds; ++g) {
+                        const int type = (int)(__float_as_uint(rec[g].w) >> 24);
+                        len[g] = __ldg(&lut_len[type]);
+                        off[g] = __ldg(&lut_off[type]);
+                        vs[g] = kViewScale ? __ldg(&fr.vscale[v * sc.n_types + type]) : 1.0f;
+                    }
+                    float4 c0[kRounds], c1[kRounds];
+                    float tau[kRounds];
+#pragma unroll
+                    for (int g = 0; g < kRounds; ++g) {
+                        const uint32_t code = __float_as_uint(rec[g].w);
+                        const float It = fminf((float)(code & kCodeMax) * (1.0f / (float)kCodeMax), 1.0f);
+                        const float f = It * (float)(len[g] - 1);
+                        const int kk = min((int)f, len[g] - 2);
+                        tau[g] = f - (float)kk;
+                        c0[g] = __ldg(&lut[off[g] + kk]);
+                        c1[g] = __ldg(&lut[off[g] + kk + 1]);
+                    }
+#pragma unroll
+                    for (int g = 0; g < kRounds; ++g)
+                        e[g] = make_float3((1.0f - tau[g]) * c0[g].x + tau[g] * c1[g].x,
+                                           (1.0f - tau[g]) * c0[g].y + tau[g] * c1[g].y,
+                                           (1.0f - tau[g]) * c0[g].z + tau[g] * c1[g].z);
                 }
-                before = __shfl_sync(0xffffffffu, before, leader);
-                rrank[q4] = before + __popc(peers & ((1u << lane) - 1u));
+                __syncwarp();
+#pragma unroll
+                for (int g = 0; g < kRounds; ++g) {
+                    const int j = g * 32 + lane;
+                    if (j >= nbuf) break;
+                    const float R2 = __fmul_rn(rec[g].z, rec[g].z);
+                    // the scale is kept finite and nonzero, so that distance^2 x scale is never
+                    // NaN (R^2 may underflow to 0 or overflow; the comparison with R^2 decides)
+                    const float kr = fminf(fmaxf(__fdividef(kexp, R2), -1e30f), -1.2e-38f);
+                    ws->pa[j] = make_float4(-rec[g].x, -rec[g].y, R2, kr);
+                    if constexpr (kViewScale || !kEmit)
+                        ws->pb[j] = make_float4(e[g].x * vs[g], e[g].y * vs[g], e[g].z * vs[g], 0.0f);
+                }
+            }
+
+            // ---- 3. per square, the batch positions of its records
+            const int other = __shfl_xor_sync(0xffffffffu, cnt, 16);
+            {
+                int dst = lane < 16 ? 0 : other;
+                // a lane with more than twice the mean is unpacked by the whole warp, a word at
+                // a time, so that a dense square does not hold up the others
+                const int all = __reduce_add_sync(0xffffffffu, cnt);
+                const bool heavy = cnt > max(8, all >> 4);
+                for (uint32_t todo = __ballot_sync(0xffffffffu, heavy); todo; todo &= todo - 1) {
+                    const int src = __ffs(todo) - 1;
+                    int at = __shfl_sync(0xffffffffu, dst, src);
+#pragma unroll
+                    for (int g = 0; g < kWords; ++g) {
+                        const uint32_t w = __shfl_sync(0xffffffffu, word[g], src);
+                        if ((w >> lane) & 1u)
+                            ws->list[src & 15][at + __popc(w & lt_mask)] =
+                                (unsigned char)((2 * g + (src >> 4)) * 32 + lane);
+                        at += __popc(w);
+                    }
+                }
+                if (!heavy) {
+                    unsigned char *p = ws->list[lane & 15] + dst;
+#pragma unroll
+                    for (int g = 0; g < kWords; ++g) {
+                        const int first = (2 * g + (lane >> 4)) * 32 + 31;
+                        uint32_t w = word[g];
+                        while (w) {
+                            const uint32_t z = leading_zeros(w);
+                            *p++ = (unsigned char)(first - z);
+                            w ^= 0x80000000u >> z;
+                        }
+                    }
+                }
                 __syncwarp();
             }
-            __syncwarp();
-            // ---- 2. group the live records by rectangle (lane = rectangle)
-            const int c = ws->cnt[lane];
-            const int incl = warp_incl_scan_i(c);
-            const int base = incl - c;
-            const int nlive = __shfl_sync(0xffffffffu, incl, 31);
+            // squares by list length, longest first: key = length, square (both half-warps sort
+            // the same 16 keys)
+            uint32_t key = ((uint32_t)(cnt + other) << 4) | (uint32_t)(lane & 15);
 #pragma unroll
-            for (int q4 = 0; q4 < kWStage / 32; ++q4) {
-                const int b = __shfl_sync(0xffffffffu, base, rid[q4] < 0 ? 0 : rid[q4]);
-                if (rid[q4] >= 0) ws->ord[b + rrank[q4]] = (unsigned char)(q4 * 32 + lane);
-            }
-            __syncwarp();
-            // colour and Gaussian scale of the live records only, one per lane
-            for (int j = lane; j < nlive; j += 32) {
-                const int k = ws->ord[j];
-                const float4 rec = recs[k];
-                const float R = rec.z;
-                const uint32_t code = __float_as_uint(rec.w);
-                int type;
-                float3 e;
-                if constexpr (kEmit) {
-                    const float4 em = __ldg(&sc.emit[code]);  // the code is the particle index
-                    type = __float_as_int(em.w);
-                    e = make_float3(em.x, em.y, em.z);
-                } else {
-                    type = (int)(code >> 24);
-                    const float It = fminf((float)(code & kCodeMax) * (1.0f / (float)kCodeMax), 1.0f);
-                    // the view's colormap in a plan with per-view sequences, else the scene's
-                    const float4 *lut = sc.lut;
-                    int len, off;
-                    if constexpr (kViewScale) {
-                        const int vi = v * sc.n_types + type;
-                        lut = fr.vlut;
-                        len = __ldg(&fr.vlut_len[vi]);
-                        off = __ldg(&fr.vlut_off[vi]);
-                    } else {
-                        len = __ldg(&sc.lut_len[type]);
-                        off = __ldg(&sc.lut_off[type]);
-                    }
-                    const float f = It * (float)(len - 1);
-                    const int kk = min((int)f, len - 2);
-                    const float tau = f - (float)kk;
-                    const float4 c0 = __ldg(&lut[off + kk]);
-                    const float4 c1 = __ldg(&lut[off + kk + 1]);
-                    e = make_float3((1.0f - tau) * c0.x + tau * c1.x, (1.0f - tau) * c0.y + tau * c1.y,
-                                    (1.0f - tau) * c0.z + tau * c1.z);
+            for (int size = 2; size <= 16; size <<= 1)
+#pragma unroll
+                for (int d = size >> 1; d; d >>= 1) {
+                    const uint32_t o = __shfl_xor_sync(0xffffffffu, key, d);
+                    const bool first = (lane & d) == 0, down = (lane & size & 15) == 0;
+                    key = (first == down) ? max(key, o) : min(key, o);
                 }
-                const float R2 = __fmul_rn(R, R);
-                float vs = 1.0f;
-                if constexpr (kViewScale) vs = __ldg(&fr.vscale[v * sc.n_types + type]);
-                float4 *d = reinterpret_cast<float4 *>(&ws->dec[j]);  // in grouped order
-                d[0] = make_float4(rec.x, rec.y, R2, __fdividef(kexp, R2));
-                d[1] = make_float4(e.x * vs, e.y * vs, e.z * vs, 0.0f);
+            // records before each place (exclusive), for the choice of the lane split
+            int before = (int)(key >> 4);
+#pragma unroll
+            for (int d = 1; d < 16; d <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, before, d, 16);
+                if ((lane & 15) >= d) before += u;
             }
+            const int total = __shfl_sync(0xffffffffu, before, 15);
+            before -= (int)(key >> 4);
             __syncwarp();
-            // ---- 3. one jump per rectangle present, then its records
-            uint32_t present = __ballot_sync(0xffffffffu, c > 0);
-            while (present) {
-                const int id = __ffs(present) - 1;
-                present &= present - 1;
-                const int j0 = __shfl_sync(0xffffffffu, base, id);
-                const int n = __shfl_sync(0xffffffffu, c, id);
-                run_dispatch<NR, NC>(id, ws, j0, n, fx, fy, ar, ag, ab);
-            }
-            __syncwarp();
-        }
 
-        // epilogue: final transform of this lane's pixels, or merge of a split tile
+            // ---- 4. passes over the squares
+            for (int i = 0; i < 16;) {
+                const int lead = (int)(__shfl_sync(0xffffffffu, key, i) >> 4);
+                if (lead == 0) break;
+                // lane split: 2^a pairs per square, 16 >> a squares; the a with the most
+                // records per instruction (about 64 per step of the loop, 36 per doubling for
+                // the shuffles, 60 per pass).  Lane a weighs option a.
+                int a;
+                {
+                    const int al = min(lane, 4);
+                    const int end = i + (16 >> al);
+                    const int upto = __shfl_sync(0xffffffffu, before, min(end, 15));
+                    const int from = __shfl_sync(0xffffffffu, before, i);
+                    const int covered = (end > 15 ? total : upto) - from;
+                    const int steps = (lead + (1 << al) - 1) >> al;
+                    const float gain = __fdividef((float)covered, (float)(64 * steps + 36 * al + 60));
+                    a = (int)(__reduce_max_sync(0xffffffffu, (__float_as_uint(gain) & ~7u) | (uint32_t)al) & 7u);
+                }
+                const int place = i + (pair >> a), r = pair & ((1 << a) - 1);
+                const uint32_t kp = __shfl_sync(0xffffffffu, key, place & 15);
+                const int sq = (int)(kp & 15u);
+                const int n = place < 16 ? (int)(kp >> 4) : 0;
+                const int mine = (n - r + (1 << a) - 1) >> a;  // list entries r, r + 2^a, ...
+                const int steps = (lead + (1 << a) - 1) >> a;
+                const unsigned char *lp = ws->list[sq] + r;
+                // this lane's pixels: rows y, y + 1 and columns x .. x + 3 of the region
+                const int x = 4 * (sq & 3), y = 4 * (sq >> 2) + 2 * (lane & 1);
+                const float fx = (float)(px0 + x) + 0.5f, fy0 = (float)(py0 + y) + 0.5f;
+                const float2 fx0 = make_float2(fx, fx + 1.0f), fx1 = make_float2(fx + 2.0f, fx + 3.0f);
+                const float2 fy = make_float2(fy0, fy0 + 1.0f);
+                float2 s[3][2][2];  // channel, row, column pair
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) s[c][k >> 1][k & 1] = f2(0.0f);
+                // the records of the next step load while this one is evaluated; a pair past
+                // the end of its list takes the record that covers nothing
+                int idx = mine > 0 ? *lp : kBatch;
+                float4 na = ws->pa[idx], nb = ws->pb[idx];
+                lp += 1 << a;
+                idx = mine > 1 ? *lp : kBatch;
+#pragma unroll 3
+                for (int k = 2; k < steps + 2; ++k) {
+                    const float4 pa = na, pb = nb;
+                    const float R2 = pa.z;
+                    na = ws->pa[idx];
+                    nb = ws->pb[idx];
+                    lp += 1 << a;
+                    idx = k < mine ? *lp : kBatch;
+                    const float2 dx0 = __fadd2_rn(fx0, f2(pa.x)), dx1 = __fadd2_rn(fx1, f2(pa.x));
+                    const float2 dy = __fadd2_rn(fy, f2(pa.y));
+                    const float2 qx0 = __fmul2_rn(dx0, dx0), qx1 = __fmul2_rn(dx1, dx1);
+                    const float2 qy = __fmul2_rn(dy, dy);
+#pragma unroll
+                    for (int row = 0; row < 2; ++row) {
+                        const float2 qr = f2(row ? qy.y : qy.x);
+#pragma unroll
+                        for (int cp = 0; cp < 2; ++cp) {
+                            const float2 d2 = __fadd2_rn(cp ? qx1 : qx0, qr);
+                            const float2 g = __fmul2_rn(d2, f2(pa.w));
+                            const float2 w = make_float2(d2.x < R2 ? ex2_fast(g.x) : 0.0f,
+                                                         d2.y < R2 ? ex2_fast(g.y) : 0.0f);
+                            s[0][row][cp] = __ffma2_rn(f2(pb.x), w, s[0][row][cp]);
+                            s[1][row][cp] = __ffma2_rn(f2(pb.y), w, s[1][row][cp]);
+                            s[2][row][cp] = __ffma2_rn(f2(pb.z), w, s[2][row][cp]);
+                        }
+                    }
+                }
+                for (int d = 2; d < (2 << a); d <<= 1) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            float2 &u = s[c][k >> 1][k & 1];
+                            u = __fadd2_rn(u, make_float2(__shfl_xor_sync(0xffffffffu, u.x, d),
+                                                          __shfl_xor_sync(0xffffffffu, u.y, d)));
+                        }
+                }
+                if (r == 0 && n > 0) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+#pragma unroll
+                        for (int row = 0; row < 2; ++row) {
+                            float4 *p = reinterpret_cast<float4 *>(&ws->acc[c][y + row][x]);
+                            float4 u = *p;
+                            u.x += s[c][row][0].x, u.y += s[c][row][0].y;
+                            u.z += s[c][row][1].x, u.w += s[c][row][1].y;
+                            *p = u;
+                        }
+                }
+                __syncwarp();
+                i += 16 >> a;
+            }
+        }
+        __syncwarp();
+
+        // epilogue: final transform of the region's pixels, or merge of a split tile
         float *o = out + (int64_t)v * H * W * 3;
         if (slot < 0) {
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                if (r * 4 + lr >= th) continue;
-#pragma unroll
-                for (int cc = 0; cc < NC; ++cc) {
-                    if (cc * 8 + lc >= tw) continue;
-                    float *p = o + ((int64_t)(py0 + r * 4 + lr) * W + px0 + cc * 8 + lc) * 3;
-                    put_pixel(p, ar[r][cc], out_accum);
-                    put_pixel(p + 1, ag[r][cc], out_accum);
-                    put_pixel(p + 2, ab[r][cc], out_accum);
+            float *reg = o + ((int64_t)py0 * W + px0) * 3;
+            if (tw == kRegion && vec_rows && (px0 & 3) == 0) {
+                // rows of 48 floats, four at a time
+                for (int k = lane; k < th * 12; k += 32) {
+                    const int r = k / 12, c = 4 * (k - 12 * r);
+                    float4 *p = reinterpret_cast<float4 *>(reg + (int64_t)r * W * 3 + c);
+                    float4 u = out_accum == 2 ? *p : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    put_pixel(&u.x, ws->acc[(c + 0) % 3][r][(c + 0) / 3], out_accum);
+                    put_pixel(&u.y, ws->acc[(c + 1) % 3][r][(c + 1) / 3], out_accum);
+                    put_pixel(&u.z, ws->acc[(c + 2) % 3][r][(c + 2) / 3], out_accum);
+                    put_pixel(&u.w, ws->acc[(c + 3) % 3][r][(c + 3) / 3], out_accum);
+                    *p = u;
+                }
+            } else {
+                for (int k = lane; k < 3 * kRegion * kRegion; k += 32) {
+                    const int r = k / (3 * kRegion), c = k % (3 * kRegion), col = c / 3;
+                    if (r < th && col < tw) put_pixel(&reg[(int64_t)r * W * 3 + c], ws->acc[c % 3][r][col], out_accum);
                 }
             }
         } else {
             unsigned long long *scr = fr.scratch + (int64_t)slot * 6 * T * T;
-            // the lane's sums go through the warp's (now idle) decode area so that one
-            // loop, not an unrolled copy per pixel, adds them: the splat's straight-line
-            // code already fills the instruction cache
-            float *park = reinterpret_cast<float *>(ws->dec) + lane;  // [NR * NC * 3][32]
-#pragma unroll
-            for (int r = 0; r < NR; ++r)
-#pragma unroll
-                for (int cc = 0; cc < NC; ++cc) {
-                    const int k = 3 * (r * NC + cc);
-                    park[32 * k] = ar[r][cc];
-                    park[32 * (k + 1)] = ag[r][cc];
-                    park[32 * (k + 2)] = ab[r][cc];
-                }
+            // 8 values per lane at a time, so that their atomics are in flight together
 #pragma unroll 1
-            for (int k = 0; k < 3 * NR * NC; ++k) {
-                const int ch = k % 3, blk = k / 3, r = blk / NC, cc = blk - r * NC;
-                if (r * 4 + lr >= th || cc * 8 + lc >= tw) continue;
-                const int pix = (qy + r * 4 + lr) * T + qx + cc * 8 + lc;
-                fix_add(&scr[2 * (ch * T * T + pix)], park[32 * k]);
+            for (int k0 = lane; k0 < 3 * kRegion * kRegion; k0 += 256) {
+                float val[8];
+                unsigned long long *dst[8];
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {
+                    const int k = k0 + 32 * g;
+                    const int ch = k / (kRegion * kRegion), r = (k / kRegion) % kRegion, col = k % kRegion;
+                    val[g] = r < th && col < tw ? acc[k] : 0.0f;
+                    dst[g] = &scr[2 * (ch * T * T + (qy + r) * T + qx + col)];
+                }
+                fix_add_n<8>(dst, val);
             }
             __threadfence();
             __syncwarp();
@@ -684,16 +497,25 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, (WarpShape<NR, NC>::kMinCta
             if (lane == 0) last = (atomicAdd(&fr.tickets[slot], 1) == arrivals - 1);
             last = __shfl_sync(0xffffffffu, last, 0);
             if (last) {
-                // the whole tile, from the scratch every square of every slice added into
+                // the whole tile, from the scratch every region of every slice added into
                 __threadfence();
                 const int TW = min(T, W - tx * T), TH = min(T, H - ty * T);
-                const int rowlen = 3 * TW;
+                const int rl = 3 * TW;
                 float *ot = o + ((int64_t)ty * T * W + (int64_t)tx * T) * 3;
-                for (int k = lane; k < TH * rowlen; k += 32) {
-                    const int rr = k / rowlen, c3 = k - rr * rowlen;
-                    const int col = c3 / 3, ch = c3 - col * 3;
-                    const float a = fix_value(&scr[2 * (ch * T * T + rr * T + col)]);
-                    put_pixel(&ot[(int64_t)rr * W * 3 + c3], a, out_accum);
+                for (int k0 = lane; k0 < TH * rl; k0 += 128) {
+                    float a[4];
+                    int64_t at[4];
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        const int k = min(k0 + 32 * g, TH * rl - 1);
+                        const int rr = k / rl, c3 = k - rr * rl;
+                        const int col = c3 / 3, ch = c3 - col * 3;
+                        a[g] = fix_value(&scr[2 * (ch * T * T + rr * T + col)]);
+                        at[g] = (int64_t)rr * W * 3 + c3;
+                    }
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+                        if (k0 + 32 * g < TH * rl) put_pixel(&ot[at[g]], a[g], out_accum);
                 }
                 __syncwarp();
                 for (int k = lane; k < 6 * T * T; k += 32) scr[k] = 0ull;
@@ -704,48 +526,26 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, (WarpShape<NR, NC>::kMinCta
     }
 }
 
-typedef void (*SplatFn)(SceneDev, FrameDev, int *, float *, int);
-typedef void (*WarpSplatFn)(SceneDev, FrameDev, int *, float *, int, int);
+typedef void (*SplatFn)(SceneDev, FrameDev, int *, float *, int, int);
 
-// Tiles up to 32 px: warp per square of up to 16 px (a tile above 16 px is split into
-// four squares); larger tiles: CTA per item.
-constexpr int kWarpTileMax = 32;
-static bool warp_kernel(int T) { return T <= kWarpTileMax; }
-int splat_split(int T) { return T > 16 && warp_kernel(T) ? 2 : 1; }
+int splat_split(int T) { return (T + kRegion - 1) / kRegion; }
 
-static WarpSplatFn warp_fn(int T, bool scaled = false, bool emit = false) {
-    if (emit) {
-        if (scaled) return T <= 8 ? k_splat_warp<2, 1, true, true> : k_splat_warp<4, 2, true, true>;
-        return T <= 8 ? k_splat_warp<2, 1, false, true> : k_splat_warp<4, 2, false, true>;
-    }
-    if (scaled) return T <= 8 ? k_splat_warp<2, 1, true, false> : k_splat_warp<4, 2, true, false>;
-    return T <= 8 ? k_splat_warp<2, 1, false, false> : k_splat_warp<4, 2, false, false>;
+static SplatFn splat_fn(bool scaled, bool emit) {
+    if (emit) return scaled ? k_splat<true, true> : k_splat<false, true>;
+    return scaled ? k_splat<true, false> : k_splat<false, false>;
 }
 
-static SplatFn cta_fn(int T) {
-    switch (block_cols(T)) {
-        case 5: return k_splat<2, 5>;
-        case 6: return k_splat<2, 6>;
-        case 7: return k_splat<2, 7>;
-        default: return k_splat<2, 8>;
-    }
-}
+static size_t splat_smem() { return sizeof(WarpSmem) * kWarpsPerCta; }
 
-static const void *splat_kernel(int T) { return warp_kernel(T) ? (const void *)warp_fn(T) : (const void *)cta_fn(T); }
-
-static size_t splat_smem(int T) { return warp_kernel(T) ? sizeof(WarpSmem) * kWarpsPerCta : splat_smem_bytes(T); }
-static int splat_cta_threads(int T) { return warp_kernel(T) ? kWarpsPerCta * 32 : kSplatThreads; }
-
-int splat_blocks_per_sm(int T) {
-    const size_t smem = splat_smem(T);
-    const void *fn = splat_kernel(T);
-    if (ensure_smem_limit(fn, smem) != cudaSuccess) return 0;
+int splat_blocks_per_sm() {
+    const void *fn = (const void *)splat_fn(false, false);
+    if (ensure_smem_limit(fn, splat_smem()) != cudaSuccess) return 0;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, splat_cta_threads(T), smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kWarpsPerCta * 32, splat_smem()) != cudaSuccess) return 0;
     return nb;
 }
 
-int splat_workers_per_sm(int T) { return splat_blocks_per_sm(T) * (warp_kernel(T) ? kWarpsPerCta : 1); }
+int splat_workers_per_sm() { return splat_blocks_per_sm() * kWarpsPerCta; }
 
 // k_item_order: one CTA.  The splat's work items (tile-list slices) ordered by record count,
 // largest first, so that the items taken last by the workers are the short ones and the
@@ -789,9 +589,9 @@ __global__ void __launch_bounds__(1024) k_item_order(FrameDev fr) {
         const long long c = fr.counts[t];
         if (n > 1) {
             const int p = atomicAdd(&s_cnt[bin_of(K)], n - 1);
-            for (int s = 0; s < n - 1; ++s) fr.order[p + s] = i0 + s;
+            for (int s = 0; s < n - 1; ++s) fr.order[p + s] = make_int2(t, s);
         }
-        fr.order[atomicAdd(&s_cnt[bin_of(c - K * (n - 1))], 1)] = i0 + n - 1;
+        fr.order[atomicAdd(&s_cnt[bin_of(c - K * (n - 1))], 1)] = make_int2(t, n - 1);
     }
 }
 
@@ -805,16 +605,10 @@ cudaError_t launch_splat(const SceneDev &sc, const FrameDev &fr, int *queue, flo
                          int grid, cudaStream_t st) {
     cudaError_t e = launch_item_order(fr, st);
     if (e != cudaSuccess) return e;
-    const size_t smem = splat_smem(fr.T);
-    const bool scaled = fr.vscale != nullptr, emit = sc.emit != nullptr;
-    cudaError_t err = ensure_smem_limit(
-        warp_kernel(fr.T) ? (const void *)warp_fn(fr.T, scaled, emit) : splat_kernel(fr.T), smem);
-    if (err != cudaSuccess) return err;
-    if (warp_kernel(fr.T))
-        warp_fn(fr.T, scaled, emit)<<<grid, splat_cta_threads(fr.T), smem, st>>>(sc, fr, queue, out, out_accum,
-                                                                                   splat_split(fr.T));
-    else
-        cta_fn(fr.T)<<<grid, splat_cta_threads(fr.T), smem, st>>>(sc, fr, queue, out, out_accum);
+    const SplatFn fn = splat_fn(fr.vscale != nullptr, sc.emit != nullptr);
+    e = ensure_smem_limit((const void *)fn, splat_smem());
+    if (e != cudaSuccess) return e;
+    fn<<<grid, kWarpsPerCta * 32, splat_smem(), st>>>(sc, fr, queue, out, out_accum, splat_split(fr.T));
     return cudaGetLastError();
 }
 

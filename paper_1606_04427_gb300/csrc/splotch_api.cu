@@ -727,7 +727,7 @@ static void layout_fixed(FrameHost &fh, const splotch_scene *sc, int V, int n_ti
 // Exact accumulators of one split tile: 3 channels x T x T pixels, 16 bytes each.
 static size_t split_scratch_bytes(int T) { return sizeof(unsigned long long) * 2 * 3 * (size_t)T * T; }
 
-// order: room for the splat's item order (one int per work item; the fixed-array render
+// order: room for the splat's item order (one int2 per work item; the fixed-array render
 // takes its items in tile order).
 static void layout_var(FrameHost &fh, int64_t pairs, int items, int splits, bool pids, bool order = true) {
     fh.pair_cap = pairs;
@@ -740,7 +740,7 @@ static void layout_var(FrameHost &fh, int64_t pairs, int items, int splits, bool
     fh.o_pids = pids ? cv.take(sizeof(int) * std::max<int64_t>(1, pairs)) : 0;
     fh.o_scratch = cv.take(split_scratch_bytes(fh.T) * std::max(1, splits));
     fh.o_tickets = cv.take(sizeof(int) * std::max(1, splits));
-    fh.o_order = order ? cv.take(sizeof(int) * (size_t)std::max(1, items)) : 0;
+    fh.o_order = order ? cv.take(sizeof(int2) * (size_t)std::max(1, items)) : 0;
     fh.var_bytes = cv.off;
 }
 
@@ -765,7 +765,7 @@ static FrameDev frame_dev(const FrameHost &fh, char *fixed, char *var) {
         fr.pids = fh.pids ? (int *)(var + fh.o_pids) : nullptr;
         fr.scratch = (unsigned long long *)(var + fh.o_scratch);
         fr.tickets = (int *)(var + fh.o_tickets);
-        fr.order = fh.order ? (int *)(var + fh.o_order) : nullptr;
+        fr.order = fh.order ? (int2 *)(var + fh.o_order) : nullptr;
     }
     fr.pair_cap = var ? fh.pair_cap : INT64_MAX;
     fr.item_cap = var ? fh.item_cap : INT32_MAX;
@@ -776,8 +776,8 @@ static FrameDev frame_dev(const FrameHost &fh, char *fixed, char *var) {
 // items: work items of the scan (tile-list slices); the splat renders each as split^2
 // squares, one worker each
 static int splat_grid(int dev, int T, int items) {
-    const int bps = std::max(1, splat_blocks_per_sm(T));
-    const int per_cta = std::max(1, splat_workers_per_sm(T) / bps);
+    const int bps = std::max(1, splat_blocks_per_sm());
+    const int per_cta = std::max(1, splat_workers_per_sm() / bps);
     const int g = sm_count(dev) * bps;
     const int64_t squares = (int64_t)std::max(1, items) * splat_split(T) * splat_split(T);
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, (squares + per_cta - 1) / per_cta));
@@ -785,7 +785,7 @@ static int splat_grid(int dev, int T, int items) {
 
 static int target_items(int dev, int T) {
     const int s = splat_split(T);
-    return std::max(1, sm_count(dev) * std::max(1, splat_workers_per_sm(T)) * 4 / (s * s));
+    return std::max(1, sm_count(dev) * std::max(1, splat_workers_per_sm()) * 4 / (s * s));
 }
 static const int kMinItemPairs = 2048;
 
@@ -1538,7 +1538,7 @@ extern "C" splotch_status splotch_render_noalloc(splotch_scene *sc, const splotc
     CUDA_TRY(launch_scan(fr, target_items(sc->dev, T), kMinItemPairs, st));
     CUDA_TRY(launch_scatter(sc->storage, sc->dev_view, fr, (pr.flags & SPLOTCH_STABLE) != 0, st));
     CUDA_TRY(launch_splat(sc->dev_view, fr, (int *)(base + fh.o_queue), out,
-                          out_mode(pr.flags), sm_count(dev) * std::max(1, splat_blocks_per_sm(T)), st));
+                          out_mode(pr.flags), sm_count(dev) * std::max(1, splat_blocks_per_sm()), st));
     int64_t sizes[8];
     int stat[4];
     CUDA_TRY(cudaMemcpyAsync(sizes, base + fh.o_sizes, sizeof(sizes), cudaMemcpyDeviceToHost, st));

@@ -17,12 +17,9 @@
 namespace spl {
 
 constexpr int kMaxTiles = 16384;   // tiles per image (per-CTA shared histogram)
-constexpr int kMaxTile = 64;       // tile edge in pixels (shared accumulator)
+constexpr int kMaxTile = 64;       // tile edge in pixels
 constexpr int kMaxTypes = 255;     // species (8-bit type field in the tile records)
 constexpr int kThreads = 1024;     // CTA size of the particle-stream kernels (one per SM: one tile histogram per SM)
-constexpr int kSplatThreads = 256; // CTA size of the splat kernel for tiles above 32 px
-constexpr int kSplatWarps = kSplatThreads / 32;
-constexpr int kStage = 512;        // tile records per bulk-copy stage (tiles above 32 px)
 constexpr int kMaxGroup = 16;      // views per CTA in the particle-stream kernels
 constexpr uint32_t kCodeMax = 16777215u;   // 24-bit normalised-intensity code
 constexpr float kLog2e = 1.4426950408889634f;
@@ -79,8 +76,8 @@ struct FrameDev {
     int *pids;                // [pair capacity] particle index per record, or null
     unsigned long long *scratch;  // [split capacity][3][T][T][2] exact accumulators (fix_add)
     int *tickets;                 // [split capacity]
-    int *order;                   // [item capacity] work items, largest first (k_item_order), or
-                                  // null: items in tile order
+    int2 *order;                  // [item capacity] work items (tile, slice of its list), largest
+                                  // first (k_item_order), or null: items in tile order
     int64_t pair_cap;
     int item_cap, split_cap;
     const float *vscale;      // [V * n_types] emission scale per view and species, or null
@@ -303,26 +300,36 @@ constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz
 // addition is associative, so the merged sum is the same whichever slice arrives first;
 // fix_value rounds it to FP32 once.
 
-__device__ __forceinline__ void fix_add(unsigned long long *acc, float v) {
+__device__ __forceinline__ bool fix_of(float v, unsigned long long &lo, unsigned long long &hi) {
     const uint32_t b = __float_as_uint(v);
     const int E = (int)((b >> 23) & 0xFFu);
-    if (E == 0) return;  // zero or subnormal: below the unit
+    lo = hi = 0ull;
+    if (E == 0) return false;  // zero or subnormal: below the unit
     const unsigned long long m = (unsigned long long)((b & 0x7FFFFFu) | 0x800000u);
     const int sh = E - 86;  // |v| * 2^64 = m * 2^(E - 150 + 64)
-    unsigned long long lo, hi;
-    if (sh <= -24) return;
-    if (sh < 0) lo = m >> (-sh), hi = 0ull;
-    else if (sh == 0) lo = m, hi = 0ull;
+    if (sh <= -24) return false;
+    if (sh < 0) lo = m >> (-sh);
+    else if (sh == 0) lo = m;
     else if (sh < 64) lo = m << sh, hi = m >> (64 - sh);
-    else if (sh < 102) lo = 0ull, hi = m << (sh - 64);
-    else lo = 0ull, hi = 1ull << 62;
+    else if (sh < 102) hi = m << (sh - 64);
+    else hi = 1ull << 62;
     if (b >> 31) {  // two's complement of the 128-bit magnitude
         lo = ~lo + 1ull;
         hi = ~hi + (lo == 0ull ? 1ull : 0ull);
     }
-    const unsigned long long old = atomicAdd(&acc[0], lo);
-    const unsigned long long up = hi + (old + lo < old ? 1ull : 0ull);
-    if (up) atomicAdd(&acc[1], up);
+    return true;
+}
+
+// Adds N values to N accumulators; the N low-word atomics are in flight together.
+template <int N> __device__ __forceinline__ void fix_add_n(unsigned long long *const (&acc)[N], const float (&v)[N]) {
+    unsigned long long lo[N], hi[N], old[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) old[k] = fix_of(v[k], lo[k], hi[k]) ? atomicAdd(&acc[k][0], lo[k]) : 0ull;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const unsigned long long up = hi[k] + (old[k] + lo[k] < old[k] ? 1ull : 0ull);
+        if (up) atomicAdd(&acc[k][1], up);
+    }
 }
 
 // Value of an accumulator pair once every addition into it is complete and visible.
@@ -360,9 +367,9 @@ cudaError_t launch_scan(const FrameDev &fr, int target_items, int kmin, cudaStre
 cudaError_t launch_scatter(int storage, const SceneDev &sc, const FrameDev &fr, bool stable, cudaStream_t st);
 cudaError_t launch_splat(const SceneDev &sc, const FrameDev &fr, int *queue, float *out,
                          int out_accum, int grid, cudaStream_t st);
-int splat_blocks_per_sm(int T);
-int splat_workers_per_sm(int T);
-int splat_split(int T);  // squares per tile edge the splat renders separately (1 or 2)
+int splat_blocks_per_sm();
+int splat_workers_per_sm();
+int splat_split(int T);  // regions of up to 16 px per tile edge, which the splat renders separately
 int bin_ctas_per_sm(int storage, size_t smem);
 
 // Raise a kernel's dynamic shared-memory limit on the current device to at least
@@ -411,7 +418,6 @@ int ordered_workers_per_sm();
 cudaError_t launch_item_order(const FrameDev &fr, cudaStream_t st);
 cudaError_t launch_splat_ordered(const SceneDev &sc, const FrameDev &fr, int *queue, float *out,
                                  const float *absorb, float *ord_scratch, int map_out, int grid, cudaStream_t st);
-size_t splat_smem_bytes(int T);
 cudaError_t launch_selftest_wait(long long limit, int *result, cudaStream_t st);
 cudaError_t launch_final(float *a, int64_t count, cudaStream_t st);
 cudaError_t launch_compose_maps(const float *maps, int n, int64_t pixels, float *out, cudaStream_t st);
