@@ -11,118 +11,114 @@
 // are sorted by depth (stably, from index order), their records are written out in that
 // order, and a stable sort by tile id groups them (depth-ordered binning).
 //
-// Layout as the additive warp kernel: one warp owns a square of up to 16 x 16 pixels (a
-// tile, or a quarter of a larger one), blocks of 8 x 4 pixels, one pixel of each block
-// per lane, state in registers.  Records are taken 32 at a time (decoded one per lane)
-// and applied strictly in list order.  Each lane keeps, per pixel and channel, the affine
-// map of the records applied so far, I_out = alpha I_in + beta: a tile that is not split
-// writes beta; the slices of a split tile store their maps, and the last slice to finish
-// composes them far to near.
-#include "splotch_internal.cuh"
+// Layout as the additive splat (splat_batch.cuh): a warp takes a region of up to 16 x 16 pixels
+// and batches of its records, lists them per 4 x 4-pixel square in list order, and evaluates a
+// square by a pair of lanes, 2 x 4 pixels each.  Each lane keeps, per pixel and channel, the
+// affine map of the records applied so far, I_out = alpha I_in + beta.  Where a square gets
+// several lane pairs, each takes a consecutive part of the list and the maps are composed by
+// shuffles; the map of a pass is composed onto the region's map in shared memory.  A tile that
+// is not split writes beta; the slices of a split tile store their maps, and the last slice to
+// finish composes them far to near.
+//
+// What bounds it: the FP32 pipe (69 % of its cycles on the 10 M-particle two-species frame; a
+// step is 168 to 300 packed operations, each two pipe cycles).  Hence the short polynomials, the
+// seven operations per channel (the update in u and 1 / s; eight with a and b apart) and squares
+// of 4 x 4 pixels: 6.7 squares, 107 pixel evaluations per particle, against 235 in the 8 x 8
+// units of a warp per record.  10 M particles at 2048^2: 3.33 -> 1.85 ms, a 1 M-particle map at
+// 1000 x 757: 0.73 -> 0.35 ms.  Batches of 192 (12 warps per SM): 128 on 16 warps took 2.47 ms
+// where 192 took 2.21.
+#include "splat_batch.cuh"
 
 namespace spl {
 
-constexpr int kOWarps = 4;     // warps per CTA
-constexpr int kOStage = 128;   // records per bulk copy, per warp
-constexpr int kONR = 4, kONC = 2;  // block rows x block columns of a 16 x 16 square
-constexpr float kOFar = 1e30f;
-
-struct __align__(16) ORec {
-    float X, Y, R2, kr;       // centre, support^2, Gaussian scale (w = 2^(d^2 kr))
-    float kxr, kxg, kxb, inv_s;  // A = s E per channel (x = A w); 1 / s (0 when s = 0)
-    float er, eg, eb;         // emission E
-    uint32_t mask;            // blocks (r * kONC + c) the record's box overlaps
-};
+constexpr int kOWarps = 2;    // warps per CTA
+constexpr int kOBatch = 192;  // records per batch
 
 struct __align__(16) OWarpSmem {
-    float4 buf[2][kOStage];
-    ORec dec[32];
-    uint64_t bar[2];
+    Batch<kOBatch> batch;            // pb: absorption A = s E per channel, and 1 / s
+    float map[6][kRegion][kRegion];  // the region's map: alpha r, g, b, beta r, g, b
 };
 
-// A record whose largest x = s E w (w <= 1) is small takes a series path: with
-// phi(x) = (1 - exp(-x)) / x = sum_k (-x)^k / (k + 1)!, a = 1 - x phi and b = E w phi, no
-// exponential per channel.  phi to degree 2 where x <= kSeries2Max (next term x^3 / 24
-// <= 1.5e-7 relative), to degree 5 where x <= kSeries5Max (x^6 / 7! <= 5e-8).
-constexpr float kSeries2Max = 0.015f, kSeries5Max = 0.25f;
-constexpr uint32_t kSeries5Flag = 1u << 31, kSeries2Flag = 1u << 30;  // in the record's block mask
+// Update of one record with x = s E w per pixel and channel and u = 1 - exp(-x):
+//     alpha <- alpha - u alpha,   beta <- beta + u (1 / s - beta),   u = x phi(x).
+// phi(x) = (1 - exp(-x)) / x is a polynomial whose degree follows the step's largest x (w <= 1,
+// so a record's x is at most its s E): degree 2 up to kDeg2Max and degree 3 up to kDeg3Max,
+// minimax with phi(0) = 1 (fitted here by iteratively reweighted least squares against expm1 in
+// 64 bits; largest relative errors 1.02e-7 and 1.19e-7).  Beyond, and for negative emissions,
+// the Taylor polynomial of degree 5 where |x| <= kTaylorMax (next term x^6 / 7! <= 5e-8) and
+// 1 - exp(-x) itself elsewhere, where the subtraction loses two bits at most.
+constexpr float kDeg2Max = 0.04f, kDeg3Max = 0.2f, kTaylorMax = 0.25f;
 
-// Per-lane state: the lane's pixels of block rows 2p and 2p + 1 (same column block c)
-// are held as the two halves of a float2, so that one packed FP32x2 instruction updates
-// both; a pair is computed when either of its two blocks is in the record's mask (a block
-// outside the record's box has no covered pixel, and an uncovered pixel's update is the
-// identity a = 1, b = 0).
-constexpr int kONP = kONR / 2;  // row pairs
+// Species that do not absorb (or hardly) use s raised to kLeastX / max E: alpha stays 1 in FP32
+// and u / s = E w to FP32 rounding.
+constexpr float kLeastX = 9.094947e-13f;  // 2^-40
 
-__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
+template <int kDeg> __device__ __forceinline__ float2 absorbed(float2 x) {  // u of degree kDeg (5: Taylor)
+    float2 phi;
+    if (kDeg == 5) {
+        phi = __ffma2_rn(x, f2(-1.0f / 720.0f), f2(1.0f / 120.0f));
+        phi = __ffma2_rn(x, phi, f2(-1.0f / 24.0f));
+        phi = __ffma2_rn(x, phi, f2(1.0f / 6.0f));
+        phi = __ffma2_rn(x, phi, f2(-0.5f));
+    } else if (kDeg == 3) {
+        phi = __ffma2_rn(x, f2(-0.03859227f), f2(0.16631325f));
+        phi = __ffma2_rn(x, phi, f2(-0.49998832f));
+    } else {
+        phi = __ffma2_rn(x, f2(0.16436407f), f2(-0.49997154f));
+    }
+    phi = __ffma2_rn(x, phi, f2(1.0f));
+    return __fmul2_rn(x, phi);
+}
 
-// Apply one record: per pixel and channel I <- a I + b, and the slice map's alpha <- a alpha.
-template <int kDeg>  // 2 or 5: series of that degree; 0: exponential
-__device__ __forceinline__ void apply_record(const float4 &pa, const float4 &pk, const float4 &pe, uint32_t m,
-                                             const float (&fx)[kONC], const float2 (&fy)[kONP],
-                                             float2 (&al)[kONP][kONC][3], float2 (&be)[kONP][kONC][3]) {
+// One step of a pass: every lane applies its record to its 2 x 4 pixels.  kDeg 5: the
+// exponential where x is beyond kTaylorMax.
+template <int kDeg>
+__device__ __forceinline__ void apply_record(const float4 &pa, const float4 &pb, const float2 (&fx)[2], const float2 &fy,
+                                             float2 (&al)[3][2][2], float2 (&be)[3][2][2]) {
+    const float kx[3] = {pb.x, pb.y, pb.z};
+    const float2 dx[2] = {__fadd2_rn(fx[0], f2(pa.x)), __fadd2_rn(fx[1], f2(pa.x))};
+    const float2 dy = __fadd2_rn(fy, f2(pa.y));
+    const float2 qx[2] = {__fmul2_rn(dx[0], dx[0]), __fmul2_rn(dx[1], dx[1])};
+    const float2 qy = __fmul2_rn(dy, dy);
 #pragma unroll
-    for (int q = 0; q < kONP; ++q) {
-        // blocks (2q, c) and (2q + 1, c), c = 0, 1: mask bits 4q .. 4q + 3
-        if (!(m & (0xFu << (4 * q)))) continue;
-        const float2 dy = __fadd2_rn(fy[q], f2(-pa.y));
-        const float2 dy2 = __fmul2_rn(dy, dy);
+    for (int row = 0; row < 2; ++row) {
+        const float2 qr = f2(row ? qy.y : qy.x);
 #pragma unroll
-        for (int c = 0; c < kONC; ++c) {
-            if (!(m & ((1u << c) | (1u << (kONC + c))) << (4 * q))) continue;
-            const float dx = __fsub_rn(fx[c], pa.x);
-            const float2 d2 = __fadd2_rn(f2(__fmul_rn(dx, dx)), dy2);
-            const float2 e = __fmul2_rn(d2, f2(pa.w));
-            float2 w = make_float2(ex2_fast(e.x), ex2_fast(e.y));
-            w.x = d2.x < pa.z ? w.x : 0.0f;  // uncovered: a = 1, b = 0
-            w.y = d2.y < pa.z ? w.y : 0.0f;
-            const float kx[3] = {pk.x, pk.y, pk.z}, E[3] = {pe.x, pe.y, pe.z};
+        for (int cp = 0; cp < 2; ++cp) {
+            const float2 d2 = __fadd2_rn(qx[cp], qr);
+            const float2 g = __fmul2_rn(d2, f2(pa.w));
+            // uncovered: u = 0
+            const float2 w = make_float2(d2.x < pa.z ? ex2_fast(g.x) : 0.0f, d2.y < pa.z ? ex2_fast(g.y) : 0.0f);
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) {
                 const float2 x = __fmul2_rn(f2(kx[ch]), w);
-                float2 a, b;
-                if (kDeg > 0) {
-                    float2 phi;
-                    if (kDeg == 5) {
-                        phi = __ffma2_rn(x, f2(-1.0f / 720.0f), f2(1.0f / 120.0f));
-                        phi = __ffma2_rn(x, phi, f2(-1.0f / 24.0f));
-                        phi = __ffma2_rn(x, phi, f2(1.0f / 6.0f));
-                    } else {
-                        phi = f2(1.0f / 6.0f);
-                    }
-                    phi = __ffma2_rn(x, phi, f2(-0.5f));
-                    phi = __ffma2_rn(x, phi, f2(1.0f));
-                    a = __ffma2_rn(make_float2(-x.x, -x.y), phi, f2(1.0f));
-                    b = __fmul2_rn(__fmul2_rn(f2(E[ch]), w), phi);
-                } else {
-                    // a = exp(-x), b = (1 - a) / s.  Where x is small, 1 - a in FP32 would
-                    // cancel most digits: there phi to degree 2 (next term x^3 / 24), so
-                    // a = 1 - x phi and b = E w phi (also the s = 0 case)
-                    const float2 phi = __ffma2_rn(x, __ffma2_rn(x, f2(1.0f / 6.0f), f2(-0.5f)), f2(1.0f));
-                    const float2 as = __ffma2_rn(make_float2(-x.x, -x.y), phi, f2(1.0f));
-                    const float2 bs = __fmul2_rn(__fmul2_rn(f2(E[ch]), w), phi);
-                    const float2 ag = make_float2(ex2_fast(x.x * -kLog2e), ex2_fast(x.y * -kLog2e));
-                    const float2 bg = __ffma2_rn(make_float2(-ag.x, -ag.y), f2(pk.w), f2(pk.w));
-                    a = make_float2(x.x < 0.015f ? as.x : ag.x, x.y < 0.015f ? as.y : ag.y);
-                    b = make_float2(x.x < 0.015f ? bs.x : bg.x, x.y < 0.015f ? bs.y : bg.y);
+                float2 u = absorbed<kDeg>(x);
+                if (kDeg == 5) {
+                    const float2 y = __fmul2_rn(x, f2(-kLog2e));
+                    const float2 v = __fadd2_rn(f2(1.0f), make_float2(-ex2_fast(y.x), -ex2_fast(y.y)));
+                    u.x = fabsf(x.x) > kTaylorMax ? v.x : u.x;
+                    u.y = fabsf(x.y) > kTaylorMax ? v.y : u.y;
                 }
-                al[q][c][ch] = __fmul2_rn(al[q][c][ch], a);
-                be[q][c][ch] = __ffma2_rn(a, be[q][c][ch], b);
+                const float2 nu = make_float2(-u.x, -u.y);
+                al[ch][row][cp] = __ffma2_rn(nu, al[ch][row][cp], al[ch][row][cp]);
+                const float2 t = __fadd2_rn(f2(pb.w), make_float2(-be[ch][row][cp].x, -be[ch][row][cp].y));
+                be[ch][row][cp] = __ffma2_rn(u, t, be[ch][row][cp]);
             }
         }
     }
 }
 
-// Element (block row r, column block c, channel ch) of a lane's paired state.
-#define OSTATE(arr, r, c, ch) (((r) & 1) ? arr[(r) >> 1][c][ch].y : arr[(r) >> 1][c][ch].x)
-
-__global__ void __launch_bounds__(kOWarps * 32, 4)
+template <bool kEmit>
+__global__ void __launch_bounds__(kOWarps * 32, 6)
     k_splat_ordered(SceneDev sc, FrameDev fr, int *queue, float *out, int split,
                     const float *__restrict__ absorb, float *ord_scratch, int map_out) {
     if (fr.status[kStatOverflow]) return;
     extern __shared__ __align__(16) unsigned char s_raw[];
     OWarpSmem *ws = reinterpret_cast<OWarpSmem *>(s_raw) + (threadIdx.x >> 5);
+    Batch<kOBatch> *bt = &ws->batch;
+    constexpr int kRounds = Batch<kOBatch>::kRounds;
     const int lane = threadIdx.x & 31;
+    const int pair = lane >> 1;
     const int nt = fr.n_tiles;
     const int S2 = split * split;
     const int total_items = (int)fr.sizes[kSizeItems] * S2;
@@ -130,21 +126,17 @@ __global__ void __launch_bounds__(kOWarps * 32, 4)
     const ViewParams g0 = fr.views[0];
     const int T = g0.T, W = g0.W, H = g0.H, ntx = g0.ntx;
     const int sub = (T + split - 1) / split;
-    const int lc = lane & 7, lr = lane >> 3;
-
-    if (lane == 0) {
-        mbar_init(&ws->bar[0], 1);
-        mbar_init(&ws->bar[1], 1);
-        mbar_fence_init();
+    if (lane == 0) {  // covers nothing
+        bt->pa[kOBatch] = make_float4(0.0f, 0.0f, -1.0f, -1.0f);
+        bt->pb[kOBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
-    __syncwarp();
-    uint32_t phase0 = 0, phase1 = 0;
 
+    int next = 0;
+    if (lane == 0) next = atomicAdd(queue, 1);
     for (;;) {
-        int item = 0;
-        if (lane == 0) item = atomicAdd(queue, 1);
-        item = __shfl_sync(0xffffffffu, item, 0);
+        const int item = __shfl_sync(0xffffffffu, next, 0);
         if (item >= total_items) break;
+        if (lane == 0) next = atomicAdd(queue, 1);
 
         const int qs = item / S2, q = item - qs * S2;
         const int2 ord = __ldg(&fr.order[qs]);  // largest slices first
@@ -161,111 +153,137 @@ __global__ void __launch_bounds__(kOWarps * 32, 4)
         const int64_t seg1 = fr.offsets[gt + 1];
         const int64_t e0 = fr.offsets[gt] + (int64_t)chunk * K;
         const int nrec = (tw > 0 && th > 0) ? (int)(min(seg1, e0 + K) - e0) : 0;
-        const int nst = (nrec + kOStage - 1) / kOStage;
+        const float4 *recs = fr.lists + e0;
 
-        float fx[kONC];
-        float2 fy[kONP], al[kONP][kONC][3], be[kONP][kONC][3];
+        float *map = &ws->map[0][0][0];
 #pragma unroll
-        for (int c = 0; c < kONC; ++c) fx[c] = c * 8 + lc < tw ? (float)(px0 + c * 8 + lc) + 0.5f : kOFar;
-#pragma unroll
-        for (int q = 0; q < kONP; ++q) {
-            const int r0 = 2 * q, r1 = 2 * q + 1;
-            fy[q] = make_float2(r0 * 4 + lr < th ? (float)(py0 + r0 * 4 + lr) + 0.5f : kOFar,
-                                r1 * 4 + lr < th ? (float)(py0 + r1 * 4 + lr) + 0.5f : kOFar);
-#pragma unroll
-            for (int c = 0; c < kONC; ++c)
-#pragma unroll
-                for (int ch = 0; ch < 3; ++ch) al[q][c][ch] = f2(1.0f), be[q][c][ch] = f2(0.0f);
+        for (int k = 0; k < 6 * kRegion * kRegion / 128; ++k) {
+            const float id = k < 3 * kRegion * kRegion / 128 ? 1.0f : 0.0f;
+            reinterpret_cast<float4 *>(map)[k * 32 + lane] = make_float4(id, id, id, id);
         }
 
-        if (lane == 0 && nrec > 0) {
-            const int c0 = min(kOStage, nrec);
-            fence_proxy_async_smem();
-            mbar_arrive_expect_tx(&ws->bar[0], (uint32_t)c0 * 16u);
-            bulk_g2s(ws->buf[0], fr.lists + e0, (uint32_t)c0 * 16u, &ws->bar[0]);
-        }
-        for (int si = 0; si < nst; ++si) {
-            const int cb = si & 1;
-            if (lane == 0 && si + 1 < nst) {
-                const int nb = (si + 1) & 1;
-                const int cn = min(kOStage, nrec - (si + 1) * kOStage);
-                fence_proxy_async_smem();
-                mbar_arrive_expect_tx(&ws->bar[nb], (uint32_t)cn * 16u);
-                bulk_g2s(ws->buf[nb], fr.lists + e0 + (int64_t)(si + 1) * kOStage, (uint32_t)cn * 16u,
-                         &ws->bar[nb]);
-            }
-            const bool ok = mbar_wait_bounded(&ws->bar[cb], cb ? phase1 : phase0, kWaitCycles);
-            if (cb) phase1 ^= 1u; else phase0 ^= 1u;
-            if (!__all_sync(0xffffffffu, ok)) {
-                if (lane == 0) atomicExch(&fr.status[kStatTimeout], 1);
-                return;
-            }
-            const int cnt = min(kOStage, nrec - si * kOStage);
-            for (int g = 0; g < cnt; g += 32) {
-                // ---- decode: one record per lane
-                uint32_t mask = 0;
-                if (g + lane < cnt) {
-                    const float4 rec = ws->buf[cb][g + lane];
-                    const float X = rec.x, Y = rec.y, R = rec.z;
-                    const uint32_t code = __float_as_uint(rec.w);
-                    const float eps = 1e-3f + 2e-6f * (fabsf(X) + fabsf(Y) + R);
-                    const int ilo = max(0, (int)ceilf(clampf(X - R - 0.5f - eps, px0 - 1.0f, (float)(px0 + tw))) - px0);
-                    const int ihi = min(tw - 1, (int)floorf(clampf(X + R - 0.5f + eps, px0 - 1.0f, (float)(px0 + tw))) - px0);
-                    const int jlo = max(0, (int)ceilf(clampf(Y - R - 0.5f - eps, py0 - 1.0f, (float)(py0 + th))) - py0);
-                    const int jhi = min(th - 1, (int)floorf(clampf(Y + R - 0.5f + eps, py0 - 1.0f, (float)(py0 + th))) - py0);
-                    if (ilo <= ihi && jlo <= jhi) {
-                        const uint32_t cm = (2u << (ihi >> 3)) - (1u << (ilo >> 3));
-                        for (int r = jlo >> 2; r <= (jhi >> 2); ++r) mask |= cm << (r * kONC);
-                        int type;
-                        float er, eg, eb;
-                        if (sc.emit) {
-                            const float4 em = __ldg(&sc.emit[code]);  // the code is the particle index
-                            type = __float_as_int(em.w);
-                            er = em.x, eg = em.y, eb = em.z;
-                        } else {
-                            type = (int)(code >> 24);
-                            const float It = fminf((float)(code & kCodeMax) * (1.0f / (float)kCodeMax), 1.0f);
-                            const int len = __ldg(&sc.lut_len[type]);
-                            const float f = It * (float)(len - 1);
-                            const int kk = min((int)f, len - 2);
-                            const float tau = f - (float)kk;
-                            const int lo = __ldg(&sc.lut_off[type]) + kk;
-                            const float4 c0 = __ldg(&sc.lut[lo]);
-                            const float4 c1 = __ldg(&sc.lut[lo + 1]);
-                            er = (1.0f - tau) * c0.x + tau * c1.x;
-                            eg = (1.0f - tau) * c0.y + tau * c1.y;
-                            eb = (1.0f - tau) * c0.z + tau * c1.z;
-                        }
-                        const float s = __ldg(&absorb[type]);
-                        const float R2 = __fmul_rn(R, R);
-                        float4 *d = reinterpret_cast<float4 *>(&ws->dec[lane]);
-                        d[0] = make_float4(X, Y, R2, __fdividef(kexp, R2));
-                        d[1] = make_float4(s * er, s * eg, s * eb, s > 0.0f ? 1.0f / s : 0.0f);
-                        const float xmax = s * fmaxf(fabsf(er), fmaxf(fabsf(eg), fabsf(eb)));
-                        const uint32_t path = xmax <= kSeries2Max ? kSeries2Flag : (xmax <= kSeries5Max ? kSeries5Flag : 0u);
-                        d[2] = make_float4(er, eg, eb, __uint_as_float(mask | path));
+        const Region rg = make_region(px0, py0, tw, th);
+        batch_start(bt, recs, nrec);
+        int base = 0, row = 0;
+        while (base < nrec) {
+            const int nbuf = batch_fill<kEmit>(bt, rg, recs, nrec, base, row, sc.emit);
+            if (nbuf == 0) continue;
+
+            // ---- decode, one record per lane
+            uint32_t word[Batch<kOBatch>::kWords];
+            int cnt;
+            {
+                float4 rec[kRounds];
+#pragma unroll
+                for (int g = 0; g < kRounds; ++g) rec[g] = bt->pa[min(g * 32 + lane, nbuf - 1)];
+                cnt = batch_words<true, kOBatch>(rec, nbuf, rg, word);
+                float3 e[kRounds];
+                float s[kRounds];
+                if constexpr (kEmit) {
+                    copy_wait_all();
+                    __syncwarp();
+#pragma unroll
+                    for (int g = 0; g < kRounds; ++g) {
+                        const float4 em = bt->pb[min(g * 32 + lane, nbuf - 1)];
+                        e[g] = make_float3(em.x, em.y, em.z);
+                        s[g] = __ldg(&absorb[__float_as_int(em.w)]);
                     }
+                } else {
+                    batch_colours<kRounds>(rec, sc.lut, sc.lut_len, sc.lut_off, e);
+#pragma unroll
+                    for (int g = 0; g < kRounds; ++g) s[g] = __ldg(&absorb[__float_as_uint(rec[g].w) >> 24]);
                 }
-                uint32_t live = __ballot_sync(0xffffffffu, mask != 0);
                 __syncwarp();
-                // ---- apply the live records in list order (far to near)
-                while (live) {
-                    const int k = __ffs(live) - 1;
-                    live &= live - 1;
-                    const float4 pa = *reinterpret_cast<const float4 *>(&ws->dec[k].X);
-                    const float4 pk = *reinterpret_cast<const float4 *>(&ws->dec[k].kxr);
-                    const float4 pe = *reinterpret_cast<const float4 *>(&ws->dec[k].er);
-                    const uint32_t m = __float_as_uint(pe.w);
-                    if (m & kSeries2Flag)
-                        apply_record<2>(pa, pk, pe, m, fx, fy, al, be);
-                    else if (m & kSeries5Flag)
-                        apply_record<5>(pa, pk, pe, m, fx, fy, al, be);
+#pragma unroll
+                for (int g = 0; g < kRounds; ++g) {
+                    const int j = g * 32 + lane;
+                    if (j >= nbuf) break;
+                    const float R2 = __fmul_rn(rec[g].z, rec[g].z);
+                    const float emax = fmaxf(fabsf(e[g].x), fmaxf(fabsf(e[g].y), fabsf(e[g].z)));
+                    const float sa = emax > 0.0f ? fmaxf(s[g], kLeastX / emax) : 1.0f;
+                    bt->pa[j] = make_float4(-rec[g].x, -rec[g].y, R2, gauss_scale(kexp, R2));
+                    bt->pb[j] = make_float4(sa * e[g].x, sa * e[g].y, sa * e[g].z, 1.0f / sa);
+                }
+            }
+            int before, total;
+            const uint32_t key = sort_squares(batch_lists<true>(bt, word, cnt), before, total);
+
+            // ---- passes over the squares
+            for (int i = 0; i < 16;) {
+                const int lead = (int)(__shfl_sync(0xffffffffu, key, i) >> 4);
+                if (lead == 0) break;
+                const int a = choose_split<160, 220, 150>(i, lead, before, total);
+                const int place = i + (pair >> a), r = pair & ((1 << a) - 1);
+                const uint32_t kp = __shfl_sync(0xffffffffu, key, place & 15);
+                const int sq = (int)(kp & 15u);
+                const int n = place < 16 ? (int)(kp >> 4) : 0;
+                const int steps = (lead + (1 << a) - 1) >> a;
+                // this pair's consecutive part of the list
+                const int part = (n + (1 << a) - 1) >> a;
+                const int mine = min(part, n - r * part);
+                const unsigned char *lp = bt->list[sq] + r * part;
+                const int x = 4 * (sq & 3), y = 4 * (sq >> 2) + 2 * (lane & 1);
+                const float fx0 = (float)(px0 + x) + 0.5f, fy0 = (float)(py0 + y) + 0.5f;
+                const float2 fx[2] = {make_float2(fx0, fx0 + 1.0f), make_float2(fx0 + 2.0f, fx0 + 3.0f)};
+                const float2 fy = make_float2(fy0, fy0 + 1.0f);
+                float2 al[3][2][2], be[3][2][2];  // channel, row, column pair
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) al[c][k >> 1][k & 1] = f2(1.0f), be[c][k >> 1][k & 1] = f2(0.0f);
+                int idx = mine > 0 ? *lp : kOBatch;
+#pragma unroll 1
+                for (int k = 1; k <= steps; ++k) {
+                    const float4 pa = bt->pa[idx];
+                    const float4 pb = bt->pb[idx];
+                    ++lp;
+                    idx = k < mine ? *lp : kOBatch;
+                    // as unsigned integers, so that a negative emission counts as the largest
+                    const uint32_t xmax = max(__float_as_uint(pb.x), max(__float_as_uint(pb.y), __float_as_uint(pb.z)));
+                    if (!__any_sync(0xffffffffu, xmax > __float_as_uint(kDeg2Max)))
+                        apply_record<2>(pa, pb, fx, fy, al, be);
+                    else if (!__any_sync(0xffffffffu, xmax > __float_as_uint(kDeg3Max)))
+                        apply_record<3>(pa, pb, fx, fy, al, be);
                     else
-                        apply_record<0>(pa, pk, pe, m, fx, fy, al, be);
+                        apply_record<5>(pa, pb, fx, fy, al, be);
+                }
+                // compose the maps of a square's pairs, parts in list order
+                for (int d = 2; d < (2 << a); d <<= 1) {
+                    const bool near = (lane & d) != 0;  // this lane's part is applied after the other's
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            float2 &A = al[c][k >> 1][k & 1], &B = be[c][k >> 1][k & 1];
+                            const float2 oa = make_float2(__shfl_xor_sync(0xffffffffu, A.x, d),
+                                                          __shfl_xor_sync(0xffffffffu, A.y, d));
+                            const float2 ob = make_float2(__shfl_xor_sync(0xffffffffu, B.x, d),
+                                                          __shfl_xor_sync(0xffffffffu, B.y, d));
+                            B = __ffma2_rn(near ? A : oa, near ? ob : B, near ? B : ob);
+                            A = __fmul2_rn(A, oa);
+                        }
+                }
+                if (r == 0 && n > 0) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+#pragma unroll
+                        for (int rr = 0; rr < 2; ++rr) {
+                            float4 *pA = reinterpret_cast<float4 *>(&ws->map[c][y + rr][x]);
+                            float4 *pB = reinterpret_cast<float4 *>(&ws->map[3 + c][y + rr][x]);
+                            const float2 a0 = al[c][rr][0], a1 = al[c][rr][1], b0 = be[c][rr][0], b1 = be[c][rr][1];
+                            float4 A = *pA, B = *pB;
+                            B.x = fmaf(a0.x, B.x, b0.x), B.y = fmaf(a0.y, B.y, b0.y);
+                            B.z = fmaf(a1.x, B.z, b1.x), B.w = fmaf(a1.y, B.w, b1.y);
+                            A.x *= a0.x, A.y *= a0.y, A.z *= a1.x, A.w *= a1.y;
+                            *pA = A;
+                            *pB = B;
+                        }
                 }
                 __syncwarp();
+                i += 16 >> a;
             }
         }
+        __syncwarp();
 
         // epilogue: a whole tile writes I = beta (black background), or with map_out the
         // map (alpha rgb, beta rgb); a slice of a split tile stores its map, and the last
@@ -273,39 +291,16 @@ __global__ void __launch_bounds__(kOWarps * 32, 4)
         const int oc = map_out ? 6 : 3;  // floats per pixel
         float *o = out + (int64_t)v * H * W * oc;
         if (slot < 0) {
-#pragma unroll
-            for (int r = 0; r < kONR; ++r) {
-                if (r * 4 + lr >= th) continue;
-#pragma unroll
-                for (int c = 0; c < kONC; ++c) {
-                    if (c * 8 + lc >= tw) continue;
-                    float *p = o + ((int64_t)(py0 + r * 4 + lr) * W + px0 + c * 8 + lc) * oc;
-                    if (map_out) {
-                        p[0] = OSTATE(al, r, c, 0);
-                        p[1] = OSTATE(al, r, c, 1);
-                        p[2] = OSTATE(al, r, c, 2);
-                        p += 3;
-                    }
-                    p[0] = OSTATE(be, r, c, 0);
-                    p[1] = OSTATE(be, r, c, 1);
-                    p[2] = OSTATE(be, r, c, 2);
-                }
+            for (int k = lane; k < kRegion * kRegion * oc; k += 32) {
+                const int p = k / oc, c = k - p * oc, r = p / kRegion, col = p % kRegion;
+                if (r < th && col < tw)
+                    o[((int64_t)(py0 + r) * W + px0 + col) * oc + c] = ws->map[map_out ? c : 3 + c][r][col];
             }
         } else {
-            float *map = ord_scratch + (int64_t)slice * 6 * T * T;  // [alpha r g b, beta r g b][T][T]
-#pragma unroll
-            for (int r = 0; r < kONR; ++r) {
-                if (r * 4 + lr >= th) continue;
-#pragma unroll
-                for (int c = 0; c < kONC; ++c) {
-                    if (c * 8 + lc >= tw) continue;
-                    const int pix = (qy + r * 4 + lr) * T + qx + c * 8 + lc;
-#pragma unroll
-                    for (int ch = 0; ch < 3; ++ch) {
-                        map[ch * T * T + pix] = OSTATE(al, r, c, ch);
-                        map[(3 + ch) * T * T + pix] = OSTATE(be, r, c, ch);
-                    }
-                }
+            float *ms = ord_scratch + (int64_t)slice * 6 * T * T;  // [alpha r g b, beta r g b][T][T]
+            for (int k = lane; k < 6 * kRegion * kRegion; k += 32) {
+                const int c = k / (kRegion * kRegion), r = (k / kRegion) % kRegion, col = k % kRegion;
+                if (r < th && col < tw) ms[c * T * T + (qy + r) * T + qx + col] = map[k];
             }
             __threadfence();
             __syncwarp();
@@ -323,17 +318,17 @@ __global__ void __launch_bounds__(kOWarps * 32, 4)
                     const int pix = rr * T + col;
                     float A = 1.0f, I = 0.0f;
                     for (int sl = s0; sl < s1; ++sl) {
-                        const float *ms = ord_scratch + (int64_t)sl * 6 * T * T;
-                        const float a = __ldcg(&ms[ch * T * T + pix]);
-                        I = fmaf(a, I, __ldcg(&ms[(3 + ch) * T * T + pix]));
+                        const float *m = ord_scratch + (int64_t)sl * 6 * T * T;
+                        const float a = __ldcg(&m[ch * T * T + pix]);
+                        I = fmaf(a, I, __ldcg(&m[(3 + ch) * T * T + pix]));
                         A *= a;
                     }
-                    float *q = ot + (int64_t)rr * W * oc + col * oc;
+                    float *p = ot + (int64_t)rr * W * oc + col * oc;
                     if (map_out) {
-                        q[ch] = A;
-                        q[3 + ch] = I;
+                        p[ch] = A;
+                        p[3 + ch] = I;
                     } else {
-                        q[ch] = I;
+                        p[ch] = I;
                     }
                 }
                 if (lane == 0) fr.tickets[slot] = 0;
@@ -362,11 +357,10 @@ int ordered_split(int T) { return T > 16 ? 2 : 1; }
 static size_t ordered_smem() { return sizeof(OWarpSmem) * kOWarps; }
 
 int ordered_ctas_per_sm() {
-    if (ensure_smem_limit((const void *)k_splat_ordered, ordered_smem()) != cudaSuccess) return 1;
+    const void *fn = (const void *)k_splat_ordered<false>;
+    if (ensure_smem_limit(fn, ordered_smem()) != cudaSuccess) return 1;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_splat_ordered, kOWarps * 32, ordered_smem()) !=
-        cudaSuccess)
-        return 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kOWarps * 32, ordered_smem()) != cudaSuccess) return 1;
     return std::max(1, nb);
 }
 
@@ -403,11 +397,11 @@ cudaError_t launch_compose_maps(const float *maps, int n, int64_t pixels, float 
 
 cudaError_t launch_splat_ordered(const SceneDev &sc, const FrameDev &fr, int *queue, float *out,
                                  const float *absorb, float *ord_scratch, int map_out, int grid, cudaStream_t st) {
-    cudaError_t err = ensure_smem_limit((const void *)k_splat_ordered, ordered_smem());
+    auto fn = sc.emit ? k_splat_ordered<true> : k_splat_ordered<false>;
+    cudaError_t err = ensure_smem_limit((const void *)fn, ordered_smem());
     if (err != cudaSuccess) return err;
     if ((err = launch_item_order(fr, st)) != cudaSuccess) return err;
-    k_splat_ordered<<<grid, kOWarps * 32, ordered_smem(), st>>>(sc, fr, queue, out, ordered_split(fr.T), absorb,
-                                                                ord_scratch, map_out);
+    fn<<<grid, kOWarps * 32, ordered_smem(), st>>>(sc, fr, queue, out, ordered_split(fr.T), absorb, ord_scratch, map_out);
     return cudaGetLastError();
 }
 

@@ -40,7 +40,7 @@
 // instead of 16 (6.7 ms); scalar instead of packed arithmetic: 18 more instructions per step
 // (6.5 ms against 6.1 before the loop was unrolled); unrolling by 3 drops the copies of the
 // prefetched record (6.1 -> 5.75 ms).
-#include "splotch_internal.cuh"
+#include "splat_batch.cuh"
 
 namespace spl {
 
@@ -59,41 +59,13 @@ __device__ __forceinline__ void put_pixel(float *p, float a, int mode) {
     *p = mode == 2 ? *p + a : (mode ? a : -expm1f(-a));
 }
 
-constexpr int kRegion = 16;     // edge of the region a warp owns, in pixels
 constexpr int kWarpsPerCta = 2;
-constexpr int kBatch = 192;     // records per batch (list entries are 8-bit batch positions)
-constexpr int kAhead = 3;       // 32-record loads in flight
-constexpr int kRounds = kBatch / 32;            // records per lane of a full batch
-constexpr int kWords = (kBatch / 32 + 1) / 2;   // 32-record words per lane (two lanes share a square's words)
-static_assert(kBatch < 256 && kBatch % 32 == 0, "8-bit list entries; entry kBatch covers nothing");
+constexpr int kBatch = 192;  // records per batch
 
 struct __align__(16) WarpSmem {
-    float4 pa[kBatch + 1];           // raw record, then (-X, -Y, R^2, Gaussian scale); the last
-    float4 pb[kBatch + 1];           // entry covers nothing.  pb: emission r, g, b
+    Batch<kBatch> batch;             // pb: emission r, g, b
     float acc[3][kRegion][kRegion];  // the region's accumulator
-    // per square: batch positions of the records that meet it (a word of padding per square
-    // keeps equal places of the 16 lists in different banks)
-    unsigned char list[16][kBatch + 4];
-    float4 ring[kAhead][32];  // records on their way from the list
 };
-
-// 16 bytes from global to shared memory, asynchronously (LDGSTS)
-__device__ __forceinline__ void copy16_async(void *dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void copy_wait() {  // all but the newest N groups done
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void copy_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-__device__ __forceinline__ uint32_t leading_zeros(uint32_t v) {  // v != 0
-    uint32_t z;
-    asm("bfind.shiftamt.u32 %0, %1;" : "=r"(z) : "r"(v));
-    return z;
-}
-
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 
 // kViewScale: multiply every record's emission by a per-view, per-species scale (plans
 // with a brightness sequence); a separate instance, so plain renders carry no extra code.
@@ -103,8 +75,9 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
     if (fr.status[kStatOverflow]) return;  // no complete tile lists
     extern __shared__ __align__(16) unsigned char s_raw[];
     WarpSmem *ws = reinterpret_cast<WarpSmem *>(s_raw) + (threadIdx.x >> 5);
+    Batch<kBatch> *bt = &ws->batch;
+    constexpr int kRounds = Batch<kBatch>::kRounds;
     const int lane = threadIdx.x & 31;
-    const uint32_t lt_mask = (1u << lane) - 1u;
     const int nt = fr.n_tiles;
     const int N = fr.V * nt;
     const int S2 = split * split;
@@ -116,8 +89,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
     const int pair = lane >> 1;               // lane pair: the unit that evaluates a square
     const bool vec_rows = (W & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;  // 16-byte rows of 4 pixels
     if (lane == 0) {
-        ws->pa[kBatch] = make_float4(0.0f, 0.0f, -1.0f, -1.0f);
-        ws->pb[kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        bt->pa[kBatch] = make_float4(0.0f, 0.0f, -1.0f, -1.0f);
+        bt->pb[kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
 
     // the next item is taken from the queue while the current one is rendered
@@ -158,90 +131,23 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
         for (int k = 0; k < 3 * kRegion * kRegion / 128; ++k)
             reinterpret_cast<float4 *>(acc)[k * 32 + lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 
-        // A support that covers a pixel centre of the region lies within R of its centres' box:
-        // max(|X - xc|, |Y - yc|) < R + half; the widening exceeds the FP32 rounding at any
-        // position, so no covered pixel is left out
-        const float hx = 0.5f * (float)(tw - 1), hy = 0.5f * (float)(th - 1);
-        const float xc = (float)px0 + 0.5f + hx, yc = (float)py0 + 0.5f + hy;
-        const float half = fmaxf(hx, hy) + 1e-3f + 4e-6f * (xc + yc);
-        const float widen = 2.5e-4f + 1e-6f * (xc + yc);  // the same in squares
-        const uint32_t ex = (tw + 3) >> 2, ey = (th + 3) >> 2;  // square columns and rows
-        const float cx = -0.25f * ((float)px0 + 0.5f), cy = -0.25f * ((float)py0 + 0.5f);
-
-        // kAhead loads of 32 records ahead, through shared memory; a lane reads what it copied
-        // itself, so waiting for its own copies is enough
-#pragma unroll
-        for (int g = 0; g < kAhead; ++g) {
-            if (g * 32 + lane < nrec) copy16_async(&ws->ring[g][lane], recs + g * 32 + lane);
-            copy_commit();
-        }
-        int at = 0;  // ring row of the next 32 records
-        int base = 0;
+        const Region rg = make_region(px0, py0, tw, th);
+        batch_start(bt, recs, nrec);
+        int base = 0, row = 0;
         while (base < nrec) {
             // ---- 1. fill the batch with records that meet the region
-            int nbuf = 0;
-            __syncwarp();
-            while (base < nrec && nbuf <= kBatch - 32) {
-                copy_wait<kAhead - 1>();
-                const float4 rec = ws->ring[at][lane];
-                const bool live = base + lane < nrec && fmaxf(fabsf(rec.x - xc), fabsf(rec.y - yc)) <
-                                                            fmaf(rec.z, 1.000004f, half);
-                const uint32_t bal = __ballot_sync(0xffffffffu, live);
-                if (live) {
-                    const int j = nbuf + __popc(bal & lt_mask);
-                    ws->pa[j] = rec;
-                    if constexpr (kEmit)  // the record's last word is the particle index
-                        copy16_async(&ws->pb[j], &sc.emit[__float_as_uint(rec.w)]);
-                }
-                nbuf += __popc(bal);
-                // the ballot has consumed these records: their row takes the next copy
-                const int nx = base + 32 * kAhead + lane;
-                if (nx < nrec) copy16_async(&ws->ring[at][lane], recs + nx);
-                copy_commit();
-                at = at + 1 == kAhead ? 0 : at + 1;
-                base += 32;
-            }
+            const int nbuf = batch_fill<kEmit>(bt, rg, recs, nrec, base, row, sc.emit);
             if (nbuf == 0) continue;
-            __syncwarp();
 
-            // ---- 2. the squares a record's box meets, its colour and Gaussian scale, one record
-            // per lane.  The loads of all the batch's records go out together, stage by stage;
-            // lanes past the end repeat the last record.
-            uint32_t word[kWords];
-            int cnt = 0;
-#pragma unroll
-            for (int g = 0; g < kWords; ++g) word[g] = 0;
+            // ---- 2. squares, colour and Gaussian scale, one record per lane; lanes past the end
+            // repeat the last record
+            uint32_t word[Batch<kBatch>::kWords];
+            int cnt;
             {
                 float4 rec[kRounds];
 #pragma unroll
-                for (int g = 0; g < kRounds; ++g) rec[g] = ws->pa[min(g * 32 + lane, nbuf - 1)];
-                // Pixel p of the region (centre p0 + p + 0.5) lies in square p / 4, so the support
-                // [X - R, X + R] meets squares ceil((X - p0 - 0.5) / 4 - 3 / 4 - R / 4) up to
-                // floor((X - p0 - 0.5) / 4 + R / 4).  (A record that meets no column or row of the
-                // region gets an empty or a meaningless mask; its pixels are tested one by one, so
-                // it adds nothing either way.)  Ballots over the four columns and rows give each
-                // square its word of 32 records; lane s keeps the even words of square s, lane
-                // 16 + s the odd ones.
-#pragma unroll
-                for (int g = 0; g < kRounds; ++g) {
-                    const float rq = fmaf(rec[g].z, 0.250001f, widen);
-                    const float qx = fmaf(rec[g].x, 0.25f, cx), qy = fmaf(rec[g].y, 0.25f, cy);
-                    // first square and one past the last (conversions below 0 give 0)
-                    const uint32_t x0 = __float2uint_ru(qx - (rq + 0.75f)), y0 = __float2uint_ru(qy - (rq + 0.75f));
-                    const uint32_t x1 = min(ex, __float2uint_rd(qx + (rq + 1.0f)));
-                    const uint32_t y1 = min(ey, __float2uint_rd(qy + (rq + 1.0f)));
-                    const uint32_t m =
-                        g * 32 + lane < nbuf ? ((1u << x1) - (1u << x0)) + (((1u << y1) - (1u << y0)) << 4) : 0u;
-                    uint32_t b[8];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) b[k] = __ballot_sync(0xffffffffu, m & (1u << k));
-                    const uint32_t c = (lane & 2) ? ((lane & 1) ? b[3] : b[2]) : ((lane & 1) ? b[1] : b[0]);
-                    const uint32_t r = (lane & 8) ? ((lane & 4) ? b[7] : b[6]) : ((lane & 4) ? b[5] : b[4]);
-                    if ((lane >> 4) == (g & 1)) {
-                        word[g >> 1] = c & r;
-                        cnt += __popc(c & r);
-                    }
-                }
+                for (int g = 0; g < kRounds; ++g) rec[g] = bt->pa[min(g * 32 + lane, nbuf - 1)];
+                cnt = batch_words<false, kBatch>(rec, nbuf, rg, word);
                 float3 e[kRounds];
                 float vs[kRounds];
                 if constexpr (kEmit) {
@@ -250,7 +156,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
                     if constexpr (kViewScale)
 #pragma unroll
                         for (int g = 0; g < kRounds; ++g) {
-                            const float4 em = ws->pb[min(g * 32 + lane, nbuf - 1)];
+                            const float4 em = bt->pb[min(g * 32 + lane, nbuf - 1)];
                             e[g] = make_float3(em.x, em.y, em.z);
                             vs[g] = __ldg(&fr.vscale[v * sc.n_types + __float_as_int(em.w)]);
                         }
@@ -259,31 +165,10 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
                     const float4 *lut = kViewScale ? fr.vlut : sc.lut;
                     const int *lut_len = kViewScale ? fr.vlut_len + v * sc.n_types : sc.lut_len;
                     const int *lut_off = kViewScale ? fr.vlut_off + v * sc.n_types : sc.lut_off;
-                    int len[kRounds], off[kRounds];
-#pragma unroll
-                    for (int g = 0; g < kRounds; ++g) {
-                        const int type = (int)(__float_as_uint(rec[g].w) >> 24);
-                        len[g] = __ldg(&lut_len[type]);
-                        off[g] = __ldg(&lut_off[type]);
-                        vs[g] = kViewScale ? __ldg(&fr.vscale[v * sc.n_types + type]) : 1.0f;
-                    }
-                    float4 c0[kRounds], c1[kRounds];
-                    float tau[kRounds];
-#pragma unroll
-                    for (int g = 0; g < kRounds; ++g) {
-                        const uint32_t code = __float_as_uint(rec[g].w);
-                        const float It = fminf((float)(code & kCodeMax) * (1.0f / (float)kCodeMax), 1.0f);
-                        const float f = It * (float)(len[g] - 1);
-                        const int kk = min((int)f, len[g] - 2);
-                        tau[g] = f - (float)kk;
-                        c0[g] = __ldg(&lut[off[g] + kk]);
-                        c1[g] = __ldg(&lut[off[g] + kk + 1]);
-                    }
+                    batch_colours<kRounds>(rec, lut, lut_len, lut_off, e);
 #pragma unroll
                     for (int g = 0; g < kRounds; ++g)
-                        e[g] = make_float3((1.0f - tau[g]) * c0[g].x + tau[g] * c1[g].x,
-                                           (1.0f - tau[g]) * c0[g].y + tau[g] * c1[g].y,
-                                           (1.0f - tau[g]) * c0[g].z + tau[g] * c1[g].z);
+                        vs[g] = kViewScale ? __ldg(&fr.vscale[v * sc.n_types + (__float_as_uint(rec[g].w) >> 24)]) : 1.0f;
                 }
                 __syncwarp();
 #pragma unroll
@@ -291,97 +176,28 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
                     const int j = g * 32 + lane;
                     if (j >= nbuf) break;
                     const float R2 = __fmul_rn(rec[g].z, rec[g].z);
-                    // the scale is kept finite and nonzero, so that distance^2 x scale is never
-                    // NaN (R^2 may underflow to 0 or overflow; the comparison with R^2 decides)
-                    const float kr = fminf(fmaxf(__fdividef(kexp, R2), -1e30f), -1.2e-38f);
-                    ws->pa[j] = make_float4(-rec[g].x, -rec[g].y, R2, kr);
+                    bt->pa[j] = make_float4(-rec[g].x, -rec[g].y, R2, gauss_scale(kexp, R2));
                     if constexpr (kViewScale || !kEmit)
-                        ws->pb[j] = make_float4(e[g].x * vs[g], e[g].y * vs[g], e[g].z * vs[g], 0.0f);
+                        bt->pb[j] = make_float4(e[g].x * vs[g], e[g].y * vs[g], e[g].z * vs[g], 0.0f);
                 }
             }
 
-            // ---- 3. per square, the batch positions of its records
-            const int other = __shfl_xor_sync(0xffffffffu, cnt, 16);
-            {
-                int dst = lane < 16 ? 0 : other;
-                // a lane with more than twice the mean is unpacked by the whole warp, a word at
-                // a time, so that a dense square does not hold up the others
-                const int all = __reduce_add_sync(0xffffffffu, cnt);
-                const bool heavy = cnt > max(8, all >> 4);
-                for (uint32_t todo = __ballot_sync(0xffffffffu, heavy); todo; todo &= todo - 1) {
-                    const int src = __ffs(todo) - 1;
-                    int at = __shfl_sync(0xffffffffu, dst, src);
-#pragma unroll
-                    for (int g = 0; g < kWords; ++g) {
-                        const uint32_t w = __shfl_sync(0xffffffffu, word[g], src);
-                        if ((w >> lane) & 1u)
-                            ws->list[src & 15][at + __popc(w & lt_mask)] =
-                                (unsigned char)((2 * g + (src >> 4)) * 32 + lane);
-                        at += __popc(w);
-                    }
-                }
-                if (!heavy) {
-                    unsigned char *p = ws->list[lane & 15] + dst;
-#pragma unroll
-                    for (int g = 0; g < kWords; ++g) {
-                        const int first = (2 * g + (lane >> 4)) * 32 + 31;
-                        uint32_t w = word[g];
-                        while (w) {
-                            const uint32_t z = leading_zeros(w);
-                            *p++ = (unsigned char)(first - z);
-                            w ^= 0x80000000u >> z;
-                        }
-                    }
-                }
-                __syncwarp();
-            }
-            // squares by list length, longest first: key = length, square (both half-warps sort
-            // the same 16 keys)
-            uint32_t key = ((uint32_t)(cnt + other) << 4) | (uint32_t)(lane & 15);
-#pragma unroll
-            for (int size = 2; size <= 16; size <<= 1)
-#pragma unroll
-                for (int d = size >> 1; d; d >>= 1) {
-                    const uint32_t o = __shfl_xor_sync(0xffffffffu, key, d);
-                    const bool first = (lane & d) == 0, down = (lane & size & 15) == 0;
-                    key = (first == down) ? max(key, o) : min(key, o);
-                }
-            // records before each place (exclusive), for the choice of the lane split
-            int before = (int)(key >> 4);
-#pragma unroll
-            for (int d = 1; d < 16; d <<= 1) {
-                const int u = __shfl_up_sync(0xffffffffu, before, d, 16);
-                if ((lane & 15) >= d) before += u;
-            }
-            const int total = __shfl_sync(0xffffffffu, before, 15);
-            before -= (int)(key >> 4);
-            __syncwarp();
+            // ---- 3. per square, the batch positions of its records; squares longest list first
+            int before, total;
+            const uint32_t key = sort_squares(batch_lists<false>(bt, word, cnt), before, total);
 
             // ---- 4. passes over the squares
             for (int i = 0; i < 16;) {
                 const int lead = (int)(__shfl_sync(0xffffffffu, key, i) >> 4);
                 if (lead == 0) break;
-                // lane split: 2^a pairs per square, 16 >> a squares; the a with the most
-                // records per instruction (about 64 per step of the loop, 36 per doubling for
-                // the shuffles, 60 per pass).  Lane a weighs option a.
-                int a;
-                {
-                    const int al = min(lane, 4);
-                    const int end = i + (16 >> al);
-                    const int upto = __shfl_sync(0xffffffffu, before, min(end, 15));
-                    const int from = __shfl_sync(0xffffffffu, before, i);
-                    const int covered = (end > 15 ? total : upto) - from;
-                    const int steps = (lead + (1 << al) - 1) >> al;
-                    const float gain = __fdividef((float)covered, (float)(64 * steps + 36 * al + 60));
-                    a = (int)(__reduce_max_sync(0xffffffffu, (__float_as_uint(gain) & ~7u) | (uint32_t)al) & 7u);
-                }
+                const int a = choose_split<64, 36, 60>(i, lead, before, total);
                 const int place = i + (pair >> a), r = pair & ((1 << a) - 1);
                 const uint32_t kp = __shfl_sync(0xffffffffu, key, place & 15);
                 const int sq = (int)(kp & 15u);
                 const int n = place < 16 ? (int)(kp >> 4) : 0;
                 const int mine = (n - r + (1 << a) - 1) >> a;  // list entries r, r + 2^a, ...
                 const int steps = (lead + (1 << a) - 1) >> a;
-                const unsigned char *lp = ws->list[sq] + r;
+                const unsigned char *lp = bt->list[sq] + r;
                 // this lane's pixels: rows y, y + 1 and columns x .. x + 3 of the region
                 const int x = 4 * (sq & 3), y = 4 * (sq >> 2) + 2 * (lane & 1);
                 const float fx = (float)(px0 + x) + 0.5f, fy0 = (float)(py0 + y) + 0.5f;
@@ -395,15 +211,15 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
                 // the records of the next step load while this one is evaluated; a pair past
                 // the end of its list takes the record that covers nothing
                 int idx = mine > 0 ? *lp : kBatch;
-                float4 na = ws->pa[idx], nb = ws->pb[idx];
+                float4 na = bt->pa[idx], nb = bt->pb[idx];
                 lp += 1 << a;
                 idx = mine > 1 ? *lp : kBatch;
 #pragma unroll 3
                 for (int k = 2; k < steps + 2; ++k) {
                     const float4 pa = na, pb = nb;
                     const float R2 = pa.z;
-                    na = ws->pa[idx];
-                    nb = ws->pb[idx];
+                    na = bt->pa[idx];
+                    nb = bt->pb[idx];
                     lp += 1 << a;
                     idx = k < mine ? *lp : kBatch;
                     const float2 dx0 = __fadd2_rn(fx0, f2(pa.x)), dx1 = __fadd2_rn(fx1, f2(pa.x));

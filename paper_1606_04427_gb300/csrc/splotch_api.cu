@@ -1868,8 +1868,9 @@ extern "C" splotch_status splotch_render_ordered(splotch_scene *sc, const splotc
     if (e == cudaSuccess)
         e = radix_sort_gather(tka, tkb, tva, tvb, P, 0, tbits, ex + o_tmp, (const float4 *)(ex + o_rec), fr.lists, st);
     const int64_t squares = (int64_t)std::max(1, items) * split * split;
+    const int per_cta = std::max(1, ordered_workers_per_sm() / ordered_ctas_per_sm());
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count(sc->dev) * ordered_ctas_per_sm(),
-                                                                (squares + 3) / 4));
+                                                                (squares + per_cta - 1) / per_cta));
     if (e == cudaSuccess)
         e = launch_splat_ordered(sc->dev_view, fr, (int *)(fixed + fh.o_queue), out, (const float *)(ex + o_abs),
                                  (float *)(ex + o_map), (rs.pr.flags & SPLOTCH_OUT_MAP) ? 1 : 0, grid, st);

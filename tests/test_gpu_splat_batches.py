@@ -77,3 +77,28 @@ def test_supports_whose_square_leaves_the_fp32_range():
     assert np.isfinite(got).all()
     want = oracle.render(ps, cam, oracle.Params(r_min_px=0.0))
     np.testing.assert_allclose(got, want, rtol=_rtol(n), atol=1e-12)
+
+
+@pytest.mark.parametrize("emax", [0.03, 0.06, 0.19, 0.24, 3.0])
+@pytest.mark.parametrize("kind,n", [("pixel", 193), ("square", 97), ("spread", 385), ("large", 64), ("large", 1)])
+def test_ordered_batch_edges_match_the_oracle(kind, n, emax):
+    """Batches of the depth-ordered splat, on every polynomial degree of the transfer and at
+    its limits (x up to 0.04, 0.2 and beyond), beside a species that does not absorb."""
+    rng = np.random.default_rng(n)
+    px, py, R = _layout(kind, n, rng)
+    x, y = _at(px, py)
+    half = n // 2
+    ps = P.make_set(x, y, rng.permutation(np.linspace(0.49, 0.51, n)), R / 0.75 * 2.0 / P.focal(H),
+                    rng.uniform(0.0, 1.0, n), type_begin=[0, half, n], betas=[emax, emax])
+    cam = P.front(W, H)
+    sc = render.Scene(ps, "f32")
+    absorb = [1.0, 0.0]
+    want = oracle.render_rt_depth(ps, cam, absorb)
+    # the weights' relative error 2.5e-6 (above) reaches I through each emission and through
+    # the absorption in front of it, at most tau of it; each of n updates rounds three times
+    # and its u is off by 1.2e-7 at most
+    tau = oracle.render(ps, cam).max()
+    rtol = 4e-6 * (1.0 + tau) + n * (3 * 2.0 ** -24 + 1.2e-7)
+    for T in (5, 16, 24, 32):
+        got = sc.render_ordered(cam, absorb, render.RenderParams(tile=T)).cpu().numpy()
+        np.testing.assert_allclose(got, want, rtol=rtol, atol=1e-12, err_msg=f"{kind} n={n} T={T}")
