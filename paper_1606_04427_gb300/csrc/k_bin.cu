@@ -284,15 +284,12 @@ __device__ __forceinline__ void count_particle(bool valid, float x, float y, flo
         }
         const bool small = tx1 >= tx0 && tx1 - tx0 <= 1 && ty1 - ty0 <= 1;
         if (small) {
-            const bool m00 = tile_member(vp, r.X, r.Y, r.R, tx0, ty0);
-            const bool m10 = tx1 > tx0 && tile_member(vp, r.X, r.Y, r.R, tx1, ty0);
-            const bool m01 = ty1 > ty0 && tile_member(vp, r.X, r.Y, r.R, tx0, ty1);
-            const bool m11 = tx1 > tx0 && ty1 > ty0 && tile_member(vp, r.X, r.Y, r.R, tx1, ty1);
+            const uint32_t m = tile_mask2(vp, r.X, r.Y, r.R, tx0, tx1, ty0, ty1);
             const int t00 = ty0 * vp.ntx + tx0;
-            if (m00) atomicAdd(&hist[t00], 1);
-            if (m10) atomicAdd(&hist[t00 + 1], 1);
-            if (m01) atomicAdd(&hist[t00 + vp.ntx], 1);
-            if (m11) atomicAdd(&hist[t00 + vp.ntx + 1], 1);
+            if (m & 1u) atomicAdd(&hist[t00], 1);
+            if (m & 2u) atomicAdd(&hist[t00 + 1], 1);
+            if (m & 4u) atomicAdd(&hist[t00 + vp.ntx], 1);
+            if (m & 8u) atomicAdd(&hist[t00 + vp.ntx + 1], 1);
         }
         uint32_t big = __ballot_sync(0xffffffffu, tx1 >= tx0 && !small);
         while (big) {
@@ -302,11 +299,11 @@ __device__ __forceinline__ void count_particle(bool valid, float x, float y, flo
             const float bR = __shfl_sync(0xffffffffu, r.R, src);
             const int bx0 = __shfl_sync(0xffffffffu, tx0, src), bx1 = __shfl_sync(0xffffffffu, tx1, src);
             const int by0 = __shfl_sync(0xffffffffu, ty0, src), by1 = __shfl_sync(0xffffffffu, ty1, src);
-            const int bw = bx1 - bx0 + 1, ncand = bw * (by1 - by0 + 1);
-            for (int k = lane; k < ncand; k += 32) {
-                const int ty = by0 + k / bw, tx = bx0 + k % bw;
-                if (tile_member(vp, bX, bY, bR, tx, ty)) atomicAdd(&hist[ty * vp.ntx + tx], 1);
-            }
+            // blocks of 8 x 4 candidates, one per lane
+            for (int ty = by0 + (lane >> 3); ty - (lane >> 3) <= by1; ty += 4)
+                for (int tx = bx0 + (lane & 7); tx - (lane & 7) <= bx1; tx += 8)
+                    if (tx <= bx1 && ty <= by1 && tile_member(vp, bX, bY, bR, tx, ty))
+                        atomicAdd(&hist[ty * vp.ntx + tx], 1);
         }
     }
 }
@@ -576,10 +573,8 @@ __device__ __forceinline__ void scatter_particle(bool valid, int64_t i, float x,
             // particle instead of one per tile
             const float4 rec = make_float4(r.X, r.Y, r.R, code);
             const int t00 = ty0 * vp.ntx + tx0;
-            const bool m00 = tile_member(vp, r.X, r.Y, r.R, tx0, ty0);
-            const bool m10 = tx1 > tx0 && tile_member(vp, r.X, r.Y, r.R, tx1, ty0);
-            const bool m01 = ty1 > ty0 && tile_member(vp, r.X, r.Y, r.R, tx0, ty1);
-            const bool m11 = tx1 > tx0 && ty1 > ty0 && tile_member(vp, r.X, r.Y, r.R, tx1, ty1);
+            const uint32_t m = tile_mask2(vp, r.X, r.Y, r.R, tx0, tx1, ty0, ty1);
+            const bool m00 = m & 1u, m10 = m & 2u, m01 = m & 4u, m11 = m & 8u;
             const int p00 = m00 ? atomicAdd(&cur[t00], 1) : 0;
             const int p10 = m10 ? atomicAdd(&cur[t00 + 1], 1) : 0;
             const int p01 = m01 ? atomicAdd(&cur[t00 + vp.ntx], 1) : 0;
@@ -605,17 +600,14 @@ __device__ __forceinline__ void scatter_particle(bool valid, int64_t i, float x,
             const int bid = __shfl_sync(0xffffffffu, (int)i, src);
             const int bx0 = __shfl_sync(0xffffffffu, tx0, src), bx1 = __shfl_sync(0xffffffffu, tx1, src);
             const int by0 = __shfl_sync(0xffffffffu, ty0, src), by1 = __shfl_sync(0xffffffffu, ty1, src);
-            const int bw = bx1 - bx0 + 1, ncand = bw * (by1 - by0 + 1);
             const float4 rec = make_float4(bX, bY, bR, bcode);
-            for (int k = lane; k < ncand; k += 32) {
-                const int ty = by0 + k / bw, tx = bx0 + k % bw;
-                if (tile_member(vp, bX, bY, bR, tx, ty)) {
-                    const int t = ty * vp.ntx + tx;
-                    const int pos = atomicAdd(&cur[t], 1);
-                    lists[pos] = rec;
-                    if (pids) pids[pos] = bid;
-                }
-            }
+            for (int ty = by0 + (lane >> 3); ty - (lane >> 3) <= by1; ty += 4)
+                for (int tx = bx0 + (lane & 7); tx - (lane & 7) <= bx1; tx += 8)
+                    if (tx <= bx1 && ty <= by1 && tile_member(vp, bX, bY, bR, tx, ty)) {
+                        const int pos = atomicAdd(&cur[ty * vp.ntx + tx], 1);
+                        lists[pos] = rec;
+                        if (pids) pids[pos] = bid;
+                    }
         }
     }
 }
@@ -711,23 +703,71 @@ template <int S> static cudaError_t scatter_impl(const SceneDev &sc, const Frame
 //   2. a block scan of the counts places every pair in the round's pair list, which is
 //      therefore in particle order; the pairs are staged in shared memory as (tile,
 //      particle slot), kStableStage at a time;
-//   3. every 32-pair slice finds, for each pair, the other pairs of its tile (the key
-//      bits compared with ballots) and its rank among them; then one warp walks the
-//      slices in order and, per tile of each slice, takes that many consecutive slots
-//      from the tile's cursor;
-//   4. all threads store the staged records at their slots (slice base + rank).
+//   3. the staged pairs are sorted by tile, stably, with a radix sort of 7 bits per pass in
+//      shared memory (one pass up to 128 tiles per view, else two);
+//   4. a tile's pairs are then consecutive: the first sets the tile's cursor relative to its
+//      place, all threads store the records at cursor + place (consecutive slots for a run),
+//      and the last moves the cursor past the run.
 // With the chunk bases in chunk order, every tile list is in ascending particle index
-// whatever the order in which CTAs and warps run, so images do not depend on it.  The
-// ranking costs about twice the scatter's time; renders ask for it with SPLOTCH_STABLE.
+// whatever the order in which CTAs and warps run, so images do not depend on it.  Renders ask
+// for it with SPLOTCH_STABLE.
 
-constexpr int kStableStage = 2048;  // staged pairs per window
-// shared memory beyond the cursors: round records, staged keys, slots and slice ranks
-constexpr size_t kStableExtra = sizeof(float4) * kThreads + (sizeof(int) + 2 * sizeof(unsigned short)) * kStableStage;
-// key bits compared per slice: tile indices are below kMaxTiles = 2^14, and bit 14 marks
-// the lanes past the window's end
-constexpr int kTileKeyBits = 15;
-constexpr uint32_t kNoTile = 1u << 14;
-static_assert(kMaxTiles <= (int)kNoTile, "tile keys need more bits");
+constexpr int kStableStage = 4096;  // staged pairs per window
+constexpr int kSlotBits = 10;       // particle slot in a staged pair (kThreads of them), tile above
+static_assert(kThreads == 1 << kSlotBits && kMaxTiles <= 1 << 14, "staged pair: 14-bit tile, 10-bit slot");
+constexpr int kDigitBits = 7, kDigits = 1 << kDigitBits, kBinWarps = kThreads / 32;
+constexpr int kSortRows = kStableStage / kThreads;  // staged pairs per lane
+// shared memory beyond the cursors: round records, two buffers of staged pairs, and the sort's
+// counters (digit-major, one per warp, padded against bank conflicts)
+constexpr size_t kStableExtra =
+    sizeof(float4) * kThreads + sizeof(uint32_t) * (2 * kStableStage + kDigits * (kBinWarps + 1));
+
+// One stable counting-sort pass of src[0, m) by 7 bits into dst, by the whole CTA: warps own
+// consecutive parts and rank their pairs in order, and the exclusive scan of the counters in
+// (digit, warp) order is where each warp's pairs of a digit go.
+__device__ __forceinline__ void sort_pairs_pass(const uint32_t *src, uint32_t *dst, int m, int shift, uint32_t *cnt,
+                                                int *s_scan) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    for (int k = tid; k < kDigits * (kBinWarps + 1); k += kThreads) cnt[k] = 0;
+    __syncthreads();
+    const int rows = (m + kThreads - 1) / kThreads;  // 32-pair rows per warp
+    const int first = warp * rows * 32 + lane;
+    uint32_t key[kSortRows];
+    int rank[kSortRows];
+#pragma unroll
+    for (int r = 0; r < kSortRows; ++r) {
+        if (r >= rows) break;
+        const int j = first + r * 32;
+        key[r] = j < m ? src[j] : 0u;
+        const uint32_t d = j < m ? (key[r] >> shift) & (kDigits - 1) : kDigits;
+        const uint32_t peers = warp_peers<kDigitBits + 1>(d);
+        const int leader = __ffs(peers) - 1;
+        int before = 0;
+        if (j < m && lane == leader) {
+            before = (int)cnt[d * (kBinWarps + 1) + warp];
+            cnt[d * (kBinWarps + 1) + warp] = before + __popc(peers);
+        }
+        rank[r] = __shfl_sync(0xffffffffu, before, leader) + __popc(peers & lt);
+        __syncwarp();
+    }
+    __syncthreads();
+    // thread t scans counters 4 t .. 4 t + 3 of the (digit, warp) sequence
+    static_assert(kDigits * kBinWarps == 4 * kThreads, "four counters per thread");
+    uint32_t *c = cnt + (tid >> 3) * (kBinWarps + 1) + 4 * (tid & 7);
+    const int c0 = (int)c[0], c1 = (int)c[1], c2 = (int)c[2], c3 = (int)c[3];
+    int all;
+    const int base = block_excl_scan<int>(c0 + c1 + c2 + c3, s_scan, &all);
+    c[0] = base, c[1] = base + c0, c[2] = base + c0 + c1, c[3] = base + c0 + c1 + c2;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSortRows; ++r) {
+        if (r >= rows) break;
+        if (first + r * 32 < m)
+            dst[cnt[((key[r] >> shift) & (kDigits - 1)) * (kBinWarps + 1) + warp] + rank[r]] = key[r];
+    }
+    __syncthreads();
+}
 
 // Member tiles of a particle whose candidate box is large, tested by the whole warp (one
 // candidate per lane, candidates in row-major order).  With kStage false, returns the
@@ -735,8 +775,8 @@ static_assert(kMaxTiles <= (int)kNoTile, "tile keys need more bits");
 // indices off, off + 1, ... (off: the particle's first pair).
 template <bool kStage>
 __device__ __forceinline__ int big_members(const ViewParams &vp, float X, float Y, float R, int bx0, int bx1,
-                                           int by0, int by1, int off, int w0, int m, int slot, int *s_key,
-                                           unsigned short *s_slot, int lane) {
+                                           int by0, int by1, int off, int w0, int m, int slot, uint32_t *s_pair,
+                                           int lane) {
     const int bw = bx1 - bx0 + 1, bh = by1 - by0 + 1;
     const uint32_t lt = (1u << lane) - 1u;
     int run = off - w0;
@@ -747,10 +787,8 @@ __device__ __forceinline__ int big_members(const ViewParams &vp, float X, float 
             const uint32_t bal = __ballot_sync(0xffffffffu, mem);
             if (kStage) {
                 const int j = run + __popc(bal & lt);
-                if (mem && (unsigned)j < (unsigned)m) {
-                    s_key[j] = ty * vp.ntx + tx;
-                    s_slot[j] = (unsigned short)slot;
-                }
+                if (mem && (unsigned)j < (unsigned)m)
+                    s_pair[j] = (uint32_t)(ty * vp.ntx + tx) << kSlotBits | (uint32_t)slot;
             }
             run += __popc(bal);
         }
@@ -762,15 +800,13 @@ template <int S>
 __global__ void __launch_bounds__(kThreads) k_scatter_stable(SceneDev sc, FrameDev fr) {
     if (fr.status[kStatOverflow]) return;
     extern __shared__ __align__(16) unsigned char s_raw[];
-    float4 *s_rec = reinterpret_cast<float4 *>(s_raw);                           // [kThreads]
-    int *s_key = reinterpret_cast<int *>(s_rec + kThreads);                      // [kStableStage]
-    unsigned short *s_slot = reinterpret_cast<unsigned short *>(s_key + kStableStage);  // [kStableStage]
-    // per staged pair: its slice's leader lane for its tile (5 bits), its rank among the
-    // slice's pairs of that tile (5 bits) and, at the leader, their count (6 bits)
-    unsigned short *s_info = s_slot + kStableStage;                              // [kStableStage]
+    float4 *s_rec = reinterpret_cast<float4 *>(s_raw);                     // [kThreads]
+    uint32_t *s_pair = reinterpret_cast<uint32_t *>(s_rec + kThreads);     // [kStableStage]
+    uint32_t *s_alt = s_pair + kStableStage;                               // [kStableStage]
+    uint32_t *s_cnt = s_alt + kStableStage;                                // [kDigits][kBinWarps + 1]
     // cursor of this chunk's slice of every tile segment, relative to the start of the
     // view's segments (a view holds fewer than 2^31 pairs: the scan checks it)
-    int *s_cur = reinterpret_cast<int *>(s_info + kStableStage);                // [g_n][n_tiles]
+    int *s_cur = reinterpret_cast<int *>(s_cnt + kDigits * (kBinWarps + 1));  // [g_n][n_tiles]
     __shared__ ViewParams s_view[kMaxGroup];
     __shared__ int64_t s_vbase[kMaxGroup];
     __shared__ int64_t s_tb[kMaxTypes + 1];
@@ -780,7 +816,6 @@ __global__ void __launch_bounds__(kThreads) k_scatter_stable(SceneDev sc, FrameD
     const int g_n = min(fr.G, fr.V - v0);
     const int nt = fr.n_tiles;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t lt = (1u << lane) - 1u;
     for (int k = tid; k < g_n * nt; k += blockDim.x) {
         const int g = k / nt, t = k - g * nt;
         const int64_t *seg = fr.offsets + (int64_t)(v0 + g) * nt;
@@ -825,10 +860,7 @@ __global__ void __launch_bounds__(kThreads) k_scatter_stable(SceneDev sc, FrameD
             // member bits of a small particle: (tx0, ty0), (tx1, ty0), (tx0, ty1), (tx1, ty1)
             uint32_t mask = 0;
             if (small) {
-                mask = (tile_member(vp, r.X, r.Y, r.R, tx0, ty0) ? 1u : 0u) |
-                       (tx1 > tx0 && tile_member(vp, r.X, r.Y, r.R, tx1, ty0) ? 2u : 0u) |
-                       (ty1 > ty0 && tile_member(vp, r.X, r.Y, r.R, tx0, ty1) ? 4u : 0u) |
-                       (tx1 > tx0 && ty1 > ty0 && tile_member(vp, r.X, r.Y, r.R, tx1, ty1) ? 8u : 0u);
+                mask = tile_mask2(vp, r.X, r.Y, r.R, tx0, tx1, ty0, ty1);
             }
             int cnt = __popc(mask);
             const uint32_t big = __ballot_sync(0xffffffffu, tx1 >= tx0 && !small);
@@ -838,7 +870,7 @@ __global__ void __launch_bounds__(kThreads) k_scatter_stable(SceneDev sc, FrameD
                     vp, __shfl_sync(0xffffffffu, r.X, src), __shfl_sync(0xffffffffu, r.Y, src),
                     __shfl_sync(0xffffffffu, r.R, src), __shfl_sync(0xffffffffu, tx0, src),
                     __shfl_sync(0xffffffffu, tx1, src), __shfl_sync(0xffffffffu, ty0, src),
-                    __shfl_sync(0xffffffffu, ty1, src), 0, 0, 0, 0, nullptr, nullptr, lane);
+                    __shfl_sync(0xffffffffu, ty1, src), 0, 0, 0, 0, nullptr, lane);
                 if (lane == src) cnt = n;
             }
             int M = 0;
@@ -856,10 +888,8 @@ __global__ void __launch_bounds__(kThreads) k_scatter_stable(SceneDev sc, FrameD
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         if (!((mask >> q) & 1u)) continue;
-                        if ((unsigned)j < (unsigned)m) {
-                            s_key[j] = t00 + (q & 1) + ((q >> 1) ? vp.ntx : 0);
-                            s_slot[j] = (unsigned short)tid;
-                        }
+                        if ((unsigned)j < (unsigned)m)
+                            s_pair[j] = (uint32_t)(t00 + (q & 1) + ((q >> 1) ? vp.ntx : 0)) << kSlotBits | (uint32_t)tid;
                         ++j;
                     }
                 }
@@ -869,44 +899,32 @@ __global__ void __launch_bounds__(kThreads) k_scatter_stable(SceneDev sc, FrameD
                                       __shfl_sync(0xffffffffu, r.R, src), __shfl_sync(0xffffffffu, tx0, src),
                                       __shfl_sync(0xffffffffu, tx1, src), __shfl_sync(0xffffffffu, ty0, src),
                                       __shfl_sync(0xffffffffu, ty1, src), __shfl_sync(0xffffffffu, off, src), w0, m,
-                                      warp * 32 + src, s_key, s_slot, lane);
+                                      warp * 32 + src, s_pair, lane);
                 }
                 __syncthreads();
-                // ---- 3a. per 32-pair slice: the pairs of each tile and their ranks
-                for (int j0 = warp * 32; j0 < m; j0 += kThreads) {
-                    const int j = j0 + lane;
-                    const uint32_t t = j < m ? (uint32_t)s_key[j] : kNoTile;
-                    const uint32_t peers = warp_peers<kTileKeyBits>(t);
-                    const int leader = __ffs(peers) - 1;
-                    if (j < m)
-                        s_info[j] = (unsigned short)(leader | (__popc(peers & lt) << 5) |
-                                                     ((lane == leader ? __popc(peers) : 0) << 10));
+                // ---- 3. sort by tile, keeping particle order within a tile
+                sort_pairs_pass(s_pair, s_alt, m, kSlotBits, s_cnt, s_scan);
+                const uint32_t *sorted = s_alt;
+                if (nt > kDigits) {
+                    sort_pairs_pass(s_alt, s_pair, m, kSlotBits + kDigitBits, s_cnt, s_scan);
+                    sorted = s_pair;
                 }
-                __syncthreads();
-                // ---- 3b. slice bases in order: one warp; each slice's leader of a tile
-                // takes its pairs' slots from the cursor and leaves the first in s_key
-                if (warp == 0) {
-                    for (int j0 = 0; j0 < m; j0 += 32) {
-                        const int j = j0 + lane;
-                        if (j < m) {
-                            const int c = (int)(s_info[j] >> 10);
-                            if (c) {
-                                const int t = s_key[j];
-                                const int base = cur[t];
-                                cur[t] = base + c;
-                                s_key[j] = base;
-                            }
-                        }
-                    }
-                }
-                __syncthreads();
-                // ---- 4. records to their slots: the leader's base plus the rank
+                // ---- 4. records to their slots; a run's cursor is relative to its first place
                 for (int j = tid; j < m; j += kThreads) {
-                    const uint32_t inf = s_info[j];
-                    const int pos = s_key[(j & ~31) + (int)(inf & 31u)] + (int)((inf >> 5) & 31u);
-                    const int sl = s_slot[j];
+                    const uint32_t t = sorted[j] >> kSlotBits;
+                    if (j == 0 || sorted[j - 1] >> kSlotBits != t) cur[t] -= j;
+                }
+                __syncthreads();
+                for (int j = tid; j < m; j += kThreads) {
+                    const uint32_t p = sorted[j], sl = p & (kThreads - 1);
+                    const int pos = cur[p >> kSlotBits] + j;
                     lists[pos] = s_rec[sl];
                     if (pids) pids[pos] = (int)(r0 + sl);
+                }
+                __syncthreads();
+                for (int j = tid; j < m; j += kThreads) {
+                    const uint32_t t = sorted[j] >> kSlotBits;
+                    if (j + 1 == m || sorted[j + 1] >> kSlotBits != t) cur[t] += j + 1;
                 }
                 __syncthreads();
             }

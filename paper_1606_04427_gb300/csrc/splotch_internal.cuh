@@ -150,7 +150,7 @@ struct Raster {
 };
 
 __device__ __forceinline__ float clampf(float v, float lo, float hi) {
-    return v < lo ? lo : (v > hi ? hi : v);
+    return fminf(fmaxf(v, lo), hi);  // v is never NaN here
 }
 
 // Returns true when the particle is active: in front of the near plane, finite, and
@@ -204,6 +204,22 @@ __device__ __forceinline__ bool tile_member(const ViewParams &v, float X, float 
     const float q = __fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey));
     const float thr = __fadd_rn(R, v.hd);
     return q < __fmul_rn(thr, thr);
+}
+
+// Membership of up to 2 x 2 candidate tiles (tx0 .. tx1, ty0 .. ty1) by the same rule: bit 0
+// (tx0, ty0), 1 (tx1, ty0), 2 (tx0, ty1), 3 (tx1, ty1).  Tile centres are multiples of 1/2
+// below 2^21, so a neighbour's centre is exactly T further and the squares are shared.
+__device__ __forceinline__ uint32_t tile_mask2(const ViewParams &v, float X, float Y, float R, int tx0, int tx1,
+                                               int ty0, int ty1) {
+    const float T = (float)v.T;
+    const float cx = __fmul_rn(__fadd_rn((float)tx0, 0.5f), T), cy = __fmul_rn(__fadd_rn((float)ty0, 0.5f), T);
+    const float ex0 = __fsub_rn(cx, X), ex1 = __fsub_rn(__fadd_rn(cx, T), X);
+    const float ey0 = __fsub_rn(cy, Y), ey1 = __fsub_rn(__fadd_rn(cy, T), Y);
+    const float x0 = __fmul_rn(ex0, ex0), x1 = __fmul_rn(ex1, ex1), y0 = __fmul_rn(ey0, ey0), y1 = __fmul_rn(ey1, ey1);
+    const float thr = __fadd_rn(R, v.hd), thr2 = __fmul_rn(thr, thr);
+    const bool wide = tx1 > tx0, tall = ty1 > ty0;
+    return (__fadd_rn(x0, y0) < thr2 ? 1u : 0u) | (wide && __fadd_rn(x1, y0) < thr2 ? 2u : 0u) |
+           (tall && __fadd_rn(x0, y1) < thr2 ? 4u : 0u) | (wide && tall && __fadd_rn(x1, y1) < thr2 ? 8u : 0u);
 }
 
 // Lanes of the (full) warp whose key equals this lane's in the low NB bits, found bit by
