@@ -266,6 +266,9 @@ cudaError_t launch_prepare(const float *x, const float *y, const float *z, const
 
 // ---------------------------------------------------------------------------------------
 // k_count: raster a chunk of particles for up to G views and count tile memberships.
+// Bound by instruction issue (raster, tile tests, histogram atomics).  On the 100 M-particle
+// frame (FP16) 1.30 -> 1.20 ms with the shared squares of tile_mask2 and candidate blocks without
+// divisions, 1.11 ms with the attributes kept as stored until they are used.
 
 // Bin one particle for every view of the group: 2 x 2 candidate tiles or fewer by this
 // lane, larger candidate boxes by the whole warp (one such particle at a time).  Called by
@@ -329,19 +332,19 @@ __global__ void __launch_bounds__(kThreads) k_count(SceneDev sc, FrameDev fr) {
     const int lane = threadIdx.x & 31;
     const int64_t stride = blockDim.x;
     int64_t i = s + threadIdx.x;
-    float ax = 0.0f, ay = 0.0f, az = 0.0f, ah = 0.0f, bx = 0.0f, by = 0.0f, bz = 0.0f, bh = 0.0f;
-    if (i < e) ax = load1<S>(sc.x, i), ay = load1<S>(sc.y, i), az = load1<S>(sc.z, i), ah = load1<S>(sc.h, i);
+    typename Stored<S>::T ax{}, ay{}, az{}, ah{}, bx{}, by{}, bz{}, bh{};
+    if (i < e) ax = load_stored<S>(sc.x, i), ay = load_stored<S>(sc.y, i), az = load_stored<S>(sc.z, i), ah = load_stored<S>(sc.h, i);
     if (i + stride < e)
-        bx = load1<S>(sc.x, i + stride), by = load1<S>(sc.y, i + stride), bz = load1<S>(sc.z, i + stride),
-        bh = load1<S>(sc.h, i + stride);
+        bx = load_stored<S>(sc.x, i + stride), by = load_stored<S>(sc.y, i + stride), bz = load_stored<S>(sc.z, i + stride),
+        bh = load_stored<S>(sc.h, i + stride);
     for (; i - lane < e; i += 2 * stride) {
-        count_particle(i < e, ax, ay, az, ah, s_view, g_n, s_hist, nt, lane);
+        count_particle(i < e, value_of(ax), value_of(ay), value_of(az), value_of(ah), s_view, g_n, s_hist, nt, lane);
         const int64_t ia = i + 2 * stride;
-        if (ia < e) ax = load1<S>(sc.x, ia), ay = load1<S>(sc.y, ia), az = load1<S>(sc.z, ia), ah = load1<S>(sc.h, ia);
+        if (ia < e) ax = load_stored<S>(sc.x, ia), ay = load_stored<S>(sc.y, ia), az = load_stored<S>(sc.z, ia), ah = load_stored<S>(sc.h, ia);
         if (i + stride - lane >= e) break;
-        count_particle(i + stride < e, bx, by, bz, bh, s_view, g_n, s_hist, nt, lane);
+        count_particle(i + stride < e, value_of(bx), value_of(by), value_of(bz), value_of(bh), s_view, g_n, s_hist, nt, lane);
         const int64_t ib = i + 3 * stride;
-        if (ib < e) bx = load1<S>(sc.x, ib), by = load1<S>(sc.y, ib), bz = load1<S>(sc.z, ib), bh = load1<S>(sc.h, ib);
+        if (ib < e) bx = load_stored<S>(sc.x, ib), by = load_stored<S>(sc.y, ib), bz = load_stored<S>(sc.z, ib), bh = load_stored<S>(sc.h, ib);
     }
     __syncthreads();
     // this chunk's count of every tile (zeros included): k_chunk_scan turns the column of
@@ -651,33 +654,34 @@ __global__ void __launch_bounds__(kThreads) k_scatter(SceneDev sc, FrameDev fr) 
     const int64_t stride = blockDim.x;
     int type = 0;
     int64_t i = s + threadIdx.x;
-    float ax = 0.0f, ay = 0.0f, az = 0.0f, ah = 0.0f, ai = 0.0f;
-    float bx = 0.0f, by = 0.0f, bz = 0.0f, bh = 0.0f, bi = 0.0f;
+    typename Stored<S>::T ax{}, ay{}, az{}, ah{}, ai{}, bx{}, by{}, bz{}, bh{}, bi{};
     if (i < e)
-        ax = load1<S>(sc.x, i), ay = load1<S>(sc.y, i), az = load1<S>(sc.z, i), ah = load1<S>(sc.h, i),
-        ai = load1<S>(sc.it, i);
+        ax = load_stored<S>(sc.x, i), ay = load_stored<S>(sc.y, i), az = load_stored<S>(sc.z, i), ah = load_stored<S>(sc.h, i),
+        ai = load_stored<S>(sc.it, i);
     if (i + stride < e)
-        bx = load1<S>(sc.x, i + stride), by = load1<S>(sc.y, i + stride), bz = load1<S>(sc.z, i + stride),
-        bh = load1<S>(sc.h, i + stride), bi = load1<S>(sc.it, i + stride);
+        bx = load_stored<S>(sc.x, i + stride), by = load_stored<S>(sc.y, i + stride), bz = load_stored<S>(sc.z, i + stride),
+        bh = load_stored<S>(sc.h, i + stride), bi = load_stored<S>(sc.it, i + stride);
     for (; i - lane < e; i += 2 * stride) {
         if (i < e)
             while (type + 1 < sc.n_types && i >= s_tb[type + 1]) ++type;
-        scatter_particle(i < e, i, ax, ay, az, ah, sc.emit ? __uint_as_float((uint32_t)i) : record_code(type, ai),
+        scatter_particle(i < e, i, value_of(ax), value_of(ay), value_of(az), value_of(ah),
+                         sc.emit ? __uint_as_float((uint32_t)i) : record_code(type, value_of(ai)),
                          s_view, s_vbase, g_n, s_cur, nt, fr, lane);
         const int64_t ia = i + 2 * stride;
         if (ia < e)
-            ax = load1<S>(sc.x, ia), ay = load1<S>(sc.y, ia), az = load1<S>(sc.z, ia), ah = load1<S>(sc.h, ia),
-            ai = load1<S>(sc.it, ia);
+            ax = load_stored<S>(sc.x, ia), ay = load_stored<S>(sc.y, ia), az = load_stored<S>(sc.z, ia), ah = load_stored<S>(sc.h, ia),
+            ai = load_stored<S>(sc.it, ia);
         const int64_t j = i + stride;
         if (j - lane >= e) break;
         if (j < e)
             while (type + 1 < sc.n_types && j >= s_tb[type + 1]) ++type;
-        scatter_particle(j < e, j, bx, by, bz, bh, sc.emit ? __uint_as_float((uint32_t)j) : record_code(type, bi),
+        scatter_particle(j < e, j, value_of(bx), value_of(by), value_of(bz), value_of(bh),
+                         sc.emit ? __uint_as_float((uint32_t)j) : record_code(type, value_of(bi)),
                          s_view, s_vbase, g_n, s_cur, nt, fr, lane);
         const int64_t ib = i + 3 * stride;
         if (ib < e)
-            bx = load1<S>(sc.x, ib), by = load1<S>(sc.y, ib), bz = load1<S>(sc.z, ib), bh = load1<S>(sc.h, ib),
-            bi = load1<S>(sc.it, ib);
+            bx = load_stored<S>(sc.x, ib), by = load_stored<S>(sc.y, ib), bz = load_stored<S>(sc.z, ib), bh = load_stored<S>(sc.h, ib),
+            bi = load_stored<S>(sc.it, ib);
     }
 }
 
@@ -710,7 +714,9 @@ template <int S> static cudaError_t scatter_impl(const SceneDev &sc, const Frame
 //      and the last moves the cursor past the run.
 // With the chunk bases in chunk order, every tile list is in ascending particle index
 // whatever the order in which CTAs and warps run, so images do not depend on it.  Renders ask
-// for it with SPLOTCH_STABLE.
+// for it with SPLOTCH_STABLE.  Bound by instruction issue and barriers; 20.7 M pairs of the
+// 10 M-particle frame in 1.35 ms (1.83 ms when one warp took the slots of all 32-pair slices in
+// turn), the scatter in arrival order 0.34 ms.
 
 constexpr int kStableStage = 4096;  // staged pairs per window
 constexpr int kSlotBits = 10;       // particle slot in a staged pair (kThreads of them), tile above
@@ -832,27 +838,27 @@ __global__ void __launch_bounds__(kThreads) k_scatter_stable(SceneDev sc, FrameD
     const int64_t e = min(sc.n, s + fr.chunk);
     int type = 0;
     int64_t i = s + tid;
-    float cx = 0.0f, cy = 0.0f, cz = 0.0f, ch = 0.0f, ci = 0.0f;
+    typename Stored<S>::T cx{}, cy{}, cz{}, ch{}, ci{};
     if (i < e)
-        cx = load1<S>(sc.x, i), cy = load1<S>(sc.y, i), cz = load1<S>(sc.z, i), ch = load1<S>(sc.h, i),
-        ci = load1<S>(sc.it, i);
+        cx = load_stored<S>(sc.x, i), cy = load_stored<S>(sc.y, i), cz = load_stored<S>(sc.z, i), ch = load_stored<S>(sc.h, i),
+        ci = load_stored<S>(sc.it, i);
     for (int64_t r0 = s; r0 < e; r0 += kThreads, i += kThreads) {
         const bool valid = i < e;
         // the next round's attributes load while this round is binned
-        float nx = 0.0f, ny = 0.0f, nz = 0.0f, nh = 0.0f, ni = 0.0f;
+        typename Stored<S>::T nx{}, ny{}, nz{}, nh{}, ni{};
         const int64_t in = i + kThreads;
         if (in < e)
-            nx = load1<S>(sc.x, in), ny = load1<S>(sc.y, in), nz = load1<S>(sc.z, in), nh = load1<S>(sc.h, in),
-            ni = load1<S>(sc.it, in);
+            nx = load_stored<S>(sc.x, in), ny = load_stored<S>(sc.y, in), nz = load_stored<S>(sc.z, in), nh = load_stored<S>(sc.h, in),
+            ni = load_stored<S>(sc.it, in);
         if (valid)
             while (type + 1 < sc.n_types && i >= s_tb[type + 1]) ++type;
-        const float code = sc.emit ? __uint_as_float((uint32_t)i) : record_code(type, ci);
+        const float code = sc.emit ? __uint_as_float((uint32_t)i) : record_code(type, value_of(ci));
         for (int g = 0; g < g_n; ++g) {
             const ViewParams &vp = s_view[g];
             Raster r;
             r.X = r.Y = r.R = 0.0f;
             int tx0 = 0, tx1 = -1, ty0 = 0, ty1 = -1;
-            if (valid && raster_one(vp, cx, cy, cz, ch, r)) {
+            if (valid && raster_one(vp, value_of(cx), value_of(cy), value_of(cz), value_of(ch), r)) {
                 tx0 = tile_of(vp, r.i0), tx1 = tile_of(vp, r.i1);
                 ty0 = tile_of(vp, r.j0), ty1 = tile_of(vp, r.j1);
             }

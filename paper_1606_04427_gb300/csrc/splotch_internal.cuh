@@ -129,6 +129,19 @@ template <> struct Store<2> {
     }
 };
 
+// One attribute of one particle as stored, and its value.  The particle-stream kernels keep
+// the stored form in registers while a load is in flight: a conversion beside the load would
+// wait for it at once.
+template <int S> struct Stored { typedef float T; };
+template <> struct Stored<1> { typedef __half T; };
+template <> struct Stored<2> { typedef __nv_bfloat16 T; };
+template <int S> __device__ __forceinline__ typename Stored<S>::T load_stored(const void *p, int64_t i) {
+    return __ldg(static_cast<const typename Stored<S>::T *>(p) + i);
+}
+__device__ __forceinline__ float value_of(float v) { return v; }
+__device__ __forceinline__ float value_of(__half v) { return __half2float(v); }
+__device__ __forceinline__ float value_of(__nv_bfloat16 v) { return __bfloat162float(v); }
+
 // One attribute of one particle (a warp reads 32 consecutive particles: coalesced).
 template <int S> __device__ __forceinline__ float load1(const void *p, int64_t i);
 template <> __device__ __forceinline__ float load1<0>(const void *p, int64_t i) {
