@@ -321,6 +321,11 @@ __global__ void __launch_bounds__(kThreads) k_count(SceneDev sc, FrameDev fr) {
     const int nt = fr.n_tiles;
     for (int k = threadIdx.x; k < g_n * nt; k += blockDim.x) s_hist[k] = 0;
     if (threadIdx.x < g_n) s_view[threadIdx.x] = fr.views[v0 + threadIdx.x];
+    // the frame's first kernel clears what the later ones count into
+    if (b == 0 && blockIdx.y == 0) {
+        for (int k = threadIdx.x; k < 2 * kOrderBins; k += blockDim.x) fr.bins[k] = 0;
+        if (threadIdx.x < 4) fr.status[threadIdx.x] = 0, fr.queue[threadIdx.x] = 0;
+    }
     __syncthreads();
 
     const int64_t s = (int64_t)b * fr.chunk;
@@ -371,8 +376,7 @@ cudaError_t launch_count(int storage, const SceneDev &sc, const FrameDev &fr, cu
 }
 
 // ---------------------------------------------------------------------------------------
-// k_scan: one CTA.  Tile segment offsets (int64), work items (a tile with more than K
-// pairs is split into ceil(count / K) items) and scratch slots of split tiles.
+// Scans of the tile counts.
 
 template <typename T> __device__ __forceinline__ T warp_incl_scan(T v) {
     const int lane = threadIdx.x & 31;
@@ -407,132 +411,185 @@ template <typename T> __device__ T block_excl_scan(T v, T *s_warp, T *total) {
 // k_chunk_scan: per (view, tile), the exclusive scan of the chunks' counts in chunk order
 // (rel becomes each chunk's base inside the tile segment) and the tile's total.  The
 // bases depend only on the counts, so the lists' layout is the same on every run.
+//
+// A CTA takes 32 tiles of a view (a lane each, so rows of rel are read 128 bytes at a time);
+// its kChunkSegs warps share the chunks, sum their parts, and write the bases in a second read.
+// Bound by the latency of the column walk: with one thread per tile it took 87 us on the 100 M
+// frame (582 chunks, 16384 tiles), now 15 us.
 
-constexpr int kChunkScanUnroll = 8;
+constexpr int kChunkScanUnroll = 8, kChunkSegs = 8;
 
-__global__ void __launch_bounds__(256) k_chunk_scan(FrameDev fr) {
-    const int nt = fr.n_tiles;
-    const int64_t N = (int64_t)fr.V * nt;
-    const int nch = fr.n_chunks;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        const int v = (int)(k / nt), t = (int)(k - (int64_t)v * nt);
-        int *col = fr.rel + (int64_t)v * nch * nt + t;
-        long long run = 0;
-        int b = 0;
-        for (; b + kChunkScanUnroll <= nch; b += kChunkScanUnroll) {
+__global__ void __launch_bounds__(32 * kChunkSegs) k_chunk_scan(FrameDev fr) {
+    __shared__ long long s_sum[kChunkSegs][32];
+    const int nt = fr.n_tiles, nch = fr.n_chunks;
+    const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+    const int per = (nch + kChunkSegs - 1) / kChunkSegs;
+    const int b0 = min(nch, seg * per), b1 = min(nch, b0 + per);
+    const int v = blockIdx.y, t = blockIdx.x * 32 + lane;
+    int *col = fr.rel + (int64_t)v * nch * nt + t;
+    long long sum = 0;
+    if (t < nt) {
+        int b = b0;
+        for (; b + kChunkScanUnroll <= b1; b += kChunkScanUnroll) {
             int c[kChunkScanUnroll];
 #pragma unroll
             for (int q = 0; q < kChunkScanUnroll; ++q) c[q] = col[(int64_t)(b + q) * nt];
 #pragma unroll
-            for (int q = 0; q < kChunkScanUnroll; ++q) {
-                col[(int64_t)(b + q) * nt] = (int)run;
-                run += c[q];
-            }
+            for (int q = 0; q < kChunkScanUnroll; ++q) sum += c[q];
         }
-        for (; b < nch; ++b) {
-            const int c = col[(int64_t)b * nt];
-            col[(int64_t)b * nt] = (int)run;
-            run += c;
+        for (; b < b1; ++b) sum += col[(int64_t)b * nt];
+    }
+    s_sum[seg][lane] = sum;
+    __syncthreads();
+    if (t >= nt) return;
+    long long run = 0, total = 0;
+#pragma unroll
+    for (int k = 0; k < kChunkSegs; ++k) {
+        if (k == seg) run = total;
+        total += s_sum[k][lane];
+    }
+    int b = b0;
+    for (; b + kChunkScanUnroll <= b1; b += kChunkScanUnroll) {
+        int c[kChunkScanUnroll];
+#pragma unroll
+        for (int q = 0; q < kChunkScanUnroll; ++q) c[q] = col[(int64_t)(b + q) * nt];
+#pragma unroll
+        for (int q = 0; q < kChunkScanUnroll; ++q) {
+            col[(int64_t)(b + q) * nt] = (int)run;
+            run += c[q];
         }
+    }
+    for (; b < b1; ++b) {
+        const int c = col[(int64_t)b * nt];
+        col[(int64_t)b * nt] = (int)run;
+        run += c;
+    }
+    if (seg == 0) {
         // a tile holding 2^31 pairs or more cannot be indexed by the 32-bit cursors
-        if (run > (long long)INT32_MAX) {
+        if (total > (long long)INT32_MAX) {
             atomicExch(&fr.status[kStatOverflow], 1);
-            run = INT32_MAX;
+            total = INT32_MAX;
         }
-        fr.counts[k] = (int)run;
+        fr.counts[(int64_t)v * nt + t] = (int)total;
     }
 }
 
-constexpr int kScanItems = 4;
+// ---------------------------------------------------------------------------------------
+// k_scan: tile segment offsets (int64), work items (a tile with more than K pairs is split
+// into ceil(count / K) items), scratch slots of split tiles, and the items' size histogram
+// for k_item_order.  A CTA scans kScanTiles tiles and sums the others itself (their counts are
+// in L2), so the CTAs need no order among them: 14 us for 16384 tiles and 22 us for 65536 (30 and
+// 113 us with one CTA for all).
 
-__global__ void __launch_bounds__(1024) k_scan(FrameDev fr, int target_items, int kmin) {
-    __shared__ long long s_l[33];
-    __shared__ int s_i[33];
-    __shared__ int s_j[33];
-    const int N = fr.V * fr.n_tiles;
-    // pass 1: total pairs and largest tile
-    long long sum = 0;
-    int mx = 0;
-    for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        const int c = fr.counts[k];
-        sum += c;
-        mx = max(mx, c);
-    }
-    long long tot;
-    block_excl_scan<long long>(sum, s_l, &tot);
-    int mx_all;
-    {
-        for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if ((threadIdx.x & 31) == 0) s_i[threadIdx.x >> 5] = mx;
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            int w = s_i[threadIdx.x];
-            for (int o = 16; o; o >>= 1) w = max(w, __shfl_xor_sync(0xffffffffu, w, o));
-            if (threadIdx.x == 0) s_i[32] = w;
-        }
-        __syncthreads();
-        mx_all = s_i[32];
-        __syncthreads();
-    }
-    long long K = (tot + target_items - 1) / (target_items > 0 ? target_items : 1);
-    if (K < kmin) K = kmin;
-    if (K > (1LL << 30)) K = (1LL << 30);
+constexpr int kScanItems = 4, kScanTiles = 1024 * kScanItems;
 
-    // pass 2: scans
-    long long run_p = 0;
-    int run_i = 0, run_s = 0;
-    for (int base = 0; base < N; base += blockDim.x * kScanItems) {
-        const int k0 = base + threadIdx.x * kScanItems;
-        int c[kScanItems], it[kScanItems], sp[kScanItems];
-        long long lp = 0;
-        int li = 0, ls = 0;
-#pragma unroll
-        for (int q = 0; q < kScanItems; ++q) {
-            const int k = k0 + q;
-            c[q] = k < N ? fr.counts[k] : 0;
-            it[q] = k < N ? max(1, (int)((c[q] + K - 1) / K)) : 0;
-            sp[q] = (k < N && c[q] > K) ? 1 : 0;
-            lp += c[q];
-            li += it[q];
-            ls += sp[q];
-        }
-        long long tp;
-        int ti, ts;
-        long long ep = block_excl_scan<long long>(lp, s_l, &tp) + run_p;
-        int ei = block_excl_scan<int>(li, s_i, &ti) + run_i;
-        int es = block_excl_scan<int>(ls, s_j, &ts) + run_s;
-#pragma unroll
-        for (int q = 0; q < kScanItems; ++q) {
-            const int k = k0 + q;
-            if (k < N) {
-                fr.offsets[k] = ep;
-                fr.item_off[k] = ei;
-                fr.split_slot[k] = sp[q] ? es : -1;
-            }
-            ep += c[q];
-            ei += it[q];
-            es += sp[q];
-        }
-        run_p += tp;
-        run_i += ti;
-        run_s += ts;
+// Sum of two values over a 1024-thread CTA, for every thread.
+__device__ __forceinline__ void block_sum2(long long &a, long long &b, long long (*s_w)[33]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int o = 16; o; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
     }
     __syncthreads();
-    // per-view segment sizes must fit the scatter's 32-bit cursors
+    if (lane == 0) s_w[0][warp] = a, s_w[1][warp] = b;
+    __syncthreads();
+    a = s_w[0][lane], b = s_w[1][lane];
+    for (int o = 16; o; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+}
+
+__global__ void __launch_bounds__(1024) k_scan(FrameDev fr, int target_items, int kmin) {
+    __shared__ long long s_w[2][33];
+    __shared__ int s_hist[kOrderBins];
+    const int N = fr.V * fr.n_tiles;
+    const int base = blockIdx.x * kScanTiles;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x < kOrderBins) s_hist[threadIdx.x] = 0;
+    // total pairs (counts is padded to a whole int4; entries past N are not added)
+    long long tot = 0, none = 0;
+#pragma unroll 4
+    for (int k = 4 * threadIdx.x; k < N; k += 4 * blockDim.x) {
+        const int4 c = *reinterpret_cast<const int4 *>(fr.counts + k);
+        tot += (long long)c.x + (k + 1 < N ? c.y : 0) + (k + 2 < N ? c.z : 0) + (k + 3 < N ? c.w : 0);
+    }
+    block_sum2(tot, none, s_w);
+    long long K64 = (tot + target_items - 1) / (target_items > 0 ? target_items : 1);
+    if (K64 < kmin) K64 = kmin;
+    if (K64 > (1LL << 30)) K64 = (1LL << 30);
+    const int K = (int)K64;
+    auto items_of = [&](int c) -> int { return c <= K ? 1 : (int)(((uint32_t)c + (uint32_t)K - 1u) / (uint32_t)K); };
+
+    // pairs, and items and split tiles (two 32-bit halves), before this CTA's tiles
+    long long pre_p = 0, pre_is = 0;
+#pragma unroll 4
+    for (int k = 4 * threadIdx.x; k < base; k += 4 * blockDim.x) {
+        const int4 c = *reinterpret_cast<const int4 *>(fr.counts + k);
+        pre_p += (long long)c.x + c.y + c.z + c.w;
+        pre_is += ((long long)(items_of(c.x) + items_of(c.y) + items_of(c.z) + items_of(c.w)) << 32) +
+                  (c.x > K) + (c.y > K) + (c.z > K) + (c.w > K);
+    }
+    if (base > 0) block_sum2(pre_p, pre_is, s_w);
+
+    const int k0 = base + threadIdx.x * kScanItems;
+    int c[kScanItems], it[kScanItems];
+    long long lp = 0, lis = 0;
+#pragma unroll
+    for (int q = 0; q < kScanItems; ++q) {
+        const bool in = k0 + q < N;
+        c[q] = in ? fr.counts[k0 + q] : 0;
+        it[q] = in ? items_of(c[q]) : 0;
+        lp += c[q];
+        lis += ((long long)it[q] << 32) + (c[q] > K);
+        // the tile's last slice, counted once per warp and bin, and its full ones
+        const int bin = in ? order_bin(c[q] - K * (it[q] - 1), K) : kOrderBins;
+        const uint32_t peers = warp_peers<7>((uint32_t)bin);
+        if (in && lane == __ffs(peers) - 1) atomicAdd(&s_hist[bin], __popc(peers));
+        if (it[q] > 1) atomicAdd(&s_hist[order_bin(K, K)], it[q] - 1);
+    }
+    // exclusive scan of both over the CTA
+    const long long wp = warp_incl_scan(lp), wis = warp_incl_scan(lis);
+    __syncthreads();
+    if (lane == 31) s_w[0][warp] = wp, s_w[1][warp] = wis;
+    __syncthreads();
+    const long long p_w = s_w[0][lane], is_w = s_w[1][lane];
+    const long long p_i = warp_incl_scan(p_w), is_i = warp_incl_scan(is_w);
+    const long long tp = __shfl_sync(0xffffffffu, p_i, 31), tis = __shfl_sync(0xffffffffu, is_i, 31);
+    long long ep = pre_p + wp - lp + __shfl_sync(0xffffffffu, p_i - p_w, warp);
+    long long eis = pre_is + wis - lis + __shfl_sync(0xffffffffu, is_i - is_w, warp);
+#pragma unroll
+    for (int q = 0; q < kScanItems; ++q) {
+        const int k = k0 + q;
+        if (k < N) {
+            fr.offsets[k] = ep;
+            fr.item_off[k] = (int)(eis >> 32);
+            fr.split_slot[k] = c[q] > K ? (int)(eis & 0xffffffffll) : -1;
+        }
+        ep += c[q];
+        eis += ((long long)it[q] << 32) + (c[q] > K);
+    }
+    if (threadIdx.x < kOrderBins && s_hist[threadIdx.x]) atomicAdd(&fr.bins[threadIdx.x], s_hist[threadIdx.x]);
+    if (blockIdx.x != gridDim.x - 1) return;
+    // the scatter's cursors are 32-bit within a view
     int big = 0;
-    for (int v = threadIdx.x; v < fr.V; v += blockDim.x)
-        big |= (fr.offsets[(int64_t)v * fr.n_tiles + fr.n_tiles - 1] + fr.counts[(int64_t)v * fr.n_tiles + fr.n_tiles - 1] -
-                fr.offsets[(int64_t)v * fr.n_tiles]) > (long long)INT32_MAX;
+    if (tot > (long long)INT32_MAX)
+        for (int v = threadIdx.x; v < fr.V; v += blockDim.x) {
+            long long sum = 0;
+            for (int t = 0; t < fr.n_tiles; ++t) sum += fr.counts[(int64_t)v * fr.n_tiles + t];
+            big |= sum > (long long)INT32_MAX;
+        }
     big = __syncthreads_or(big);
     if (threadIdx.x == 0) {
-        fr.offsets[N] = run_p;
-        fr.item_off[N] = run_i;
-        fr.sizes[kSizePairs] = run_p;
-        fr.sizes[kSizeItems] = run_i;
-        fr.sizes[kSizeSplits] = run_s;
+        const long long is = pre_is + tis;
+        const int items = (int)(is >> 32), splits = (int)(is & 0xffffffffll);
+        fr.offsets[N] = tot;
+        fr.item_off[N] = items;
+        fr.sizes[kSizePairs] = tot;
+        fr.sizes[kSizeItems] = items;
+        fr.sizes[kSizeSplits] = splits;
         fr.sizes[kSizeK] = K;
-        fr.sizes[kSizeMaxCount] = mx_all;
-        const bool over = run_p > fr.pair_cap || run_i > fr.item_cap || run_s > fr.split_cap || big ||
+        const bool over = tot > fr.pair_cap || items > fr.item_cap || splits > fr.split_cap || big ||
                           fr.status[kStatOverflow];
         fr.status[kStatOverflow] = over ? 1 : 0;
     }
@@ -540,9 +597,14 @@ __global__ void __launch_bounds__(1024) k_scan(FrameDev fr, int target_items, in
 
 cudaError_t launch_scan(const FrameDev &fr, int target_items, int kmin, cudaStream_t st) {
     const int64_t N = (int64_t)fr.V * fr.n_tiles;
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((N + 255) / 256, 8192));
-    k_chunk_scan<<<blocks, 256, 0, st>>>(fr);
-    k_scan<<<1, 1024, 0, st>>>(fr, target_items, kmin);
+    for (int v0 = 0; v0 < fr.V; v0 += 65535) {  // the grid's second dimension holds 65535 views
+        FrameDev part = fr;
+        part.V = std::min(65535, fr.V - v0);
+        part.rel = fr.rel + (int64_t)v0 * fr.n_chunks * fr.n_tiles;
+        part.counts = fr.counts + (int64_t)v0 * fr.n_tiles;
+        k_chunk_scan<<<dim3((fr.n_tiles + 31) / 32, part.V), 32 * kChunkSegs, 0, st>>>(part);
+    }
+    k_scan<<<(int)((N + kScanTiles - 1) / kScanTiles), 1024, 0, st>>>(fr, target_items, kmin);
     return cudaGetLastError();
 }
 

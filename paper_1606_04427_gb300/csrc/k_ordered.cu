@@ -395,13 +395,13 @@ cudaError_t launch_compose_maps(const float *maps, int n, int64_t pixels, float 
     return cudaGetLastError();
 }
 
-cudaError_t launch_splat_ordered(const SceneDev &sc, const FrameDev &fr, int *queue, float *out,
-                                 const float *absorb, float *ord_scratch, int map_out, int grid, cudaStream_t st) {
+cudaError_t launch_splat_ordered(const SceneDev &sc, const FrameDev &fr, float *out, const float *absorb,
+                                 float *ord_scratch, int map_out, int grid, cudaStream_t st) {
     auto fn = sc.emit ? k_splat_ordered<true> : k_splat_ordered<false>;
     cudaError_t err = ensure_smem_limit((const void *)fn, ordered_smem());
     if (err != cudaSuccess) return err;
     if ((err = launch_item_order(fr, st)) != cudaSuccess) return err;
-    fn<<<grid, kOWarps * 32, ordered_smem(), st>>>(sc, fr, queue, out, ordered_split(fr.T), absorb, ord_scratch, map_out);
+    fn<<<grid, kOWarps * 32, ordered_smem(), st>>>(sc, fr, fr.queue, out, ordered_split(fr.T), absorb, ord_scratch, map_out);
     return cudaGetLastError();
 }
 

@@ -363,68 +363,73 @@ int splat_blocks_per_sm() {
 
 int splat_workers_per_sm() { return splat_blocks_per_sm() * kWarpsPerCta; }
 
-// k_item_order: one CTA.  The splat's work items (tile-list slices) ordered by record count,
-// largest first, so that the items taken last by the workers are the short ones and the
-// kernel does not end waiting for a few long slices started late.  Slices fall into
-// kOrderBins bins of equal width up to K (the slice length of a split tile); within a bin
-// the order is that of the atomic cursors.  Each item writes its own tile, or adds into
-// the exact accumulators of a split tile, so images do not depend on the order.
-constexpr int kOrderBins = 64;
-
+// k_item_order: the splat's work items (tile-list slices) ordered by record count, largest
+// first, so that the items taken last by the workers are the short ones and the kernel does
+// not end waiting for a few long slices started late.  Slices fall into kOrderBins bins of
+// equal width up to K (the slice length of a split tile), whose sizes k_scan has counted;
+// within a bin the order is that of the atomic cursors.  Each item writes its own tile, or adds
+// into the exact accumulators of a split tile, so images do not depend on the order.  One tile
+// per thread: 8 us for 16384 tiles and 5 us for 65536 that are hardly split (33 and 84 us with
+// one CTA for all).
 __global__ void __launch_bounds__(1024) k_item_order(FrameDev fr) {
-    __shared__ int s_cnt[kOrderBins];
+    __shared__ int s_cnt[kOrderBins], s_all[kOrderBins], s_pos[kOrderBins];
     if (fr.status[kStatOverflow]) return;
-    const int N = fr.V * fr.n_tiles;
-    const long long K = fr.sizes[kSizeK];
-    auto bin_of = [&](long long size) -> int {
-        return (int)min((long long)(kOrderBins - 1), size * kOrderBins / (K + 1));
-    };
-    for (int b = threadIdx.x; b < kOrderBins; b += blockDim.x) s_cnt[b] = 0;
+    const int N = fr.V * fr.n_tiles, lane = threadIdx.x & 31;
+    const int K = (int)fr.sizes[kSizeK];
+    if (threadIdx.x < kOrderBins) s_cnt[threadIdx.x] = 0, s_all[threadIdx.x] = fr.bins[threadIdx.x];
     __syncthreads();
-    // (1) slices per size bin: every slice of a split tile holds K records but the last
-    for (int t = threadIdx.x; t < N; t += blockDim.x) {
-        const int i0 = fr.item_off[t], n = fr.item_off[t + 1] - i0;
-        const long long c = fr.counts[t];
-        if (n > 1) atomicAdd(&s_cnt[bin_of(K)], n - 1);
-        atomicAdd(&s_cnt[bin_of(c - K * (n - 1))], 1);
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    // every slice of a split tile holds K records but the last; tiles of a warp whose last slices
+    // share a bin are counted and placed together
+    int n = 0, last_bin = kOrderBins;
+    if (t < N) {
+        n = fr.item_off[t + 1] - fr.item_off[t];
+        last_bin = order_bin(fr.counts[t] - K * (n - 1), K);
+    }
+    const uint32_t peers = warp_peers<7>((uint32_t)last_bin);
+    const int leader = __ffs(peers) - 1;
+    if (t < N && lane == leader) atomicAdd(&s_cnt[last_bin], __popc(peers));
+    if (n > 1) atomicAdd(&s_cnt[order_bin(K, K)], n - 1);
+    __syncthreads();
+    // this CTA's place in each bin: the bins before it (the largest first), then the CTAs that
+    // came earlier
+    if (threadIdx.x < kOrderBins) {
+        int start = 0;
+        for (int b = kOrderBins - 1; b > (int)threadIdx.x; --b) start += s_all[b];
+        const int c = s_cnt[threadIdx.x];
+        s_pos[threadIdx.x] = start + (c ? atomicAdd(&fr.bins[kOrderBins + threadIdx.x], c) : 0);
     }
     __syncthreads();
-    // (2) bin starts, the largest bin first
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int b = kOrderBins - 1; b >= 0; --b) {
-            const int c = s_cnt[b];
-            s_cnt[b] = run;
-            run += c;
-        }
-    }
-    __syncthreads();
-    // (3) every slice at its bin's next place
-    for (int t = threadIdx.x; t < N; t += blockDim.x) {
-        const int i0 = fr.item_off[t], n = fr.item_off[t + 1] - i0;
-        const long long c = fr.counts[t];
-        if (n > 1) {
-            const int p = atomicAdd(&s_cnt[bin_of(K)], n - 1);
-            for (int s = 0; s < n - 1; ++s) fr.order[p + s] = make_int2(t, s);
-        }
-        fr.order[atomicAdd(&s_cnt[bin_of(c - K * (n - 1))], 1)] = make_int2(t, n - 1);
+    int at = 0;
+    if (t < N && lane == leader) at = atomicAdd(&s_pos[last_bin], __popc(peers));
+    at = __shfl_sync(0xffffffffu, at, leader) + __popc(peers & ((1u << lane) - 1u));
+    if (t < N) fr.order[at] = make_int2(t, n - 1);
+    // the full slices of a split tile, by its warp
+    for (uint32_t todo = __ballot_sync(0xffffffffu, n > 1); todo; todo &= todo - 1) {
+        const int src = __ffs(todo) - 1;
+        const int m = __shfl_sync(0xffffffffu, n, src) - 1, tt = __shfl_sync(0xffffffffu, t, src);
+        int p = 0;
+        if (lane == 0) p = atomicAdd(&s_pos[order_bin(K, K)], m);
+        p = __shfl_sync(0xffffffffu, p, 0);
+        for (int k = lane; k < m; k += 32) fr.order[p + k] = make_int2(tt, k);
     }
 }
 
 cudaError_t launch_item_order(const FrameDev &fr, cudaStream_t st) {
     if (!fr.order) return cudaSuccess;
-    k_item_order<<<1, 1024, 0, st>>>(fr);
+    const int64_t N = (int64_t)fr.V * fr.n_tiles;
+    k_item_order<<<(int)((N + 1023) / 1024), 1024, 0, st>>>(fr);
     return cudaGetLastError();
 }
 
-cudaError_t launch_splat(const SceneDev &sc, const FrameDev &fr, int *queue, float *out, int out_accum,
-                         int grid, cudaStream_t st) {
+cudaError_t launch_splat(const SceneDev &sc, const FrameDev &fr, float *out, int out_accum, int grid,
+                         cudaStream_t st) {
     cudaError_t e = launch_item_order(fr, st);
     if (e != cudaSuccess) return e;
     const SplatFn fn = splat_fn(fr.vscale != nullptr, sc.emit != nullptr);
     e = ensure_smem_limit((const void *)fn, splat_smem());
     if (e != cudaSuccess) return e;
-    fn<<<grid, kWarpsPerCta * 32, splat_smem(), st>>>(sc, fr, queue, out, out_accum, splat_split(fr.T));
+    fn<<<grid, kWarpsPerCta * 32, splat_smem(), st>>>(sc, fr, fr.queue, out, out_accum, splat_split(fr.T));
     return cudaGetLastError();
 }
 

@@ -665,7 +665,7 @@ struct FrameHost {
     int64_t chunk = 0;
     int storage = 0;
     // fixed part
-    size_t o_views, o_counts, o_rel, o_offsets, o_item, o_split, o_sizes, o_status, o_queue, fixed_bytes;
+    size_t o_views, o_counts, o_rel, o_offsets, o_item, o_split, o_sizes, o_status, o_queue, o_bins, fixed_bytes;
     // variable part (capacities)
     int64_t pair_cap = 0;
     int item_cap = 0, split_cap = 0;
@@ -683,7 +683,7 @@ static void layout_fixed(FrameHost &fh, const splotch_scene *sc, int V, int n_ti
     fh.T = T;
     fh.n_tiles = n_tiles;
     fh.storage = sc->storage;
-    fh.G = std::max(1, std::min({V, kMaxGroup, kMaxTiles / std::max(1, n_tiles)}));
+    fh.G = std::max(1, std::min({V, kMaxGroup, kGroupTiles / std::max(1, n_tiles)}));
     const int n_sm = sm_count(sc->dev);
     const int vec = sc->storage == 0 ? 4 : 8;
     const int64_t unit = (int64_t)kThreads * vec;
@@ -721,6 +721,7 @@ static void layout_fixed(FrameHost &fh, const splotch_scene *sc, int V, int n_ti
     fh.o_sizes = cv.take(sizeof(int64_t) * 8);
     fh.o_status = cv.take(sizeof(int) * 4);
     fh.o_queue = cv.take(sizeof(int) * 4);
+    fh.o_bins = cv.take(sizeof(int) * 2 * kOrderBins);
     fh.fixed_bytes = cv.off;
 }
 
@@ -760,6 +761,8 @@ static FrameDev frame_dev(const FrameHost &fh, char *fixed, char *var) {
     fr.split_slot = (int *)(fixed + fh.o_split);
     fr.sizes = (int64_t *)(fixed + fh.o_sizes);
     fr.status = (int *)(fixed + fh.o_status);
+    fr.queue = (int *)(fixed + fh.o_queue);
+    fr.bins = (int *)(fixed + fh.o_bins);
     if (var) {
         fr.lists = (float4 *)(var + fh.o_lists);
         fr.pids = fh.pids ? (int *)(var + fh.o_pids) : nullptr;
@@ -771,6 +774,12 @@ static FrameDev frame_dev(const FrameHost &fh, char *fixed, char *var) {
     fr.item_cap = var ? fh.item_cap : INT32_MAX;
     fr.split_cap = var ? fh.split_cap : INT32_MAX;
     return fr;
+}
+
+// Accumulators and tickets of the frame's split tiles.
+static cudaError_t clear_split_scratch(const FrameHost &fh, char *var, int splits, cudaStream_t st) {
+    if (splits <= 0) return cudaSuccess;
+    return cudaMemsetAsync(var + fh.o_scratch, 0, fh.o_tickets - fh.o_scratch + sizeof(int) * (size_t)splits, st);
 }
 
 // items: work items of the scan (tile-list slices); the splat renders each as split^2
@@ -827,8 +836,6 @@ static splotch_status count_and_size(splotch_scene *sc, const RenderSetup &rs, F
     FrameDev fr = frame_dev(fh, fixed, nullptr);
     CUDA_TRY(cudaMemcpyAsync(fixed + fh.o_views, rs.views.data(), sizeof(ViewParams) * rs.V,
                              cudaMemcpyHostToDevice, st));
-    CUDA_TRY(cudaMemsetAsync(fixed + fh.o_counts, 0, sizeof(int) * (size_t)rs.V * fh.n_tiles, st));
-    CUDA_TRY(cudaMemsetAsync(fixed + fh.o_status, 0, sizeof(int) * 4, st));
     if (ev) CUDA_TRY(cudaEventRecord(ev[0], st));
     CUDA_TRY(launch_count(sc->storage, sc->dev_view, fr, st));
     if (ev) CUDA_TRY(cudaEventRecord(ev[1], st));
@@ -847,11 +854,10 @@ static splotch_status scatter_and_splat(splotch_scene *sc, FrameHost &fh, char *
                                         int out_accum, bool stable, int items, cudaStream_t st,
                                         cudaEvent_t *ev = nullptr) {
     FrameDev fr = frame_dev(fh, fixed, var);
-    CUDA_TRY(cudaMemsetAsync(fixed + fh.o_queue, 0, sizeof(int) * 4, st));
     if (ev) CUDA_TRY(cudaEventRecord(ev[3], st));
     CUDA_TRY(launch_scatter(sc->storage, sc->dev_view, fr, stable, st));
     if (ev) CUDA_TRY(cudaEventRecord(ev[4], st));
-    CUDA_TRY(launch_splat(sc->dev_view, fr, (int *)(fixed + fh.o_queue), out, out_accum,
+    CUDA_TRY(launch_splat(sc->dev_view, fr, out, out_accum,
                           splat_grid(sc->dev, fh.T, items), st));
     if (ev) CUDA_TRY(cudaEventRecord(ev[5], st));
     return SPLOTCH_OK;
@@ -894,8 +900,7 @@ static splotch_status render_frame(splotch_scene *sc, const RenderSetup &rs, flo
     }
     s = SPLOTCH_OK;
     do {
-        if (cudaMemsetAsync(var + fh.o_scratch, 0, fh.o_tickets - fh.o_scratch + sizeof(int) * std::max(1, splits),
-                            st) != cudaSuccess) {
+        if (clear_split_scratch(fh, var, splits, st) != cudaSuccess) {
             s = fail(SPLOTCH_ERR_CUDA, "memset scratch");
             break;
         }
@@ -1078,8 +1083,7 @@ static splotch_status frame_scatter(splotch_frame *f, cudaStream_t st) {
     if (s != SPLOTCH_OK) return s;
     f->var = (char *)f->sc->mem.alloc(f->fh.var_bytes, st);
     if (!f->var) return fail(SPLOTCH_ERR_OOM, "tile lists (%zu bytes)", f->fh.var_bytes);
-    CUDA_TRY(cudaMemsetAsync(f->var + f->fh.o_scratch, 0, f->fh.var_bytes - f->fh.o_scratch, st));
-    CUDA_TRY(cudaMemsetAsync(f->fixed + f->fh.o_queue, 0, sizeof(int) * 4, st));
+    CUDA_TRY(clear_split_scratch(f->fh, f->var, (int)f->sizes[kSizeSplits], st));
     CUDA_TRY(launch_scatter(f->sc->storage, f->sc->dev_view, frame_dev(f->fh, f->fixed, f->var),
                             (f->rs.pr.flags & SPLOTCH_STABLE) != 0, st));
     return SPLOTCH_OK;
@@ -1089,9 +1093,8 @@ static splotch_status frame_scatter(splotch_frame *f, cudaStream_t st) {
 static splotch_status frame_splat(splotch_frame *f, float *out, cudaStream_t st) {
     splotch_status s = frame_follow(f, st);
     if (s != SPLOTCH_OK) return s;
-    CUDA_TRY(launch_splat(f->sc->dev_view, frame_dev(f->fh, f->fixed, f->var), (int *)(f->fixed + f->fh.o_queue),
-                          out, out_mode(f->rs.pr.flags), splat_grid(f->sc->dev, f->fh.T, (int)f->sizes[kSizeItems]),
-                          st));
+    CUDA_TRY(launch_splat(f->sc->dev_view, frame_dev(f->fh, f->fixed, f->var), out, out_mode(f->rs.pr.flags),
+                          splat_grid(f->sc->dev, f->fh.T, (int)f->sizes[kSizeItems]), st));
     return SPLOTCH_OK;
 }
 
@@ -1150,13 +1153,10 @@ static splotch_status plan_enqueue(splotch_plan *pl, float *out, cudaStream_t st
     fr.vlut = pl->vlut;
     fr.vlut_off = pl->vlut_tab;
     fr.vlut_len = pl->vlut_tab + nvt;
-    CUDA_TRY(cudaMemsetAsync(pl->fixed + fh.o_counts, 0, sizeof(int) * (size_t)fh.V * fh.n_tiles, st));
-    CUDA_TRY(cudaMemsetAsync(pl->fixed + fh.o_status, 0, sizeof(int) * 4, st));
-    CUDA_TRY(cudaMemsetAsync(pl->fixed + fh.o_queue, 0, sizeof(int) * 4, st));
     CUDA_TRY(launch_count(sc->storage, sc->dev_view, fr, st));
     CUDA_TRY(launch_scan(fr, target_items(sc->dev, fh.T), kMinItemPairs, st));
     CUDA_TRY(launch_scatter(sc->storage, sc->dev_view, fr, (pl->rs.pr.flags & SPLOTCH_STABLE) != 0, st));
-    CUDA_TRY(launch_splat(sc->dev_view, fr, (int *)(pl->fixed + fh.o_queue), out,
+    CUDA_TRY(launch_splat(sc->dev_view, fr, out,
                           out_mode(pl->rs.pr.flags), pl->grid, st));
     CUDA_TRY(cudaMemcpyAsync(pl->box, pl->fixed + fh.o_sizes, sizeof(int64_t) * 8, cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaMemcpyAsync(pl->box + 8, pl->fixed + fh.o_status, sizeof(int) * 4, cudaMemcpyDeviceToHost, st));
@@ -1530,14 +1530,11 @@ extern "C" splotch_status splotch_render_noalloc(splotch_scene *sc, const splotc
     // every call shares the array: zero what the kernels count into before they start
     cudaStream_t st = (cudaStream_t)stream;
     CUDA_TRY(cudaMemcpyAsync(base + fh.o_views, &vp, sizeof(ViewParams), cudaMemcpyHostToDevice, st));
-    CUDA_TRY(cudaMemsetAsync(base + fh.o_counts, 0, sizeof(int) * (size_t)vp.n_tiles, st));
-    CUDA_TRY(cudaMemsetAsync(base + fh.o_status, 0, sizeof(int) * 4, st));
-    CUDA_TRY(cudaMemsetAsync(base + fh.o_queue, 0, sizeof(int) * 4, st));
     CUDA_TRY(cudaMemsetAsync(var + fh.o_scratch, 0, fh.var_bytes - fh.o_scratch, st));
     CUDA_TRY(launch_count(sc->storage, sc->dev_view, fr, st));
     CUDA_TRY(launch_scan(fr, target_items(sc->dev, T), kMinItemPairs, st));
     CUDA_TRY(launch_scatter(sc->storage, sc->dev_view, fr, (pr.flags & SPLOTCH_STABLE) != 0, st));
-    CUDA_TRY(launch_splat(sc->dev_view, fr, (int *)(base + fh.o_queue), out,
+    CUDA_TRY(launch_splat(sc->dev_view, fr, out,
                           out_mode(pr.flags), sm_count(dev) * std::max(1, splat_blocks_per_sm()), st));
     int64_t sizes[8];
     int stat[4];
@@ -1822,8 +1819,8 @@ extern "C" splotch_status splotch_render_ordered(splotch_scene *sc, const splotc
         sc->mem.release(fixed, st);
         return fail(SPLOTCH_ERR_OOM, "ordered render workspace (%zu + %zu bytes)", fh.var_bytes, cv.off);
     }
-    cudaError_t e = cudaMemsetAsync(var + fh.o_scratch, 0, fh.var_bytes - fh.o_scratch, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(fixed + fh.o_queue, 0, sizeof(int) * 4, st);
+    // the tickets of split tiles (their slices store maps, not sums)
+    cudaError_t e = splits ? cudaMemsetAsync(var + fh.o_tickets, 0, sizeof(int) * (size_t)splits, st) : cudaSuccess;
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(ex + o_abs, absorb, sizeof(float) * sc->n_types, cudaMemcpyHostToDevice, st);
     FrameDev fr = frame_dev(fh, fixed, var);
@@ -1872,7 +1869,7 @@ extern "C" splotch_status splotch_render_ordered(splotch_scene *sc, const splotc
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count(sc->dev) * ordered_ctas_per_sm(),
                                                                 (squares + per_cta - 1) / per_cta));
     if (e == cudaSuccess)
-        e = launch_splat_ordered(sc->dev_view, fr, (int *)(fixed + fh.o_queue), out, (const float *)(ex + o_abs),
+        e = launch_splat_ordered(sc->dev_view, fr, out, (const float *)(ex + o_abs),
                                  (float *)(ex + o_map), (rs.pr.flags & SPLOTCH_OUT_MAP) ? 1 : 0, grid, st);
     int stat[4] = {0, 0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(stat, fixed + fh.o_status, sizeof(stat), cudaMemcpyDeviceToHost, st);

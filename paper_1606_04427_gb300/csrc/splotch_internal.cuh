@@ -20,7 +20,13 @@ constexpr int kMaxTiles = 16384;   // tiles per image (per-CTA shared histogram)
 constexpr int kMaxTile = 64;       // tile edge in pixels
 constexpr int kMaxTypes = 255;     // species (8-bit type field in the tile records)
 constexpr int kThreads = 1024;     // CTA size of the particle-stream kernels (one per SM: one tile histogram per SM)
-constexpr int kMaxGroup = 16;      // views per CTA in the particle-stream kernels
+// Views per CTA in the particle-stream kernels: at most kMaxGroup, and as many as keep the
+// tile counters of a CTA within kGroupTiles.  More views share the attribute loads, but the
+// scatter then writes more list fronts at once than stay in L2 until their sectors are full
+// (16 views of 1024^2, 20 M particles: 23.1 ms with 4 views per CTA, 22.4 with 2, 22.0 with 1),
+// and fewer CTAs run (64 views of 300 tiles, 300 k particles: 1.10 ms with 16, 1.05 with 4,
+// 1.13 with 1).
+constexpr int kMaxGroup = 4, kGroupTiles = 4096;
 constexpr uint32_t kCodeMax = 16777215u;   // 24-bit normalised-intensity code
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -65,13 +71,15 @@ struct FrameDev {
     int T;                    // tile edge (all views)
     int64_t chunk;            // particles per particle-stream CTA
     int n_chunks;
-    int *counts;              // [V * n_tiles]
+    int *counts;              // [V * n_tiles], 16-byte aligned and padded to whole int4s
     int *rel;                 // [V * n_chunks * n_tiles] chunk base inside the tile segment
     int64_t *offsets;         // [V * n_tiles + 1] tile segment starts in `lists`
     int *item_off;            // [V * n_tiles + 1] first work item of each tile
     int *split_slot;          // [V * n_tiles] scratch slot of tiles split over items, else -1
-    int64_t *sizes;           // [8] pairs, items, splits, K, max tile count
-    int *status;              // [4] 0: capacity overflow, 1: timeout, 2: work queue
+    int64_t *sizes;           // [8] pairs, items, splits, K
+    int *status;              // [4] 0: capacity overflow, 1: timeout
+    int *bins;                // [2 * kOrderBins] work items per size bin, and k_item_order's cursors
+    int *queue;               // [4] the splat's work queue
     float4 *lists;            // [pair capacity] tile records (X, Y, R, code)
     int *pids;                // [pair capacity] particle index per record, or null
     unsigned long long *scratch;  // [split capacity][3][T][T][2] exact accumulators (fix_add)
@@ -87,8 +95,14 @@ struct FrameDev {
     const int *vlut_off, *vlut_len;
 };
 
-enum { kSizePairs = 0, kSizeItems = 1, kSizeSplits = 2, kSizeK = 3, kSizeMaxCount = 4 };
-enum { kStatOverflow = 0, kStatTimeout = 1, kStatQueue = 2 };
+enum { kSizePairs = 0, kSizeItems = 1, kSizeSplits = 2, kSizeK = 3 };
+enum { kStatOverflow = 0, kStatTimeout = 1 };
+
+// Size bin of a work item of `size` <= K records, for the splat's largest-first order.
+constexpr int kOrderBins = 64;
+__device__ __forceinline__ int order_bin(int size, int K) {
+    return min(kOrderBins - 1, (int)(__fdividef((float)size, (float)K) * (float)kOrderBins));
+}
 
 // ------------------------------------------------------------------------------------
 // Storage loaders: VEC consecutive particles with one 16-byte load per attribute.
@@ -394,8 +408,8 @@ cudaError_t launch_scan(const FrameDev &fr, int target_items, int kmin, cudaStre
 // stable: every tile list in ascending particle index (k_scatter_stable); else each
 // chunk's members in arrival order (k_scatter)
 cudaError_t launch_scatter(int storage, const SceneDev &sc, const FrameDev &fr, bool stable, cudaStream_t st);
-cudaError_t launch_splat(const SceneDev &sc, const FrameDev &fr, int *queue, float *out,
-                         int out_accum, int grid, cudaStream_t st);
+cudaError_t launch_splat(const SceneDev &sc, const FrameDev &fr, float *out, int out_accum, int grid,
+                         cudaStream_t st);
 int splat_blocks_per_sm();
 int splat_workers_per_sm();
 int splat_split(int T);  // regions of up to 16 px per tile edge, which the splat renders separately
@@ -445,8 +459,8 @@ int ordered_workers_per_sm();
 // Work items of the frame ordered largest first into fr.order (k_item_order; no-op when
 // fr.order is null).
 cudaError_t launch_item_order(const FrameDev &fr, cudaStream_t st);
-cudaError_t launch_splat_ordered(const SceneDev &sc, const FrameDev &fr, int *queue, float *out,
-                                 const float *absorb, float *ord_scratch, int map_out, int grid, cudaStream_t st);
+cudaError_t launch_splat_ordered(const SceneDev &sc, const FrameDev &fr, float *out, const float *absorb,
+                                 float *ord_scratch, int map_out, int grid, cudaStream_t st);
 cudaError_t launch_selftest_wait(long long limit, int *result, cudaStream_t st);
 cudaError_t launch_final(float *a, int64_t count, cudaStream_t st);
 cudaError_t launch_compose_maps(const float *maps, int n, int64_t pixels, float *out, cudaStream_t st);
