@@ -9,7 +9,12 @@
 // up to 16 x 16 pixels (a tile, or one of the split x split regions of a tile above 16 px)
 // and a tile list, or a K-record slice of a crowded tile's list; slices of a split tile add
 // their partial sums into an exact scratch tile and the last one to finish writes the
-// result.  Warps never wait on one another.
+// result.  In frames of few records teams of 2, 4 or 8 warps of a CTA take the long items
+// together (team_of): each warp renders a consecutive part of the list and the parts' sums are
+// added in order, so a frame of 256 tiles occupies 2048 warps instead of 256.  The items come
+// longest first; at the first short one a team parts and its warps go on alone.  (Without that
+// order the short items are the team's first warp's, so which warps add what depends on the
+// items alone.)  Teams never wait on one another.
 //
 // What a warp does with an item.  The kernel is bound by instruction issue and the latency
 // between its phases (the records are read once, DRAM is nearly idle), so the layout is
@@ -34,9 +39,9 @@
 // pixels in 6.7 such squares (107 lane evaluations, against 142 in 8 x 4 blocks with a warp per
 // record), a step of the pass loop serves 16 records instead of one, and the small records,
 // most of a list, no longer cost a whole warp each.  The 10 M-particle frame at 2048^2 takes
-// 500 M warp instructions (792 M with a warp per record), the 100 M-particle frame 5.75 ms
-// (7.35), 10 M close particles at 4096^2 4.5 ms (5.2), 1 M at 637 x 483 119 us (195), 100 k at
-// 256^2 48 us (107).  Batches of 192: 128 balance worse (6.2 ms), 224 leave 14 warps per SM
+// 500 M warp instructions (792 M with a warp per record), the 100 M-particle frame 5.5 ms
+// (7.35), 10 M close particles at 4096^2 4.4 ms (5.1), 1 M at 637 x 483 67 us (196), 100 k at
+// 256^2 21 us (107).  Batches of 192: 128 balance worse (6.2 ms), 224 leave 14 warps per SM
 // instead of 16 (6.7 ms); scalar instead of packed arithmetic: 18 more instructions per step
 // (6.5 ms against 6.1 before the loop was unrolled); unrolling by 3 drops the copies of the
 // prefetched record (6.1 -> 5.75 ms).
@@ -53,53 +58,310 @@ __device__ __forceinline__ int find_tile(const int *__restrict__ item_off, int N
     return a;
 }
 
-// Output of a pixel's accumulation a: mode 0 writes 1 - exp(-a) (final transform),
-// 1 writes a, 2 adds a to what the pixel holds (several renders summed in one image).
-__device__ __forceinline__ void put_pixel(float *p, float a, int mode) {
-    *p = mode == 2 ? *p + a : (mode ? a : -expm1f(-a));
+// Output of a pixel's accumulation a: mode 0 gives 1 - exp(-a) (final transform), 1 gives a,
+// 2 adds a to what the pixel held (several renders summed in one image).
+__device__ __forceinline__ float pixel(float held, float a, int mode) {
+    return mode == 2 ? held + a : (mode ? a : -expm1f(-a));
 }
 
-constexpr int kWarpsPerCta = 2;
+constexpr int kWarps = 8;    // per CTA: the largest team
 constexpr int kBatch = 192;  // records per batch
+constexpr int kFew = 64;     // records up to which a lone warp's item takes render_few; a
+                             // team's part: half of that
+
+// Warps per team, from the frame's `records` (times the regions per tile edge: a region reads its
+// tile's whole list and keeps a part of it), items of at most K records and `warps` warps.  A warp alone has the least overhead per
+// item, but a frame with fewer records than `warps` full items ends with its longest ones.
+// Measured on 2432 warps, us with teams of 1 / 2 / 4 / 8 (kernel and k_item_order; 50 k to 8 M
+// clustered particles at 256^2, 1024^2 and 2048^2):
+//   records / (warps K)
+//   0.01 - 0.02   99 / 64 / 44 / 35     109 / 78 / 52 / 47     107 / 72 / 52 / 50
+//   0.08 - 0.14   134 / 83 / 54 / 42    135 / 89 / 70 / 60     154 / 97 / 76 / 81
+//   0.25 - 0.47   140 / 88 / 91 / 91    166 / 107 / 99 / 116   191 / 150 / 142 / 154
+//   0.8 - 1.4     224 / 154 / 140 / 164    271 / 199 / 205 / 248    342 / 300 / 314 / 369
+//   2.0 - 3.8     283 / 283 / 302 / 380    428 / 459 / 478 / 590    654 / 707 / 750 / 908
+__device__ __forceinline__ int team_of(int64_t records, int64_t K, int64_t warps) {
+    const float r = __fdividef((float)records, (float)(warps * K));
+    return r < 0.2f ? 8 : r < 0.5f ? 4 : r < 1.5f ? 2 : 1;
+}
+
+// Size bin from which a team shares an item: an eighth of K, 256 records (from a quarter, 50 k
+// particles at 256^2 take 48 us instead of 35), for teams of 2 a quarter (from an eighth, 1 M uniform
+// particles at 2048^2 take 167 us against 151).
+__device__ __forceinline__ int shared_from(int team) { return team > 2 ? kOrderBins / 8 : kOrderBins / 4; }
+
+// Barrier of one team's warps (`team` of them, a power of two).
+__device__ __forceinline__ void team_sync(int team) {
+    __syncwarp();
+    if (team > 1)
+        asm volatile("barrier.sync %0, %1;" ::"r"(1 + (int)(threadIdx.x >> 5) / team), "r"(team * 32) : "memory");
+}
+
+// What the epilogue of an item needs, kept in shared memory over the item's passes: its view,
+// its tile and region (pixels), the tile's scratch slot (-1: not split) and the items that
+// add into it.
+struct __align__(16) Place {
+    int v, tx0, ty0, qx, qy, tw, th, slot, arrivals;
+};
+
+// What a warp knows of the frame and its team, in shared memory as well: image size, tiles per
+// row and the size of the team.
+struct __align__(16) Known {
+    int W, H, ntx, team;
+};
 
 struct __align__(16) WarpSmem {
     Batch<kBatch> batch;             // pb: emission r, g, b
     float acc[3][kRegion][kRegion];  // the region's accumulator
 };
 
+// End of an item: the final transform of the region's pixels, or the merge of a split tile.
+// kAlone: the item was a lone warp's; else its whole team takes part.
+template <bool kAlone>
+__device__ __forceinline__ void finish_item(const FrameDev &fr, float *out, int out_accum, WarpSmem *ws,
+                                            const Place &at, const Known &kn, int *s_last) {
+    const int team = kAlone ? 1 : kn.team, unit = 32 * team, me = (int)threadIdx.x & (unit - 1);
+    float *acc = &ws->acc[0][0][0];
+    if (!kAlone) {  // the warps' sums, in warp order, into the first one's accumulator
+        team_sync(team);
+        WarpSmem *first = ws - (me >> 5);
+        acc = &first->acc[0][0][0];
+        for (int k = me; k < 3 * kRegion * kRegion; k += unit) {
+            float sum = acc[k];
+            for (int w = 1; w < team; ++w) sum += (&first[w].acc[0][0][0])[k];
+            acc[k] = sum;
+        }
+        team_sync(team);
+    }
+    const float(*sums)[kRegion][kRegion] = reinterpret_cast<const float(*)[kRegion][kRegion]>(acc);
+    const int W = kn.W, H = kn.H, px0 = at.tx0 + at.qx, py0 = at.ty0 + at.qy, tw = at.tw, th = at.th, slot = at.slot;
+    const bool vec_rows = (W & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;  // 16-byte rows of 4 pixels
+    float *o = out + (int64_t)at.v * H * W * 3;
+    if (slot < 0) {
+        float *reg = o + ((int64_t)py0 * W + px0) * 3;
+        // rows of 48 floats, four at a time where they are aligned
+        const bool wide = tw == kRegion && vec_rows && (px0 & 3) == 0;
+        // What the pixels held comes through the batch's space, all of a lane's values in flight
+        // together (read one by one, a warp's 24 trips to memory: 485 instead of 338 us for 400 k
+        // clustered particles added to an image of 3958 x 4096).
+        float *held = reinterpret_cast<float *>(ws->batch.pa) + (wide ? 4 : 1) * (threadIdx.x & 31);
+        static_assert(sizeof(ws->batch.pa) >= 3 * kRegion * kRegion * sizeof(float), "a region's values");
+        if (out_accum == 2) {
+            if (wide) {
+                for (int k = me, i = 0; k < th * 12; k += unit, i += 128)
+                    copy16_async(held + i, reg + (int64_t)(k / 12) * W * 3 + 4 * (k % 12));
+            } else {
+                for (int k = me, i = 0; k < 3 * kRegion * kRegion; k += unit, i += 32) {
+                    const int r = k / (3 * kRegion), c = k % (3 * kRegion);
+                    if (r < th && c / 3 < tw) copy4_async(held + i, reg + (int64_t)r * W * 3 + c);
+                }
+            }
+            copy_wait_all();
+        }
+        if (wide) {
+            for (int k = me, i = 0; k < th * 12; k += unit, i += 128) {
+                const int r = k / 12, c = 4 * (k - 12 * r);
+                float4 u = *reinterpret_cast<float4 *>(held + i);
+                u.x = pixel(u.x, sums[(c + 0) % 3][r][(c + 0) / 3], out_accum);
+                u.y = pixel(u.y, sums[(c + 1) % 3][r][(c + 1) / 3], out_accum);
+                u.z = pixel(u.z, sums[(c + 2) % 3][r][(c + 2) / 3], out_accum);
+                u.w = pixel(u.w, sums[(c + 3) % 3][r][(c + 3) / 3], out_accum);
+                *reinterpret_cast<float4 *>(reg + (int64_t)r * W * 3 + c) = u;
+            }
+        } else {
+            for (int k = me, i = 0; k < 3 * kRegion * kRegion; k += unit, i += 32) {
+                const int r = k / (3 * kRegion), c = k % (3 * kRegion), col = c / 3;
+                if (r < th && col < tw)
+                    reg[(int64_t)r * W * 3 + c] = pixel(held[i], sums[c % 3][r][col], out_accum);
+            }
+        }
+    } else {
+        const int T = fr.T;
+        unsigned long long *scr = fr.scratch + (int64_t)slot * 6 * T * T;
+        // 8 values per thread at a time, so that their atomics are in flight together
+#pragma unroll 1
+        for (int k0 = me; k0 < 3 * kRegion * kRegion; k0 += 8 * unit) {
+            float val[8];
+            unsigned long long *dst[8];
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                const int k = k0 + unit * g;
+                const int ch = k / (kRegion * kRegion), r = (k / kRegion) % kRegion, col = k % kRegion;
+                val[g] = k < 3 * kRegion * kRegion && r < th && col < tw ? acc[k] : 0.0f;
+                dst[g] = &scr[2 * (ch * T * T + (at.qy + r) * T + at.qx + col)];
+            }
+            fix_add_n<8>(dst, val);
+        }
+        __threadfence();
+        int last = 0;
+        team_sync(team);
+        if (!kAlone) {
+            if (me == 0) s_last[threadIdx.x / unit] = (atomicAdd(&fr.tickets[slot], 1) == at.arrivals - 1);
+            team_sync(team);
+            last = s_last[threadIdx.x / unit];
+        } else {
+            if (me == 0) last = (atomicAdd(&fr.tickets[slot], 1) == at.arrivals - 1);
+            last = __shfl_sync(0xffffffffu, last, 0);
+        }
+        if (last) {
+            // the whole tile, from the scratch every region of every slice added into
+            __threadfence();
+            const int TW = min(T, W - at.tx0), TH = min(T, H - at.ty0);
+            const int rl = 3 * TW;
+            float *ot = o + ((int64_t)at.ty0 * W + at.tx0) * 3;
+            for (int k0 = me; k0 < TH * rl; k0 += 4 * unit) {
+                float a[4];
+                int64_t pos[4];
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    const int k = min(k0 + unit * g, TH * rl - 1);
+                    const int rr = k / rl, c3 = k - rr * rl;
+                    const int col = c3 / 3, ch = c3 - col * 3;
+                    a[g] = fix_value(&scr[2 * (ch * T * T + rr * T + col)]);
+                    pos[g] = (int64_t)rr * W * 3 + c3;
+                }
+#pragma unroll
+                for (int g = 0; g < 4; ++g)
+                    if (k0 + unit * g < TH * rl) ot[pos[g]] = pixel(ot[pos[g]], a[g], out_accum);
+            }
+            team_sync(team);
+            for (int k = me; k < 6 * T * T; k += unit) scr[k] = 0ull;
+            if (me == 0) fr.tickets[slot] = 0;
+        }
+    }
+}
+
+// Adds a record (pa: -X, -Y, R^2, Gaussian scale; pb: its emission) to 2 x 4 pixels with
+// centres at columns fx0, fx1 and rows fy.
+__device__ __forceinline__ void add_record(float4 pa, float4 pb, float2 fx0, float2 fx1, float2 fy,
+                                           float2 (&s)[3][2][2]) {
+    const float R2 = pa.z;
+    const float2 dx0 = __fadd2_rn(fx0, f2(pa.x)), dx1 = __fadd2_rn(fx1, f2(pa.x));
+    const float2 dy = __fadd2_rn(fy, f2(pa.y));
+    const float2 qx0 = __fmul2_rn(dx0, dx0), qx1 = __fmul2_rn(dx1, dx1);
+    const float2 qy = __fmul2_rn(dy, dy);
+#pragma unroll
+    for (int row = 0; row < 2; ++row) {
+        const float2 qr = f2(row ? qy.y : qy.x);
+#pragma unroll
+        for (int cp = 0; cp < 2; ++cp) {
+            const float2 d2 = __fadd2_rn(cp ? qx1 : qx0, qr);
+            const float2 g = __fmul2_rn(d2, f2(pa.w));
+            const float2 w = make_float2(d2.x < R2 ? ex2_fast(g.x) : 0.0f, d2.y < R2 ? ex2_fast(g.y) : 0.0f);
+            s[0][row][cp] = __ffma2_rn(f2(pb.x), w, s[0][row][cp]);
+            s[1][row][cp] = __ffma2_rn(f2(pb.y), w, s[1][row][cp]);
+            s[2][row][cp] = __ffma2_rn(f2(pb.z), w, s[2][row][cp]);
+        }
+    }
+}
+
+// An item of few records, into the accumulator: 32 records at a time are decoded, one per lane,
+// and evaluated one after another by the whole warp, 2 x 4 pixels per lane.  Batches, lists and
+// sorted squares cost an item about 15 us of a warp's time whatever it holds, nearly all of it
+// latency: 50 k particles at 4096^2 take 142 us instead of 213.  The limit: with 32 / 64 / 96
+// records, 300 k clustered particles at 4096^2 take 253 / 232 / 232 us; 1 M at 256^2 (teams of 4)
+// 76 / 85 / 85.
+template <bool kViewScale, bool kEmit>
+__device__ __forceinline__ void render_few(const SceneDev &sc, const FrameDev &fr, WarpSmem *ws, const Region &rg,
+                                           const float4 *recs, int nrec, int v, float kexp) {
+    const int lane = threadIdx.x & 31, x = 4 * (lane & 3), y = 2 * (lane >> 2);
+    Batch<kBatch> *bt = &ws->batch;
+    const float fx = (float)(rg.px0 + x) + 0.5f, fy0 = (float)(rg.py0 + y) + 0.5f;
+    const float2 fx0 = make_float2(fx, fx + 1.0f), fx1 = make_float2(fx + 2.0f, fx + 3.0f);
+    const float2 fy = make_float2(fy0, fy0 + 1.0f);
+    float2 s[3][2][2];  // channel, row, column pair
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s[c][k >> 1][k & 1] = f2(0.0f);
+    for (int base = 0; base < nrec; base += 32) {
+        const float4 rec[1] = {__ldcs(&recs[min(base + lane, nrec - 1)])};
+        const bool live = base + lane < nrec && fmaxf(fabsf(rec[0].x - rg.xc), fabsf(rec[0].y - rg.yc)) <
+                                                    fmaf(rec[0].z, 1.000004f, rg.half);
+        const uint32_t bal = __ballot_sync(0xffffffffu, live);
+        float3 e[1];
+        float vs = 1.0f;
+        if constexpr (kEmit) {  // the record's last word is the particle index
+            const float4 em = __ldg(&sc.emit[__float_as_uint(rec[0].w)]);
+            e[0] = make_float3(em.x, em.y, em.z);
+            if constexpr (kViewScale) vs = __ldg(&fr.vscale[v * sc.n_types + __float_as_int(em.w)]);
+        } else {
+            batch_colours<1>(rec, kViewScale ? fr.vlut : sc.lut, kViewScale ? fr.vlut_len + v * sc.n_types : sc.lut_len,
+                             kViewScale ? fr.vlut_off + v * sc.n_types : sc.lut_off, e);
+            if constexpr (kViewScale) vs = __ldg(&fr.vscale[v * sc.n_types + (__float_as_uint(rec[0].w) >> 24)]);
+        }
+        if (live) {
+            const int j = __popc(bal & ((1u << lane) - 1u));
+            const float R2 = __fmul_rn(rec[0].z, rec[0].z);
+            bt->pa[j] = make_float4(-rec[0].x, -rec[0].y, R2, gauss_scale(kexp, R2));
+            bt->pb[j] = make_float4(e[0].x * vs, e[0].y * vs, e[0].z * vs, 0.0f);
+        }
+        __syncwarp();
+        const int n = __popc(bal);
+#pragma unroll 2
+        for (int j = 0; j < n; ++j) {
+            const float4 pa = bt->pa[j], pb = bt->pb[j];
+            add_record(pa, pb, fx0, fx1, fy, s);
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int row = 0; row < 2; ++row)
+            *reinterpret_cast<float4 *>(&ws->acc[c][y + row][x]) =
+                make_float4(s[c][row][0].x, s[c][row][0].y, s[c][row][1].x, s[c][row][1].y);
+}
+
 // kViewScale: multiply every record's emission by a per-view, per-species scale (plans
 // with a brightness sequence); a separate instance, so plain renders carry no extra code.
 template <bool kViewScale, bool kEmit>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
+__global__ void __launch_bounds__(kWarps * 32, 2)
     k_splat(SceneDev sc, FrameDev fr, int *queue, float *out, int out_accum, int split) {
     if (fr.status[kStatOverflow]) return;  // no complete tile lists
     extern __shared__ __align__(16) unsigned char s_raw[];
+    __shared__ int s_item[kWarps], s_last[kWarps];  // per team
+    __shared__ Known s_known[kWarps];
+    __shared__ Place s_place[kWarps];
     WarpSmem *ws = reinterpret_cast<WarpSmem *>(s_raw) + (threadIdx.x >> 5);
+    const int total_items = (int)fr.sizes[kSizeItems] * split * split;
     Batch<kBatch> *bt = &ws->batch;
     constexpr int kRounds = Batch<kBatch>::kRounds;
     const int lane = threadIdx.x & 31;
     const int nt = fr.n_tiles;
     const int N = fr.V * nt;
     const int S2 = split * split;
-    const int total_items = (int)fr.sizes[kSizeItems] * S2;
     const int64_t K = fr.sizes[kSizeK];
-    const ViewParams g0 = fr.views[0];
-    const int T = g0.T, W = g0.W, H = g0.H, ntx = g0.ntx;
-    const int sub = (T + split - 1) / split;  // edge of the region a warp owns
-    const int pair = lane >> 1;               // lane pair: the unit that evaluates a square
-    const bool vec_rows = (W & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;  // 16-byte rows of 4 pixels
+    const int pair = lane >> 1;  // lane pair: the unit that evaluates a square
     if (lane == 0) {
         bt->pa[kBatch] = make_float4(0.0f, 0.0f, -1.0f, -1.0f);
         bt->pb[kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
 
+    // What a warp knows of the frame, its team and its item is read from shared memory before
+    // and after the item's passes: they leave no registers for it.
+    if (lane == 0)
+        s_known[threadIdx.x >> 5] = {fr.views[0].W, fr.views[0].H, fr.views[0].ntx,
+                                     team_of(fr.sizes[kSizePairs] * split, K, (int)gridDim.x * kWarps)};
+    __syncwarp();
+
     // the next item is taken from the queue while the current one is rendered
     int next = 0;
-    if (lane == 0) next = atomicAdd(queue, 1);
+    if ((threadIdx.x & (32 * s_known[threadIdx.x >> 5].team - 1)) == 0) next = atomicAdd(queue, 1);
     for (;;) {
-        const int item = __shfl_sync(0xffffffffu, next, 0);
+        const Known kn = s_known[threadIdx.x >> 5];
+        const int me = (int)threadIdx.x & (32 * kn.team - 1);  // of the team's threads
+        int item;
+        if (kn.team > 1) {
+            int *box = &s_item[threadIdx.x / (32 * kn.team)];
+            if (me == 0) *box = next;
+            team_sync(kn.team);
+            item = *box;
+        } else {
+            item = __shfl_sync(0xffffffffu, next, 0);
+        }
         if (item >= total_items) break;
-        if (lane == 0) next = atomicAdd(queue, 1);
+        if (me == 0) next = atomicAdd(queue, 1);
 
         // item = (slice of a tile list, region of the tile); the regions of a slice are
         // consecutive items, so they run at once and share the slice's records in L2
@@ -113,26 +375,57 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
             chunk = qs - fr.item_off[gt];
         }
         const int v = gt / nt, t = gt - v * nt;
-        const int arrivals = (fr.item_off[gt + 1] - fr.item_off[gt]) * S2;
-        const int slot = fr.split_slot[gt];
         const float kexp = fr.views[v].kexp;
-        const int tx = t % ntx, ty = t / ntx;
-        const int qx = (q % split) * sub, qy = (q / split) * sub;
-        const int px0 = tx * T + qx, py0 = ty * T + qy;
-        const int tw = max(0, min(min(sub, T - qx), W - px0));
-        const int th = max(0, min(min(sub, T - qy), H - py0));
+        Region rg;
+        int nrec;
+        {
+            const int T = fr.T, sub = (T + split - 1) / split;  // edge of the region a team owns
+            Place p;
+            p.v = v;
+            p.tx0 = t % kn.ntx * T, p.ty0 = t / kn.ntx * T;
+            p.qx = (q % split) * sub, p.qy = (q / split) * sub;
+            p.tw = max(0, min(min(sub, T - p.qx), kn.W - p.tx0 - p.qx));
+            p.th = max(0, min(min(sub, T - p.qy), kn.H - p.ty0 - p.qy));
+            p.slot = fr.split_slot[gt];
+            p.arrivals = (fr.item_off[gt + 1] - fr.item_off[gt]) * S2;
+            if (lane == 0) s_place[threadIdx.x >> 5] = p;
+            rg = make_region(p.tx0 + p.qx, p.ty0 + p.qy, p.tw, p.th);
+            nrec = p.tw > 0 && p.th > 0;
+        }
         const int64_t seg1 = fr.offsets[gt + 1];
         const int64_t e0 = fr.offsets[gt] + (int64_t)chunk * K;
-        const int nrec = (tw > 0 && th > 0) ? (int)(min(seg1, e0 + K) - e0) : 0;
+        if (nrec) nrec = (int)(min(seg1, e0 + K) - e0);
+        if (nrec == 0 && out_accum == 2 && kn.team == 1 && fr.split_slot[gt] < 0) continue;  // adds nothing
         const float4 *recs = fr.lists + e0;
+        if (kn.team > 1) {
+            int part = ((nrec + kn.team - 1) / kn.team + 31) & ~31;
+            if (order_bin(nrec, (int)K) < shared_from(kn.team)) {  // the first warp's alone
+                part = nrec;
+                if (fr.order) {  // and so are all later items: the team parts
+                    if (lane == 0) s_known[threadIdx.x >> 5].team = 1;
+                    __syncwarp();
+                    if (me >= 32) {
+                        if (lane == 0) next = atomicAdd(queue, 1);
+                        continue;
+                    }
+                }
+            }
+            // this warp's consecutive part of the slice
+            const int first = min(nrec, (me >> 5) * part);
+            recs += first;
+            nrec = min(part, nrec - first);
+        }
 
-        float *acc = &ws->acc[0][0][0];
+        if (nrec <= (kn.team == 1 ? kFew : kFew / 2)) {
+            render_few<kViewScale, kEmit>(sc, fr, ws, rg, recs, nrec, v, kexp);
+            nrec = 0;
+        } else {
+            float *acc = &ws->acc[0][0][0];
 #pragma unroll
-        for (int k = 0; k < 3 * kRegion * kRegion / 128; ++k)
-            reinterpret_cast<float4 *>(acc)[k * 32 + lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-
-        const Region rg = make_region(px0, py0, tw, th);
-        batch_start(bt, recs, nrec);
+            for (int k = 0; k < 3 * kRegion * kRegion / 128; ++k)
+                reinterpret_cast<float4 *>(acc)[k * 32 + lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            batch_start(bt, recs, nrec);
+        }
         int base = 0, row = 0;
         while (base < nrec) {
             // ---- 1. fill the batch with records that meet the region
@@ -200,7 +493,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
                 const unsigned char *lp = bt->list[sq] + r;
                 // this lane's pixels: rows y, y + 1 and columns x .. x + 3 of the region
                 const int x = 4 * (sq & 3), y = 4 * (sq >> 2) + 2 * (lane & 1);
-                const float fx = (float)(px0 + x) + 0.5f, fy0 = (float)(py0 + y) + 0.5f;
+                const float fx = (float)(rg.px0 + x) + 0.5f, fy0 = (float)(rg.py0 + y) + 0.5f;
                 const float2 fx0 = make_float2(fx, fx + 1.0f), fx1 = make_float2(fx + 2.0f, fx + 3.0f);
                 const float2 fy = make_float2(fy0, fy0 + 1.0f);
                 float2 s[3][2][2];  // channel, row, column pair
@@ -222,24 +515,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
                     nb = bt->pb[idx];
                     lp += 1 << a;
                     idx = k < mine ? *lp : kBatch;
-                    const float2 dx0 = __fadd2_rn(fx0, f2(pa.x)), dx1 = __fadd2_rn(fx1, f2(pa.x));
-                    const float2 dy = __fadd2_rn(fy, f2(pa.y));
-                    const float2 qx0 = __fmul2_rn(dx0, dx0), qx1 = __fmul2_rn(dx1, dx1);
-                    const float2 qy = __fmul2_rn(dy, dy);
-#pragma unroll
-                    for (int row = 0; row < 2; ++row) {
-                        const float2 qr = f2(row ? qy.y : qy.x);
-#pragma unroll
-                        for (int cp = 0; cp < 2; ++cp) {
-                            const float2 d2 = __fadd2_rn(cp ? qx1 : qx0, qr);
-                            const float2 g = __fmul2_rn(d2, f2(pa.w));
-                            const float2 w = make_float2(d2.x < R2 ? ex2_fast(g.x) : 0.0f,
-                                                         d2.y < R2 ? ex2_fast(g.y) : 0.0f);
-                            s[0][row][cp] = __ffma2_rn(f2(pb.x), w, s[0][row][cp]);
-                            s[1][row][cp] = __ffma2_rn(f2(pb.y), w, s[1][row][cp]);
-                            s[2][row][cp] = __ffma2_rn(f2(pb.z), w, s[2][row][cp]);
-                        }
-                    }
+                    add_record(pa, pb, fx0, fx1, fy, s);
                 }
                 for (int d = 2; d < (2 << a); d <<= 1) {
 #pragma unroll
@@ -268,76 +544,12 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 8)
             }
         }
         __syncwarp();
-
-        // epilogue: final transform of the region's pixels, or merge of a split tile
-        float *o = out + (int64_t)v * H * W * 3;
-        if (slot < 0) {
-            float *reg = o + ((int64_t)py0 * W + px0) * 3;
-            if (tw == kRegion && vec_rows && (px0 & 3) == 0) {
-                // rows of 48 floats, four at a time
-                for (int k = lane; k < th * 12; k += 32) {
-                    const int r = k / 12, c = 4 * (k - 12 * r);
-                    float4 *p = reinterpret_cast<float4 *>(reg + (int64_t)r * W * 3 + c);
-                    float4 u = out_accum == 2 ? *p : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                    put_pixel(&u.x, ws->acc[(c + 0) % 3][r][(c + 0) / 3], out_accum);
-                    put_pixel(&u.y, ws->acc[(c + 1) % 3][r][(c + 1) / 3], out_accum);
-                    put_pixel(&u.z, ws->acc[(c + 2) % 3][r][(c + 2) / 3], out_accum);
-                    put_pixel(&u.w, ws->acc[(c + 3) % 3][r][(c + 3) / 3], out_accum);
-                    *p = u;
-                }
-            } else {
-                for (int k = lane; k < 3 * kRegion * kRegion; k += 32) {
-                    const int r = k / (3 * kRegion), c = k % (3 * kRegion), col = c / 3;
-                    if (r < th && col < tw) put_pixel(&reg[(int64_t)r * W * 3 + c], ws->acc[c % 3][r][col], out_accum);
-                }
-            }
-        } else {
-            unsigned long long *scr = fr.scratch + (int64_t)slot * 6 * T * T;
-            // 8 values per lane at a time, so that their atomics are in flight together
-#pragma unroll 1
-            for (int k0 = lane; k0 < 3 * kRegion * kRegion; k0 += 256) {
-                float val[8];
-                unsigned long long *dst[8];
-#pragma unroll
-                for (int g = 0; g < 8; ++g) {
-                    const int k = k0 + 32 * g;
-                    const int ch = k / (kRegion * kRegion), r = (k / kRegion) % kRegion, col = k % kRegion;
-                    val[g] = r < th && col < tw ? acc[k] : 0.0f;
-                    dst[g] = &scr[2 * (ch * T * T + (qy + r) * T + qx + col)];
-                }
-                fix_add_n<8>(dst, val);
-            }
-            __threadfence();
-            __syncwarp();
-            int last = 0;
-            if (lane == 0) last = (atomicAdd(&fr.tickets[slot], 1) == arrivals - 1);
-            last = __shfl_sync(0xffffffffu, last, 0);
-            if (last) {
-                // the whole tile, from the scratch every region of every slice added into
-                __threadfence();
-                const int TW = min(T, W - tx * T), TH = min(T, H - ty * T);
-                const int rl = 3 * TW;
-                float *ot = o + ((int64_t)ty * T * W + (int64_t)tx * T) * 3;
-                for (int k0 = lane; k0 < TH * rl; k0 += 128) {
-                    float a[4];
-                    int64_t at[4];
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        const int k = min(k0 + 32 * g, TH * rl - 1);
-                        const int rr = k / rl, c3 = k - rr * rl;
-                        const int col = c3 / 3, ch = c3 - col * 3;
-                        a[g] = fix_value(&scr[2 * (ch * T * T + rr * T + col)]);
-                        at[g] = (int64_t)rr * W * 3 + c3;
-                    }
-#pragma unroll
-                    for (int g = 0; g < 4; ++g)
-                        if (k0 + 32 * g < TH * rl) put_pixel(&ot[at[g]], a[g], out_accum);
-                }
-                __syncwarp();
-                for (int k = lane; k < 6 * T * T; k += 32) scr[k] = 0ull;
-                if (lane == 0) fr.tickets[slot] = 0;
-            }
-        }
+        const Known end = s_known[threadIdx.x >> 5];
+        const Place at = s_place[threadIdx.x >> 5];
+        if (end.team == 1)
+            finish_item<true>(fr, out, out_accum, ws, at, end, s_last);
+        else
+            finish_item<false>(fr, out, out_accum, ws, at, end, s_last);
         __syncwarp();
     }
 }
@@ -351,17 +563,17 @@ static SplatFn splat_fn(bool scaled, bool emit) {
     return scaled ? k_splat<true, false> : k_splat<false, false>;
 }
 
-static size_t splat_smem() { return sizeof(WarpSmem) * kWarpsPerCta; }
+static size_t splat_smem() { return sizeof(WarpSmem) * kWarps; }
 
 int splat_blocks_per_sm() {
     const void *fn = (const void *)splat_fn(false, false);
     if (ensure_smem_limit(fn, splat_smem()) != cudaSuccess) return 0;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kWarpsPerCta * 32, splat_smem()) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kWarps * 32, splat_smem()) != cudaSuccess) return 0;
     return nb;
 }
 
-int splat_workers_per_sm() { return splat_blocks_per_sm() * kWarpsPerCta; }
+int splat_workers_per_sm() { return splat_blocks_per_sm() * kWarps; }
 
 // k_item_order: the splat's work items (tile-list slices) ordered by record count, largest
 // first, so that the items taken last by the workers are the short ones and the kernel does
@@ -429,7 +641,7 @@ cudaError_t launch_splat(const SceneDev &sc, const FrameDev &fr, float *out, int
     const SplatFn fn = splat_fn(fr.vscale != nullptr, sc.emit != nullptr);
     e = ensure_smem_limit((const void *)fn, splat_smem());
     if (e != cudaSuccess) return e;
-    fn<<<grid, kWarpsPerCta * 32, splat_smem(), st>>>(sc, fr, fr.queue, out, out_accum, splat_split(fr.T));
+    fn<<<grid, kWarps * 32, splat_smem(), st>>>(sc, fr, fr.queue, out, out_accum, splat_split(fr.T));
     return cudaGetLastError();
 }
 

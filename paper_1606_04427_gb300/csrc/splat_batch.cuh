@@ -33,6 +33,9 @@ template <int B> struct __align__(16) Batch {
 __device__ __forceinline__ void copy16_async(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
+__device__ __forceinline__ void copy4_async(void *dst, const void *src) {  // 4 bytes
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
 __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void copy_wait() {  // all but the newest N groups done
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");

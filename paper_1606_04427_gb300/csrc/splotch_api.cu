@@ -782,15 +782,9 @@ static cudaError_t clear_split_scratch(const FrameHost &fh, char *var, int split
     return cudaMemsetAsync(var + fh.o_scratch, 0, fh.o_tickets - fh.o_scratch + sizeof(int) * (size_t)splits, st);
 }
 
-// items: work items of the scan (tile-list slices); the splat renders each as split^2
-// squares, one worker each
-static int splat_grid(int dev, int T, int items) {
-    const int bps = std::max(1, splat_blocks_per_sm());
-    const int per_cta = std::max(1, splat_workers_per_sm() / bps);
-    const int g = sm_count(dev) * bps;
-    const int64_t squares = (int64_t)std::max(1, items) * splat_split(T) * splat_split(T);
-    return (int)std::max<int64_t>(1, std::min<int64_t>(g, (squares + per_cta - 1) / per_cta));
-}
+// The whole chip, whatever the frame holds: the kernel shares a frame's few work items among
+// all warps.
+static int splat_grid(int dev) { return sm_count(dev) * std::max(1, splat_blocks_per_sm()); }
 
 static int target_items(int dev, int T) {
     const int s = splat_split(T);
@@ -851,14 +845,13 @@ static splotch_status count_and_size(splotch_scene *sc, const RenderSetup &rs, F
 
 // Enqueue scatter + splat for a sized frame.
 static splotch_status scatter_and_splat(splotch_scene *sc, FrameHost &fh, char *fixed, char *var, float *out,
-                                        int out_accum, bool stable, int items, cudaStream_t st,
+                                        int out_accum, bool stable, cudaStream_t st,
                                         cudaEvent_t *ev = nullptr) {
     FrameDev fr = frame_dev(fh, fixed, var);
     if (ev) CUDA_TRY(cudaEventRecord(ev[3], st));
     CUDA_TRY(launch_scatter(sc->storage, sc->dev_view, fr, stable, st));
     if (ev) CUDA_TRY(cudaEventRecord(ev[4], st));
-    CUDA_TRY(launch_splat(sc->dev_view, fr, out, out_accum,
-                          splat_grid(sc->dev, fh.T, items), st));
+    CUDA_TRY(launch_splat(sc->dev_view, fr, out, out_accum, splat_grid(sc->dev), st));
     if (ev) CUDA_TRY(cudaEventRecord(ev[5], st));
     return SPLOTCH_OK;
 }
@@ -919,7 +912,7 @@ static splotch_status render_frame(splotch_scene *sc, const RenderSetup &rs, flo
             break;
         }
         s = scatter_and_splat(sc, fh, fixed, var, out, out_mode(rs.pr.flags), (rs.pr.flags & SPLOTCH_STABLE) != 0,
-                              items, st, ev);
+                              st, ev);
         if (s != SPLOTCH_OK) break;
         if (sync) {
             int64_t *box = host_box();
@@ -1094,7 +1087,7 @@ static splotch_status frame_splat(splotch_frame *f, float *out, cudaStream_t st)
     splotch_status s = frame_follow(f, st);
     if (s != SPLOTCH_OK) return s;
     CUDA_TRY(launch_splat(f->sc->dev_view, frame_dev(f->fh, f->fixed, f->var), out, out_mode(f->rs.pr.flags),
-                          splat_grid(f->sc->dev, f->fh.T, (int)f->sizes[kSizeItems]), st));
+                          splat_grid(f->sc->dev), st));
     return SPLOTCH_OK;
 }
 
@@ -1156,8 +1149,7 @@ static splotch_status plan_enqueue(splotch_plan *pl, float *out, cudaStream_t st
     CUDA_TRY(launch_count(sc->storage, sc->dev_view, fr, st));
     CUDA_TRY(launch_scan(fr, target_items(sc->dev, fh.T), kMinItemPairs, st));
     CUDA_TRY(launch_scatter(sc->storage, sc->dev_view, fr, (pl->rs.pr.flags & SPLOTCH_STABLE) != 0, st));
-    CUDA_TRY(launch_splat(sc->dev_view, fr, out,
-                          out_mode(pl->rs.pr.flags), pl->grid, st));
+    CUDA_TRY(launch_splat(sc->dev_view, fr, out, out_mode(pl->rs.pr.flags), pl->grid, st));
     CUDA_TRY(cudaMemcpyAsync(pl->box, pl->fixed + fh.o_sizes, sizeof(int64_t) * 8, cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaMemcpyAsync(pl->box + 8, pl->fixed + fh.o_status, sizeof(int) * 4, cudaMemcpyDeviceToHost, st));
     return SPLOTCH_OK;
@@ -1225,7 +1217,7 @@ extern "C" splotch_status splotch_plan_create(splotch_scene *sc, const splotch_c
         splotch_plan_destroy(pl);
         return fail(SPLOTCH_ERR_CUDA, "plan scratch");
     }
-    pl->grid = splat_grid(sc->dev, pl->rs.T, INT32_MAX);
+    pl->grid = splat_grid(sc->dev);
     // emission scale per view and species (1 until splotch_plan_set_brightness): a fixed
     // device array, so a captured graph reads the current scales at every replay
     {
@@ -1534,8 +1526,7 @@ extern "C" splotch_status splotch_render_noalloc(splotch_scene *sc, const splotc
     CUDA_TRY(launch_count(sc->storage, sc->dev_view, fr, st));
     CUDA_TRY(launch_scan(fr, target_items(sc->dev, T), kMinItemPairs, st));
     CUDA_TRY(launch_scatter(sc->storage, sc->dev_view, fr, (pr.flags & SPLOTCH_STABLE) != 0, st));
-    CUDA_TRY(launch_splat(sc->dev_view, fr, out,
-                          out_mode(pr.flags), sm_count(dev) * std::max(1, splat_blocks_per_sm()), st));
+    CUDA_TRY(launch_splat(sc->dev_view, fr, out, out_mode(pr.flags), splat_grid(dev), st));
     int64_t sizes[8];
     int stat[4];
     CUDA_TRY(cudaMemcpyAsync(sizes, base + fh.o_sizes, sizeof(sizes), cudaMemcpyDeviceToHost, st));
