@@ -1103,8 +1103,14 @@ cudaError_t launch_debug_raster(int storage, const SceneDev &sc, const ViewParam
 //   k_sorted_counts  in that order: the gathered record and the number of tiles it belongs
 //                    to (plus a zero past the end, so the exclusive scan ends with the total);
 //   (exclusive scan of the counts: each particle's first output slot)
-//   k_expand         each particle's records at its slots, keyed by tile id;
-//   (stable radix sort by tile id: each tile's records stay in depth order)
+//   k_expand         each particle's place in the depth order, at its slots, keyed by tile id;
+//   (stable radix sort by tile id: each tile's records stay in depth order; its last pass
+//   writes the records of the places)
+// All three stream over the particles and are bound by the latency of their loads, so the next
+// particle's loads are issued before the current one is worked on.
+// 10 M particles, 20.7 M pairs (FP16 storage): k_depth_records 135 -> 72 us, k_sorted_counts
+// 204 -> 168, k_expand 202 -> 117 (places instead of 16-byte records), the last pass of the sort
+// by tile 317 -> 238 (the records of 10 M places instead of 20.7 M pairs).
 
 // krange: {min, max} of the active particles' depth keys (atomicMin / atomicMax; the
 // caller sets {all ones, 0} first), so that the sort covers only the bits they span.
@@ -1120,13 +1126,21 @@ __global__ void __launch_bounds__(256) k_depth_records(SceneDev sc, const ViewPa
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int type = 0;
     uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < sc.n; i += stride) {
+    typename Stored<S>::T nx{}, ny{}, nz{}, nh{}, ni{};
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < sc.n)
+        nx = load_stored<S>(sc.x, i), ny = load_stored<S>(sc.y, i), nz = load_stored<S>(sc.z, i),
+        nh = load_stored<S>(sc.h, i), ni = load_stored<S>(sc.it, i);
+    for (; i < sc.n; i += stride) {
+        const float x = value_of(nx), y = value_of(ny), z = value_of(nz), h = value_of(nh), it = value_of(ni);
+        if (i + stride < sc.n)
+            nx = load_stored<S>(sc.x, i + stride), ny = load_stored<S>(sc.y, i + stride),
+            nz = load_stored<S>(sc.z, i + stride), nh = load_stored<S>(sc.h, i + stride),
+            ni = load_stored<S>(sc.it, i + stride);
         while (type + 1 < sc.n_types && i >= s_tb[type + 1]) ++type;
         Raster r;
-        const bool act = raster_one(s_v, load1<S>(sc.x, i), load1<S>(sc.y, i), load1<S>(sc.z, i),
-                                    load1<S>(sc.h, i), r);
-        prec[i] = make_float4(r.X, r.Y, r.R,
-                              sc.emit ? __uint_as_float((uint32_t)i) : record_code(type, load1<S>(sc.it, i)));
+        const bool act = raster_one(s_v, x, y, z, h, r);
+        prec[i] = make_float4(r.X, r.Y, r.R, sc.emit ? __uint_as_float((uint32_t)i) : record_code(type, it));
         const uint32_t k = act ? depth_key(r.zc) : kInactiveKey;
         dkey[i] = k;
         pid[i] = (uint32_t)i;
@@ -1142,13 +1156,6 @@ __global__ void __launch_bounds__(256) k_depth_records(SceneDev sc, const ViewPa
 
 // Depth keys relative to the smallest active one (active: key - base in [0, span];
 // inactive: span + 1, sorted last).
-__global__ void k_rebase_keys(uint32_t *dkey, int64_t n, uint32_t base, uint32_t span) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t k = dkey[i];
-        dkey[i] = k == kInactiveKey ? span + 1u : k - base;
-    }
-}
-
 // Tiles of a rasterised particle, in row-major order over its tile box: the first
 // `small` boxes (up to 2 x 2) by one lane, larger ones by the whole warp.
 __device__ __forceinline__ void tile_box(const ViewParams &v, float X, float Y, float R, int &tx0, int &tx1,
@@ -1162,26 +1169,38 @@ __global__ void __launch_bounds__(256) k_sorted_counts(const ViewParams *__restr
                                                        const float4 *__restrict__ prec,
                                                        const uint32_t *__restrict__ skey,
                                                        const uint32_t *__restrict__ spid, int64_t n,
-                                                       uint32_t inactive, float4 *srec, uint32_t *cnt) {
+                                                       uint32_t inactive, float4 *srec, uint32_t *cnt,
+                                                       uint32_t *arrivals) {
     __shared__ ViewParams s_v;
     if (threadIdx.x == 0) s_v = views[0];
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t wstride = (int64_t)gridDim.x * blockDim.x;
-    if (blockIdx.x == 0 && threadIdx.x == 0) cnt[n] = 0;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += wstride) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) cnt[n] = 0, *arrivals = 0;
+    const int64_t base0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
+    // ahead: the next particle's record, and the key and index of the one after it
+    float4 nrec = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    bool nact = false;
+    uint32_t key = inactive, pid = 0;
+    if (base0 + lane < n) {
+        nact = skey[base0 + lane] != inactive;
+        if (nact) nrec = prec[spid[base0 + lane]];
+    }
+    if (base0 + lane + wstride < n) key = skey[base0 + lane + wstride], pid = spid[base0 + lane + wstride];
+    for (int64_t base = base0; base < n; base += wstride) {
         const int64_t q = base + lane;
-        float4 rec = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        const float4 rec = nrec;
+        const bool act = nact;
+        nrec = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        nact = key != inactive;
+        if (nact) nrec = prec[pid];
+        key = inactive;
+        if (q + 2 * wstride < n) key = skey[q + 2 * wstride], pid = spid[q + 2 * wstride];
         int tx0 = 0, tx1 = -1, ty0 = 0, ty1 = -1;
-        if (q < n && skey[q] != inactive) {
-            rec = prec[spid[q]];
-            tile_box(s_v, rec.x, rec.y, rec.z, tx0, tx1, ty0, ty1);
-        }
+        if (act) tile_box(s_v, rec.x, rec.y, rec.z, tx0, tx1, ty0, ty1);
         const bool small = tx1 >= tx0 && tx1 - tx0 <= 1 && ty1 - ty0 <= 1;
         uint32_t c = 0;
-        if (small)
-            for (int ty = ty0; ty <= ty1; ++ty)
-                for (int tx = tx0; tx <= tx1; ++tx) c += tile_member(s_v, rec.x, rec.y, rec.z, tx, ty) ? 1u : 0u;
+        if (small) c = __popc(tile_mask2(s_v, rec.x, rec.y, rec.z, tx0, tx1, ty0, ty1));
         uint32_t big = __ballot_sync(0xffffffffu, tx1 >= tx0 && !small);
         while (big) {
             const int src = __ffs(big) - 1;
@@ -1190,10 +1209,10 @@ __global__ void __launch_bounds__(256) k_sorted_counts(const ViewParams *__restr
             const float bR = __shfl_sync(0xffffffffu, rec.z, src);
             const int bx0 = __shfl_sync(0xffffffffu, tx0, src), bx1 = __shfl_sync(0xffffffffu, tx1, src);
             const int by0 = __shfl_sync(0xffffffffu, ty0, src), by1 = __shfl_sync(0xffffffffu, ty1, src);
-            const int bw = bx1 - bx0 + 1, ncand = bw * (by1 - by0 + 1);
             uint32_t mine = 0;
-            for (int k = lane; k < ncand; k += 32)
-                mine += tile_member(s_v, bX, bY, bR, bx0 + k % bw, by0 + k / bw) ? 1u : 0u;
+            for (int ty = by0 + (lane >> 3); ty <= by1; ty += 4)
+                for (int tx = bx0 + (lane & 7); tx <= bx1; tx += 8)
+                    mine += tile_member(s_v, bX, bY, bR, tx, ty) ? 1u : 0u;
             const uint32_t tot = __reduce_add_sync(0xffffffffu, mine);
             if (lane == src) c = tot;
         }
@@ -1206,7 +1225,8 @@ __global__ void __launch_bounds__(256) k_sorted_counts(const ViewParams *__restr
 
 __global__ void __launch_bounds__(256) k_expand(const ViewParams *__restrict__ views,
                                                 const float4 *__restrict__ srec, const uint32_t *__restrict__ poff,
-                                                int64_t n, int64_t P, float4 *recs, uint32_t *tkey, uint32_t *tval,
+                                                const uint32_t *__restrict__ sums, int64_t n, int64_t P,
+                                                uint32_t *__restrict__ tkey, uint32_t *__restrict__ tval,
                                                 int *status) {
     __shared__ ViewParams s_v;
     if (threadIdx.x == 0) s_v = views[0];
@@ -1214,64 +1234,69 @@ __global__ void __launch_bounds__(256) k_expand(const ViewParams *__restrict__ v
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     const int64_t wstride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += wstride) {
-        const int64_t q = base + lane;
-        float4 rec = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        uint32_t o0 = 0, c = 0;
-        int tx0 = 0, tx1 = -1, ty0 = 0, ty1 = -1;
+    const int64_t base0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
+    float4 nrec = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    uint32_t n0 = 0, n1 = 0;  // first slot of the next particle and of the one after it
+    auto ahead = [&](int64_t q) {
+        n0 = n1 = 0;
         if (q < n) {
-            o0 = poff[q];
-            c = poff[q + 1] - o0;
-            if (c) {
-                rec = srec[q];
-                tile_box(s_v, rec.x, rec.y, rec.z, tx0, tx1, ty0, ty1);
-            }
+            nrec = srec[q];
+            n0 = poff[q] + sums[q / kScanChunk];
+            n1 = poff[q + 1] + sums[(q + 1) / kScanChunk];
         }
+    };
+    ahead(base0 + lane);
+    for (int64_t base = base0; base < n; base += wstride) {
+        const int64_t q = base + lane;
+        const float4 rec = nrec;
+        const uint32_t o0 = n0, c = n1 - n0;
+        ahead(q + wstride);
+        int tx0 = 0, tx1 = -1, ty0 = 0, ty1 = -1;
+        if (c) tile_box(s_v, rec.x, rec.y, rec.z, tx0, tx1, ty0, ty1);
         const bool small = c && tx1 >= tx0 && tx1 - tx0 <= 1 && ty1 - ty0 <= 1;
         if (small) {
-            uint32_t k = 0;
-            for (int ty = ty0; ty <= ty1; ++ty)
-                for (int tx = tx0; tx <= tx1; ++tx) {
-                    if (!tile_member(s_v, rec.x, rec.y, rec.z, tx, ty)) continue;
-                    const uint32_t pos = o0 + k++;
-                    if (k > c || (int64_t)pos >= P) {
-                        atomicExch(&status[kStatOverflow], 1);
-                        continue;
+            const uint32_t m = tile_mask2(s_v, rec.x, rec.y, rec.z, tx0, tx1, ty0, ty1);
+            const uint32_t t00 = (uint32_t)(ty0 * s_v.ntx + tx0);
+            uint32_t pos = o0;
+            if ((uint32_t)__popc(m) > c || (int64_t)o0 + __popc(m) > P) {
+                atomicExch(&status[kStatOverflow], 1);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (m & (1u << k)) {
+                        tkey[pos] = t00 + (k & 1 ? 1u : 0u) + (k & 2 ? (uint32_t)s_v.ntx : 0u);
+                        tval[pos++] = (uint32_t)q;
                     }
-                    recs[pos] = rec;
-                    tkey[pos] = (uint32_t)(ty * s_v.ntx + tx);
-                    tval[pos] = pos;
-                }
+            }
         }
         uint32_t big = __ballot_sync(0xffffffffu, c && tx1 >= tx0 && !small);
         while (big) {
             const int src = __ffs(big) - 1;
             big &= big - 1;
-            const float4 b = make_float4(__shfl_sync(0xffffffffu, rec.x, src), __shfl_sync(0xffffffffu, rec.y, src),
-                                         __shfl_sync(0xffffffffu, rec.z, src), __shfl_sync(0xffffffffu, rec.w, src));
+            const float bX = __shfl_sync(0xffffffffu, rec.x, src), bY = __shfl_sync(0xffffffffu, rec.y, src);
+            const float bR = __shfl_sync(0xffffffffu, rec.z, src);
             const uint32_t bo = __shfl_sync(0xffffffffu, o0, src), bc = __shfl_sync(0xffffffffu, c, src);
             const int bx0 = __shfl_sync(0xffffffffu, tx0, src), bx1 = __shfl_sync(0xffffffffu, tx1, src);
             const int by0 = __shfl_sync(0xffffffffu, ty0, src), by1 = __shfl_sync(0xffffffffu, ty1, src);
-            const int bw = bx1 - bx0 + 1, ncand = bw * (by1 - by0 + 1);
             uint32_t k = 0;
-            for (int kb = 0; kb < ncand; kb += 32) {
-                const int kc = kb + lane;
-                const int tx = bx0 + kc % bw, ty = by0 + kc / bw;
-                const bool m = kc < ncand && tile_member(s_v, b.x, b.y, b.z, tx, ty);
-                const uint32_t bal = __ballot_sync(0xffffffffu, m);
-                if (m) {
-                    const uint32_t kk = k + (uint32_t)__popc(bal & lt);
-                    const uint32_t pos = bo + kk;
-                    if (kk >= bc || (int64_t)pos >= P) {
-                        atomicExch(&status[kStatOverflow], 1);
-                    } else {
-                        recs[pos] = b;
-                        tkey[pos] = (uint32_t)(ty * s_v.ntx + tx);
-                        tval[pos] = pos;
+            // blocks of 8 x 4 candidates, one per lane
+            for (int y = by0; y <= by1; y += 4)
+                for (int x = bx0; x <= bx1; x += 8) {
+                    const int tx = x + (lane & 7), ty = y + (lane >> 3);
+                    const bool m = tx <= bx1 && ty <= by1 && tile_member(s_v, bX, bY, bR, tx, ty);
+                    const uint32_t bal = __ballot_sync(0xffffffffu, m);
+                    if (m) {
+                        const uint32_t kk = k + (uint32_t)__popc(bal & lt);
+                        const uint32_t pos = bo + kk;
+                        if (kk >= bc || (int64_t)pos >= P) {
+                            atomicExch(&status[kStatOverflow], 1);
+                        } else {
+                            tkey[pos] = (uint32_t)(ty * s_v.ntx + tx);
+                            tval[pos] = (uint32_t)(base + src);
+                        }
                     }
+                    k += (uint32_t)__popc(bal);
                 }
-                k += (uint32_t)__popc(bal);
-            }
         }
     }
 }
@@ -1294,24 +1319,18 @@ cudaError_t launch_depth_records(int storage, const SceneDev &sc, const ViewPara
     return cudaGetLastError();
 }
 
-cudaError_t launch_rebase_keys(uint32_t *dkey, int64_t n, uint32_t base, uint32_t span, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    k_rebase_keys<<<stream_grid(n, 256), 256, 0, st>>>(dkey, n, base, span);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_sorted_counts(const ViewParams *views, const float4 *prec, const uint32_t *skey,
                                  const uint32_t *spid, int64_t n, uint32_t inactive, float4 *srec, uint32_t *cnt,
-                                 cudaStream_t st) {
+                                 uint32_t *arrivals, cudaStream_t st) {
     k_sorted_counts<<<stream_grid(std::max<int64_t>(1, n), 256), 256, 0, st>>>(views, prec, skey, spid, n, inactive,
-                                                                               srec, cnt);
+                                                                               srec, cnt, arrivals);
     return cudaGetLastError();
 }
 
-cudaError_t launch_expand(const ViewParams *views, const float4 *srec, const uint32_t *poff, int64_t n, int64_t P,
-                          float4 *recs, uint32_t *tkey, uint32_t *tval, int *status, cudaStream_t st) {
+cudaError_t launch_expand(const ViewParams *views, const float4 *srec, const uint32_t *poff, const uint32_t *sums,
+                          int64_t n, int64_t P, uint32_t *tkey, uint32_t *tval, int *status, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_expand<<<stream_grid(n, 256), 256, 0, st>>>(views, srec, poff, n, P, recs, tkey, tval, status);
+    k_expand<<<stream_grid(n, 256), 256, 0, st>>>(views, srec, poff, sums, n, P, tkey, tval, status);
     return cudaGetLastError();
 }
 

@@ -1794,7 +1794,6 @@ extern "C" splotch_status splotch_render_ordered(splotch_scene *sc, const splotc
     const size_t o_id0 = cv.take(sizeof(uint32_t) * (size_t)n);
     const size_t o_id1 = cv.take(sizeof(uint32_t) * (size_t)n);
     const size_t o_cnt = cv.take(sizeof(uint32_t) * (size_t)(n + 1));
-    const size_t o_rec = cv.take(sizeof(float4) * (size_t)Pm);
     const size_t o_tk0 = cv.take(sizeof(uint32_t) * (size_t)Pm);
     const size_t o_tk1 = cv.take(sizeof(uint32_t) * (size_t)Pm);
     const size_t o_tv0 = cv.take(sizeof(uint32_t) * (size_t)Pm);
@@ -1830,31 +1829,31 @@ extern "C" splotch_status splotch_render_ordered(splotch_scene *sc, const splotc
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     int dbits = 32;
     uint32_t inactive = 0xFFFFFFFFu;  // the key of a particle that is not active
-    if (e == cudaSuccess && kr[0] <= kr[1] && kr[1] - kr[0] < 0xFFFFFFFEu) {
-        const uint32_t span = kr[1] - kr[0];
-        inactive = span + 1u;
+    KeyRange range;
+    if (e == cudaSuccess && sc->n > 1 && kr[0] <= kr[1] && kr[1] - kr[0] < 0xFFFFFFFEu) {
+        range.base = kr[0], range.span = kr[1] - kr[0];
+        inactive = range.span + 1u;
         dbits = 8;
-        while (dbits < 32 && ((uint64_t)span + 1u) >> dbits) dbits += 8;
-        e = launch_rebase_keys(dka, sc->n, kr[0], span, st);
+        while (dbits < 32 && ((uint64_t)range.span + 1u) >> dbits) dbits += 8;
     }
-    if (e == cudaSuccess) e = radix_sort_pairs(dka, dkb, ida, idb, sc->n, 0, dbits, ex + o_tmp, st, &alt);
+    if (e == cudaSuccess) e = radix_sort_pairs(dka, dkb, ida, idb, sc->n, 0, dbits, ex + o_tmp, st, &alt, range);
     if (alt) std::swap(dka, dkb), std::swap(ida, idb);
     // each particle's records at the scanned offsets of its tile counts, keyed by tile
     uint32_t *cnt = (uint32_t *)(ex + o_cnt);
     if (e == cudaSuccess)
         e = launch_sorted_counts(fr.views, (const float4 *)(ex + o_prec), dka, ida, sc->n, inactive,
-                                 (float4 *)(ex + o_srec), cnt, st);
+                                 (float4 *)(ex + o_srec), cnt, scan_arrivals(sc->n + 1, ex + o_tmp), st);
     if (e == cudaSuccess) e = exclusive_scan_u32(cnt, sc->n + 1, ex + o_tmp, st);
     uint32_t *tka = (uint32_t *)(ex + o_tk0), *tkb = (uint32_t *)(ex + o_tk1);
     uint32_t *tva = (uint32_t *)(ex + o_tv0), *tvb = (uint32_t *)(ex + o_tv1);
     if (e == cudaSuccess)
-        e = launch_expand(fr.views, (const float4 *)(ex + o_srec), cnt, sc->n, P, (float4 *)(ex + o_rec), tka, tva,
-                          fr.status, st);
+        e = launch_expand(fr.views, (const float4 *)(ex + o_srec), cnt, (const uint32_t *)(ex + o_tmp), sc->n, P, tka,
+                          tva, fr.status, st);
     // stable by tile id: every tile list keeps depth order
     int tbits = 8;
     while (tbits < 32 && ((int64_t)(rs.views[0].n_tiles - 1) >> tbits) > 0) tbits += 8;
     if (e == cudaSuccess)
-        e = radix_sort_gather(tka, tkb, tva, tvb, P, 0, tbits, ex + o_tmp, (const float4 *)(ex + o_rec), fr.lists, st);
+        e = radix_sort_gather(tka, tkb, tva, tvb, P, 0, tbits, ex + o_tmp, (const float4 *)(ex + o_srec), fr.lists, st);
     const int64_t squares = (int64_t)std::max(1, items) * split * split;
     const int per_cta = std::max(1, ordered_workers_per_sm() / ordered_ctas_per_sm());
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count(sc->dev) * ordered_ctas_per_sm(),

@@ -422,33 +422,41 @@ cudaError_t ensure_smem_limit(const void *kernel, size_t bytes);
 
 // Stable LSD radix sort of (64- or 32-bit key, 32-bit value) pairs by key bits
 // [bit_lo, bit_hi) (8 bits per pass); the result is in the alternate buffers when *in_alt.
+// KeyRange (32-bit keys): sort key - base for keys up to base + span, span + 1 for the all-ones
+// key; the sorted keys are these.  The default changes no key.
+struct KeyRange {
+    uint32_t base = 0u, span = 0xFFFFFFFEu;
+};
 size_t sort_temp_bytes(int64_t n);
 cudaError_t radix_sort_pairs(uint64_t *keys, uint64_t *keys_alt, uint32_t *vals, uint32_t *vals_alt, int64_t n,
                              int bit_lo, int bit_hi, void *temp, cudaStream_t st, bool *in_alt);
 cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *keys_alt, uint32_t *vals, uint32_t *vals_alt, int64_t n,
-                             int bit_lo, int bit_hi, void *temp, cudaStream_t st, bool *in_alt);
+                             int bit_lo, int bit_hi, void *temp, cudaStream_t st, bool *in_alt,
+                             KeyRange range = KeyRange{});
 // Sort by key bits [bit_lo, bit_hi) whose values index `payload`, and write the payload in
 // sorted order to payload_out (the last pass gathers; keys and values end up undefined).
 cudaError_t radix_sort_gather(uint32_t *keys, uint32_t *keys_alt, uint32_t *vals, uint32_t *vals_alt, int64_t n,
                               int bit_lo, int bit_hi, void *temp, const float4 *payload, float4 *payload_out,
                               cudaStream_t st);
-// In-place exclusive scan of 32-bit counts whose total stays below 2^32.
+// Exclusive scan of 32-bit counts whose total stays below 2^32, in two parts: entry i is
+// a[i] + temp[i / kScanChunk].  *scan_arrivals(n, temp) must be 0 before.
+constexpr int kScanChunk = 4096;  // entries per CTA
 size_t scan_temp_bytes(int64_t n);
+uint32_t *scan_arrivals(int64_t n, void *temp);
 cudaError_t exclusive_scan_u32(uint32_t *a, int64_t n, void *temp, cudaStream_t st);
 
 // Depth-ordered binning of one view (views[0]): per-particle records and depth keys (with
-// the range of the active keys, and their rebasing to it), the
-// counts in sorted order (cnt has n + 1 entries, the last set to 0), and the expansion
-// into (tile id, slot) pairs at the scanned offsets; k_expand flags kStatOverflow in
-// `status` if a particle's tiles disagree with its count.
+// the range of the active keys), the records and counts in sorted order (cnt has n + 1 entries,
+// the last set to 0; *arrivals is set to 0 for the scan of cnt), and the expansion into pairs
+// (tile id, place in sorted order) at the scanned offsets poff, sums; k_expand flags
+// kStatOverflow in `status` if a particle's tiles disagree with its count.
 cudaError_t launch_depth_records(int storage, const SceneDev &sc, const ViewParams *views, float4 *prec,
                                  uint32_t *dkey, uint32_t *pid, uint32_t *krange, cudaStream_t st);
-cudaError_t launch_rebase_keys(uint32_t *dkey, int64_t n, uint32_t base, uint32_t span, cudaStream_t st);
 cudaError_t launch_sorted_counts(const ViewParams *views, const float4 *prec, const uint32_t *skey,
                                  const uint32_t *spid, int64_t n, uint32_t inactive, float4 *srec, uint32_t *cnt,
-                                 cudaStream_t st);
-cudaError_t launch_expand(const ViewParams *views, const float4 *srec, const uint32_t *poff, int64_t n, int64_t P,
-                          float4 *recs, uint32_t *tkey, uint32_t *tval, int *status, cudaStream_t st);
+                                 uint32_t *arrivals, cudaStream_t st);
+cudaError_t launch_expand(const ViewParams *views, const float4 *srec, const uint32_t *poff, const uint32_t *sums,
+                          int64_t n, int64_t P, uint32_t *tkey, uint32_t *tval, int *status, cudaStream_t st);
 
 // Depth-ordered render: record gather by sorted index and the ordered splat (tiles up to
 // 32 px; squares of up to 16 px, split when T > 16).
