@@ -17,16 +17,16 @@
 // affine map of the records applied so far, I_out = alpha I_in + beta.  Where a square gets
 // several lane pairs, each takes a consecutive part of the list and the maps are composed by
 // shuffles; the map of a pass is composed onto the region's map in shared memory.  A tile that
-// is not split writes beta; the slices of a split tile store their maps, and the last slice to
-// finish composes them far to near.
+// is not split writes beta; the slices of a split tile store their maps, which k_compose_slices
+// composes far to near.
 //
 // What bounds it: the FP32 pipe (69 % of its cycles on the 10 M-particle two-species frame; a
 // step is 168 to 300 packed operations, each two pipe cycles).  Hence the short polynomials, the
 // seven operations per channel (the update in u and 1 / s; eight with a and b apart) and squares
 // of 4 x 4 pixels: 6.7 squares, 107 pixel evaluations per particle, against 235 in the 8 x 8
-// units of a warp per record.  10 M particles at 2048^2: 3.33 -> 1.85 ms, a 1 M-particle map at
-// 1000 x 757: 0.73 -> 0.35 ms.  Batches of 192 (12 warps per SM): 128 on 16 warps took 2.47 ms
-// where 192 took 2.21.
+// units of a warp per record.  10 M particles at 2048^2: 3.33 -> 1.57 ms, a 1 M-particle map at
+// 1000 x 757: 0.73 -> 0.18 ms (with the composition).  Batches of 192 (12 warps per SM): 128 on
+// 16 warps took 2.47 ms where 192 took 2.21.
 #include "splat_batch.cuh"
 
 namespace spl {
@@ -142,7 +142,6 @@ __global__ void __launch_bounds__(kOWarps * 32, 6)
         const int2 ord = __ldg(&fr.order[qs]);  // largest slices first
         const int gt = ord.x, chunk = ord.y, slice = fr.item_off[gt] + chunk;
         const int v = gt / nt, t = gt - v * nt;
-        const int arrivals = (fr.item_off[gt + 1] - fr.item_off[gt]) * S2;
         const int slot = fr.split_slot[gt];
         const float kexp = fr.views[v].kexp;
         const int tx = t % ntx, ty = t / ntx;
@@ -286,8 +285,7 @@ __global__ void __launch_bounds__(kOWarps * 32, 6)
         __syncwarp();
 
         // epilogue: a whole tile writes I = beta (black background), or with map_out the
-        // map (alpha rgb, beta rgb); a slice of a split tile stores its map, and the last
-        // slice composes the tile far to near
+        // map (alpha rgb, beta rgb); a slice of a split tile stores its map
         const int oc = map_out ? 6 : 3;  // floats per pixel
         float *o = out + (int64_t)v * H * W * oc;
         if (slot < 0) {
@@ -298,43 +296,73 @@ __global__ void __launch_bounds__(kOWarps * 32, 6)
             }
         } else {
             float *ms = ord_scratch + (int64_t)slice * 6 * T * T;  // [alpha r g b, beta r g b][T][T]
-            for (int k = lane; k < 6 * kRegion * kRegion; k += 32) {
-                const int c = k / (kRegion * kRegion), r = (k / kRegion) % kRegion, col = k % kRegion;
-                if (r < th && col < tw) ms[c * T * T + (qy + r) * T + qx + col] = map[k];
-            }
-            __threadfence();
-            __syncwarp();
-            int last = 0;
-            if (lane == 0) last = (atomicAdd(&fr.tickets[slot], 1) == arrivals - 1);
-            last = __shfl_sync(0xffffffffu, last, 0);
-            if (last) {
-                __threadfence();
-                const int TW = min(T, W - tx * T), TH = min(T, H - ty * T);
-                const int s0 = fr.item_off[gt], s1 = fr.item_off[gt + 1];
-                float *ot = o + ((int64_t)ty * T * W + (int64_t)tx * T) * oc;
-                for (int k = lane; k < TH * TW * 3; k += 32) {
-                    const int pix3 = k / 3, ch = k - pix3 * 3;
-                    const int rr = pix3 / TW, col = pix3 - rr * TW;
-                    const int pix = rr * T + col;
-                    float A = 1.0f, I = 0.0f;
-                    for (int sl = s0; sl < s1; ++sl) {
-                        const float *m = ord_scratch + (int64_t)sl * 6 * T * T;
-                        const float a = __ldcg(&m[ch * T * T + pix]);
-                        I = fmaf(a, I, __ldcg(&m[(3 + ch) * T * T + pix]));
-                        A *= a;
-                    }
-                    float *p = ot + (int64_t)rr * W * oc + col * oc;
-                    if (map_out) {
-                        p[ch] = A;
-                        p[3 + ch] = I;
-                    } else {
-                        p[ch] = I;
-                    }
+            if (((T | sub) & 3) == 0) {  // rows of the region in fours (past its width: another pixel of it)
+                for (int k = lane; k < 6 * kRegion * kRegion / 4; k += 32) {
+                    const int c = k / (kRegion * kRegion / 4), r = (k / (kRegion / 4)) % kRegion, col = 4 * (k % (kRegion / 4));
+                    if (r < th && col < sub)
+                        *reinterpret_cast<float4 *>(&ms[c * T * T + (qy + r) * T + qx + col]) =
+                            reinterpret_cast<const float4 *>(map)[k];
                 }
-                if (lane == 0) fr.tickets[slot] = 0;
+            } else {
+                for (int k = lane; k < 6 * kRegion * kRegion; k += 32) {
+                    const int c = k / (kRegion * kRegion), r = (k / kRegion) % kRegion, col = k % kRegion;
+                    if (r < th && col < tw) ms[c * T * T + (qy + r) * T + qx + col] = map[k];
+                }
             }
         }
         __syncwarp();
+    }
+}
+
+// k_compose_slices: the maps of a split tile's slices, far to near, one thread per pixel and
+// channel, the maps of several slices on their way together.  A CTA takes 256 pixels and channels
+// of a tile at a time; it collects those of split tiles among every gridDim-th, so that
+// neighbouring crowded tiles go to different CTAs.  Bound by the latency of the loads: 41 us on
+// the 10 M-particle frame at 2048^2 (crowded tiles of some 350 slices), 109 with the loads left to
+// the compiler.  The last warp to finish a tile used to compose it, which held the splat up: 1.90
+// ms, now 1.53 and these 41 us; 4 M particles at 1024^2: 0.89 ms, now 0.40 + 0.09.
+constexpr int kComposeThreads = 256;
+constexpr int kAtOnce = 16;  // slices loaded together
+
+__global__ void __launch_bounds__(kComposeThreads) k_compose_slices(FrameDev fr, const float *__restrict__ slices,
+                                                                    float *__restrict__ out, int map_out) {
+    if (fr.status[kStatOverflow]) return;
+    __shared__ int s_todo[kComposeThreads], s_n;
+    const int T = fr.T, T2 = T * T, W = fr.views[0].W, H = fr.views[0].H, ntx = fr.views[0].ntx;
+    const int oc = map_out ? 6 : 3, parts = (3 * T2 + kComposeThreads - 1) / kComposeThreads;
+    const int count = fr.n_tiles * parts;  // at most 16384 tiles of 12 parts
+    for (int i0 = blockIdx.x; i0 < count; i0 += gridDim.x * kComposeThreads) {
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        const int mine = i0 + threadIdx.x * gridDim.x;
+        if (mine < count && fr.split_slot[mine / parts] >= 0) s_todo[atomicAdd(&s_n, 1)] = mine;
+        __syncthreads();
+        for (int e = 0; e < s_n; ++e) {
+            const int t = s_todo[e] / parts, part = s_todo[e] - t * parts, tx = t % ntx, ty = t / ntx;
+            const int j = part * kComposeThreads + threadIdx.x;
+            const int ch = j / T2, pix = j - ch * T2, r = pix / T, col = pix - r * T;
+            if (ch >= 3 || ty * T + r >= H || tx * T + col >= W) continue;
+            const int s0 = fr.item_off[t], s1 = fr.item_off[t + 1];
+            const float *m = slices + (int64_t)s0 * 6 * T2 + j;
+            float A = 1.0f, I = 0.0f;
+            for (int k = s0; k < s1; k += kAtOnce, m += kAtOnce * 6 * T2) {
+                float a[kAtOnce], b[kAtOnce];
+#pragma unroll
+                for (int g = 0; g < kAtOnce; ++g) {  // past the last slice: the map that changes nothing
+                    a[g] = k + g < s1 ? __ldg(m + g * 6 * T2) : 1.0f;
+                    b[g] = k + g < s1 ? __ldg(m + g * 6 * T2 + 3 * T2) : 0.0f;
+                }
+#pragma unroll
+                for (int g = 0; g < kAtOnce; ++g) {
+                    I = fmaf(a[g], I, b[g]);
+                    A *= a[g];
+                }
+            }
+            float *p = out + ((int64_t)(ty * T + r) * W + tx * T + col) * oc;
+            if (map_out) p[ch] = A, p[3 + ch] = I;
+            else p[ch] = I;
+        }
+        __syncthreads();
     }
 }
 
@@ -396,12 +424,16 @@ cudaError_t launch_compose_maps(const float *maps, int n, int64_t pixels, float 
 }
 
 cudaError_t launch_splat_ordered(const SceneDev &sc, const FrameDev &fr, float *out, const float *absorb,
-                                 float *ord_scratch, int map_out, int grid, cudaStream_t st) {
+                                 float *ord_scratch, int map_out, int grid, int splits, cudaStream_t st) {
     auto fn = sc.emit ? k_splat_ordered<true> : k_splat_ordered<false>;
     cudaError_t err = ensure_smem_limit((const void *)fn, ordered_smem());
     if (err != cudaSuccess) return err;
     if ((err = launch_item_order(fr, st)) != cudaSuccess) return err;
     fn<<<grid, kOWarps * 32, ordered_smem(), st>>>(sc, fr, fr.queue, out, ordered_split(fr.T), absorb, ord_scratch, map_out);
+    if (splits) {
+        const int ctas = std::min(fr.n_tiles * ((3 * fr.T * fr.T + kComposeThreads - 1) / kComposeThreads), 152 * 6);
+        k_compose_slices<<<ctas, kComposeThreads, 0, st>>>(fr, ord_scratch, out, map_out);
+    }
     return cudaGetLastError();
 }
 

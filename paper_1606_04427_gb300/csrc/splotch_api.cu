@@ -791,6 +791,11 @@ static int target_items(int dev, int T) {
     return std::max(1, sm_count(dev) * std::max(1, splat_workers_per_sm()) * 4 / (s * s));
 }
 static const int kMinItemPairs = 2048;
+// Depth-ordered: a record costs several times as much, so that small frames end later with their
+// longest item, and slices are composed in a pass of their own.  1 M particles at 1000 x 757 / 4 M
+// at 1024^2, splat and composition in us: 256 records 185 / 498, 512 179 / 491, 1024 212 / 487,
+// 2048 287 / 520.
+static const int kMinOrderedPairs = 512;
 
 struct RenderSetup {
     int W = 0, H = 0, T = 0, V = 0;
@@ -826,14 +831,14 @@ static splotch_status setup_views(const splotch_camera *cams, int n_views, const
 // Count + scan for all views and read the sizes back (blocking).
 static splotch_status count_and_size(splotch_scene *sc, const RenderSetup &rs, FrameHost &fh, char *fixed,
                                      cudaStream_t st, int64_t sizes[8], cudaEvent_t *ev = nullptr,
-                                     int scan_target = 0) {
+                                     int scan_target = 0, int scan_kmin = kMinItemPairs) {
     FrameDev fr = frame_dev(fh, fixed, nullptr);
     CUDA_TRY(cudaMemcpyAsync(fixed + fh.o_views, rs.views.data(), sizeof(ViewParams) * rs.V,
                              cudaMemcpyHostToDevice, st));
     if (ev) CUDA_TRY(cudaEventRecord(ev[0], st));
     CUDA_TRY(launch_count(sc->storage, sc->dev_view, fr, st));
     if (ev) CUDA_TRY(cudaEventRecord(ev[1], st));
-    CUDA_TRY(launch_scan(fr, scan_target > 0 ? scan_target : target_items(sc->dev, fh.T), kMinItemPairs, st));
+    CUDA_TRY(launch_scan(fr, scan_target > 0 ? scan_target : target_items(sc->dev, fh.T), scan_kmin, st));
     if (ev) CUDA_TRY(cudaEventRecord(ev[2], st));
     int64_t *box = host_box();
     if (!box) return fail(SPLOTCH_ERR_OOM, "pinned host buffer");
@@ -1772,7 +1777,7 @@ extern "C" splotch_status splotch_render_ordered(splotch_scene *sc, const splotc
     char *fixed = (char *)sc->mem.alloc(fh.fixed_bytes, st);
     if (!fixed) return fail(SPLOTCH_ERR_OOM, "frame workspace (%zu bytes)", fh.fixed_bytes);
     int64_t sizes[8];
-    s = count_and_size(sc, rs, fh, fixed, st, sizes, nullptr, target);
+    s = count_and_size(sc, rs, fh, fixed, st, sizes, nullptr, target, kMinOrderedPairs);
     if (s != SPLOTCH_OK) {
         sc->mem.release(fixed, st);
         return s;
@@ -1809,10 +1814,7 @@ extern "C" splotch_status splotch_render_ordered(splotch_scene *sc, const splotc
         sc->mem.release(fixed, st);
         return fail(SPLOTCH_ERR_OOM, "ordered render workspace (%zu + %zu bytes)", fh.var_bytes, cv.off);
     }
-    // the tickets of split tiles (their slices store maps, not sums)
-    cudaError_t e = splits ? cudaMemsetAsync(var + fh.o_tickets, 0, sizeof(int) * (size_t)splits, st) : cudaSuccess;
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ex + o_abs, absorb, sizeof(float) * sc->n_types, cudaMemcpyHostToDevice, st);
+    cudaError_t e = cudaMemcpyAsync(ex + o_abs, absorb, sizeof(float) * sc->n_types, cudaMemcpyHostToDevice, st);
     FrameDev fr = frame_dev(fh, fixed, var);
     // particles in depth order (stable from index order: equal depths keep index order)
     uint32_t *dka = (uint32_t *)(ex + o_dk0), *dkb = (uint32_t *)(ex + o_dk1);
@@ -1860,7 +1862,7 @@ extern "C" splotch_status splotch_render_ordered(splotch_scene *sc, const splotc
                                                                 (squares + per_cta - 1) / per_cta));
     if (e == cudaSuccess)
         e = launch_splat_ordered(sc->dev_view, fr, out, (const float *)(ex + o_abs),
-                                 (float *)(ex + o_map), (rs.pr.flags & SPLOTCH_OUT_MAP) ? 1 : 0, grid, st);
+                                 (float *)(ex + o_map), (rs.pr.flags & SPLOTCH_OUT_MAP) ? 1 : 0, grid, splits, st);
     int stat[4] = {0, 0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(stat, fixed + fh.o_status, sizeof(stat), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

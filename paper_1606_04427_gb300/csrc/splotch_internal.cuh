@@ -468,7 +468,7 @@ int ordered_workers_per_sm();
 // fr.order is null).
 cudaError_t launch_item_order(const FrameDev &fr, cudaStream_t st);
 cudaError_t launch_splat_ordered(const SceneDev &sc, const FrameDev &fr, float *out, const float *absorb,
-                                 float *ord_scratch, int map_out, int grid, cudaStream_t st);
+                                 float *ord_scratch, int map_out, int grid, int splits, cudaStream_t st);
 cudaError_t launch_selftest_wait(long long limit, int *result, cudaStream_t st);
 cudaError_t launch_final(float *a, int64_t count, cudaStream_t st);
 cudaError_t launch_compose_maps(const float *maps, int n, int64_t pixels, float *out, cudaStream_t st);

@@ -42,3 +42,24 @@ def test_ordered_binning_edges_match_the_oracle(n, depth):
     for T in (8, 16, 32):
         got = sc.render_ordered(cam, [1.0], render.RenderParams(tile=T)).cpu().numpy()
         np.testing.assert_allclose(got, want, rtol=rtol, atol=1e-12, err_msg=f"T={T}")
+
+
+@pytest.mark.parametrize("n", [513, 8192, 9001])  # 2, 16 and 18 slices of the tile at (16, 16)
+@pytest.mark.parametrize("T", [16, 20, 24, 32])
+def test_slices_of_a_crowded_tile_compose_far_to_near(n, T):
+    rng = np.random.default_rng(n)
+    z = rng.uniform(0.49, 0.51, n)
+    s = (2.5 - z) / P.focal(H)
+    px, py, R = rng.uniform(18.0, 30.0, n), rng.uniform(18.0, 30.0, n), rng.uniform(0.8, 5.0, n)
+    ps = P.make_set(0.5 + (px - 0.5 * W) * s, 0.5 - (py - 0.5 * H) * s, z, R / 0.75 * s,
+                    rng.uniform(0.0, 1.0, n), beta=0.01)
+    cam = P.front(W, H)
+    want = oracle.render_rt_depth(ps, cam, [1.0])
+    rtol = 4e-6 * (1.0 + oracle.render(ps, cam).max()) + n * (3 * 2.0 ** -24 + 1.2e-7)
+    sc = render.Scene(ps, "f32")
+    got = sc.render_ordered(cam, [1.0], render.RenderParams(tile=T)).cpu().numpy()
+    np.testing.assert_allclose(got, want, rtol=rtol, atol=1e-12)
+    maps = sc.render_ordered(cam, [1.0], render.RenderParams(tile=T, map=True)).cpu().numpy()
+    np.testing.assert_array_equal(maps[..., 3:], got)
+    # with absorption equal to emission, I = 1 - alpha
+    np.testing.assert_allclose(1.0 - maps[..., :3], want, rtol=rtol, atol=n * 2.0 ** -23)
