@@ -156,7 +156,7 @@ typedef struct {
  *                 splotch_last_timing; SPLOTCH_STABLE: build every tile list in ascending
  *                 particle index (Section 3.2.1 fills each thread's index vectors by walking
  *                 its particles in order), which makes the image bitwise reproducible; the
- *                 binning takes about three times as long.  Without it a list holds the
+ *                 scatter takes about three and a half times as long.  Without it a list holds the
  *                 same members, each chunk's in the order its warps reached them, and two
  *                 renders may differ by the FP32 rounding of a pixel's sum in another order
  *                 (at most 2 (n - 1) 2^-24 of the sum, n its contributions). */
@@ -225,9 +225,9 @@ splotch_status splotch_render(splotch_scene *scene, const splotch_camera *cams, 
  * depth slabs (cameras with consecutive near / far planes) compose far to near into the
  * whole frame.  Particles at exactly equal depth are applied in index order.  Tiles up
  * to 32 px (larger: UNSUPPORTED); other output flags are ignored.  The particles are sorted by
- * depth (stable radix sort from index order), their records written out in that order and
- * grouped by a stable sort on tile id; device memory besides the tile lists: about 52
- * bytes per particle and 32 per particle-tile pair.  Synchronous.  Errors: INVALID_ARG,
+ * depth (stable radix sort from index order) and their tile entries, written out in that
+ * order, grouped by a stable sort on tile id; device memory besides the tile lists: about 52
+ * bytes per particle, 16 per particle-tile pair and 24 T^2 per slice of a tile list.  Synchronous.  Errors: INVALID_ARG,
  * UNSUPPORTED, OOM, CUDA, TIMEOUT. */
 splotch_status splotch_render_ordered(splotch_scene *scene, const splotch_camera *cam,
                                       const splotch_render_params *params, const float *absorb, float *out,
