@@ -1,10 +1,10 @@
-// Stable LSD radix sort of (64-bit key, 32-bit value) pairs on the device.
+// Stable LSD radix sort of (32- or 64-bit key, 32-bit value) pairs on the device.
 //
 // The depth-ordered render (Section 2.1: with absorption different from emission the
 // transfer equation must be applied along each line of sight in order) needs every tile
-// list in depth order.  Records carry the key (tile << 32) | depth key; sorting the depth
-// bits and then the tile bits, each pass stable, gives tile-major, far-to-near order (a
-// first sort by particle index makes equal depths keep index order).
+// list in depth order.  It sorts the particles by a 32-bit depth key, from index order (so
+// equal depths keep it), and then their (tile, place in depth order) pairs by tile: each pass
+// is stable, so the lists are tile-major and far to near.
 //
 // One pass over 8 key bits:
 //   k_digit_hist   each CTA counts the digits of its 4096 elements (shared counters per warp),

@@ -1756,8 +1756,9 @@ extern "C" splotch_status splotch_debug_sort(void *keys, int32_t key_bytes, uint
 // Depth-ordered render (absorption != emission).  Section 2.1 solves the radiative-transfer
 // equation along each line of sight; with absorption A = s_t x emission per species the
 // particles' updates do not commute, so every tile list is put in depth order (farthest
-// first) before the splat: the scatter writes a (tile, depth) key per record, a stable
-// radix sort orders the keys, and the records are gathered in that order.
+// first) before the splat: the particles are sorted by depth, each writes its place in that
+// order once per tile it meets, a stable radix sort groups the places by tile, and its last
+// pass gathers the records.
 extern "C" splotch_status splotch_render_ordered(splotch_scene *sc, const splotch_camera *cam,
                                                  const splotch_render_params *params, const float *absorb,
                                                  float *out, void *stream) {
