@@ -66,8 +66,10 @@ __device__ __forceinline__ float pixel(float held, float a, int mode) {
 
 constexpr int kWarps = 8;    // per CTA: the largest team
 constexpr int kBatch = 192;  // records per batch
-constexpr int kFew = 64;     // records up to which a lone warp's item takes render_few; a
-                             // team's part: half of that
+// Records up to which an item that one warp renders takes render_few; the part of a warp in an
+// item that its team shares: half of that.  (Whether the warp's team is still together does not
+// count: which team meets an item changes from run to run, the sums must not.)
+constexpr int kFew = 64;
 
 // Warps per team, from the frame's `records` (times the regions per tile edge: a region reads its
 // tile's whole list and keeps a part of it), items of at most K records and `warps` warps.  A warp alone has the least overhead per
@@ -397,17 +399,18 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
         if (nrec) nrec = (int)(min(seg1, e0 + K) - e0);
         if (nrec == 0 && out_accum == 2 && kn.team == 1 && fr.split_slot[gt] < 0) continue;  // adds nothing
         const float4 *recs = fr.lists + e0;
+        int few = kFew;
         if (kn.team > 1) {
-            int part = ((nrec + kn.team - 1) / kn.team + 31) & ~31;
-            if (order_bin(nrec, (int)K) < shared_from(kn.team)) {  // the first warp's alone
-                part = nrec;
-                if (fr.order) {  // and so are all later items: the team parts
-                    if (lane == 0) s_known[threadIdx.x >> 5].team = 1;
-                    __syncwarp();
-                    if (me >= 32) {
-                        if (lane == 0) next = atomicAdd(queue, 1);
-                        continue;
-                    }
+            int part = nrec;  // the first warp's alone
+            if (order_bin(nrec, (int)K) >= shared_from(kn.team)) {
+                part = ((nrec + kn.team - 1) / kn.team + 31) & ~31;
+                few = kFew / 2;
+            } else if (fr.order) {  // all later items are a warp's alone as well: the team parts
+                if (lane == 0) s_known[threadIdx.x >> 5].team = 1;
+                __syncwarp();
+                if (me >= 32) {
+                    if (lane == 0) next = atomicAdd(queue, 1);
+                    continue;
                 }
             }
             // this warp's consecutive part of the slice
@@ -416,7 +419,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
             nrec = min(part, nrec - first);
         }
 
-        if (nrec <= (kn.team == 1 ? kFew : kFew / 2)) {
+        if (nrec <= few) {
             render_few<kViewScale, kEmit>(sc, fr, ws, rg, recs, nrec, v, kexp);
             nrec = 0;
         } else {
