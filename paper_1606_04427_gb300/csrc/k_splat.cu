@@ -396,13 +396,15 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
         }
         const int64_t seg1 = fr.offsets[gt + 1];
         const int64_t e0 = fr.offsets[gt] + (int64_t)chunk * K;
-        if (nrec) nrec = (int)(min(seg1, e0 + K) - e0);
+        const int len = (int)(min(seg1, e0 + K) - e0);
+        if (nrec) nrec = len;
         if (nrec == 0 && out_accum == 2 && kn.team == 1 && fr.split_slot[gt] < 0) continue;  // adds nothing
         const float4 *recs = fr.lists + e0;
         int few = kFew;
         if (kn.team > 1) {
             int part = nrec;  // the first warp's alone
-            if (order_bin(nrec, (int)K) >= shared_from(kn.team)) {
+            // by the slice's length: that of the order, also where the region has no pixel
+            if (order_bin(len, (int)K) >= shared_from(kn.team)) {
                 part = ((nrec + kn.team - 1) / kn.team + 31) & ~31;
                 few = kFew / 2;
             } else if (fr.order) {  // all later items are a warp's alone as well: the team parts

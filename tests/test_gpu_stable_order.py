@@ -55,3 +55,20 @@ def test_short_items_do_not_depend_on_when_a_team_parts():
     for _ in range(20):
         assert torch.equal(sc.render(cam, p), want)
         assert torch.equal(sc.render_noalloc(cam, torch.empty_like(want), p), want)
+
+
+@pytest.mark.parametrize("T,W,H", [(24, 490, 480), (32, 1000, 520), (40, 1010, 1000)])
+def test_regions_off_the_image_do_not_part_teams(T, W, H):
+    """Tiles above 16 pixels are rendered as regions of up to 16; those of the last column and row
+    can lie wholly off a ragged image.  Every tile's list is long, so every other region is a
+    team's, in any order."""
+    rng = np.random.default_rng(T)
+    nt = -(-W // T) * -(-H // T)
+    assert -(-W // T) * T - W >= -(-T // -(-T // 16))  # a column of regions has no pixel
+    px, py = _tiles(W, H, T, rng.integers(500, 900, nt), 0.05, rng)
+    sc = _scene(W, H, px, py, rng.uniform(0.8, 3.0, px.size), 5)
+    cam = P.front(W, H)
+    p = render.RenderParams(tile=T, accum=True, stable=True)
+    want = sc.render(cam, p)
+    for _ in range(20):
+        assert torch.equal(sc.render(cam, p), want)
