@@ -20,13 +20,12 @@
 // is not split writes beta; the slices of a split tile store their maps, which k_compose_slices
 // composes far to near.
 //
-// What bounds it: the FP32 pipe (69 % of its cycles on the 10 M-particle two-species frame; a
-// step is 168 to 300 packed operations, each two pipe cycles).  Hence the short polynomials, the
-// seven operations per channel (the update in u and 1 / s; eight with a and b apart) and squares
-// of 4 x 4 pixels: 6.7 squares, 107 pixel evaluations per particle, against 235 in the 8 x 8
-// units of a warp per record.  10 M particles at 2048^2: 3.33 -> 1.57 ms, a 1 M-particle map at
-// 1000 x 757: 0.73 -> 0.18 ms (with the composition).  Batches of 192 (12 warps per SM): 128 on
-// 16 warps took 2.47 ms where 192 took 2.21.
+// What bounds it: the FP32 pipe.  Hence the short polynomials (8 to 10 packed operations per channel
+// and two pixels, 15 with the exponential) and squares of 4 x 4 pixels: 6.7 squares, 107 pixel
+// evaluations per particle, against 235 in the 8 x 8 units of a warp per record.  10 M particles at
+// 2048^2: frame 4.97 ms with a warp per record, 3.22 now (3.03 with the cheaper and less accurate
+// update that apply_record's comment names); a 1 M-particle map at 1000 x 757: 1.21 -> 0.58 ms
+// (0.54).  Batches of 192 (12 warps per SM): 128 on 16 warps took 2.47 ms where 192 took 2.21.
 #include "splat_batch.cuh"
 
 namespace spl {
@@ -35,47 +34,54 @@ constexpr int kOWarps = 2;    // warps per CTA
 constexpr int kOBatch = 192;  // records per batch
 
 struct __align__(16) OWarpSmem {
-    Batch<kOBatch> batch;            // pb: absorption A = s E per channel, and 1 / s
+    Batch<kOBatch> batch;            // pb: emission E per channel, and s
     float map[6][kRegion][kRegion];  // the region's map: alpha r, g, b, beta r, g, b
 };
 
-// Update of one record with x = s E w per pixel and channel and u = 1 - exp(-x):
-//     alpha <- alpha - u alpha,   beta <- beta + u (1 / s - beta),   u = x phi(x).
-// phi(x) = (1 - exp(-x)) / x is a polynomial whose degree follows the step's largest x (w <= 1,
-// so a record's x is at most its s E): degree 2 up to kDeg2Max and degree 3 up to kDeg3Max,
-// minimax with phi(0) = 1 (fitted here by iteratively reweighted least squares against expm1 in
-// 64 bits; largest relative errors 1.02e-7 and 1.19e-7).  Beyond, and for negative emissions,
-// the Taylor polynomial of degree 5 where |x| <= kTaylorMax (next term x^6 / 7! <= 5e-8) and
-// 1 - exp(-x) itself elsewhere, where the subtraction loses two bits at most.
-constexpr float kDeg2Max = 0.04f, kDeg3Max = 0.2f, kTaylorMax = 0.25f;
+// Update of one record with e = E w, x = s e and phi(x) = (1 - exp(-x)) / x per pixel and channel:
+//     alpha <- alpha - x phi alpha,   beta <- beta + phi (e - x beta),
+// which needs no 1 / s: a species with s = 0 has x = 0, phi = 1, and a pixel of few records has as
+// few roundings as e phi itself.  (With u = x phi and beta <- beta + u (1 / s - beta), an operation
+// less and polynomials a degree shorter, the errors of u, 1 / s and phi reached beta: 1.0e-7 instead
+// of 4e-8 RMS on pixels of one to three records, with a bias of 5e-8 to 9e-8; and 1 / s overflowed
+// where s = 0 stood for 2^-40 / E.  Emulated against 64 bits for 1 to 200 records, x from 0.001 to 2,
+// the present form is nowhere less accurate than a beta + b with a and b rounded apart.)
+// phi is a polynomial whose degree follows the step's largest x (w <= 1, so a record's x is at most
+// its s E): degree 2 up to kDeg2Max, 3 up to kDeg3Max, 4 up to kDeg4Max, minimax with phi(0) = 1
+// (fitted here by iteratively reweighted least squares against expm1 in 64 bits; largest relative
+// errors 5.4e-9, 8.0e-9 and 3.0e-9).  Beyond, and for negative emissions, the Taylor polynomial of
+// degree 5 where |x| <= kDeg4Max (next term x^6 / 7! <= 5e-8) and the exponential itself elsewhere:
+// alpha <- a alpha, beta <- a beta + (1 - a) / s, a = exp(-x).
+constexpr float kDeg2Max = 0.015f, kDeg3Max = 0.1f, kDeg4Max = 0.25f;
 
-// Species that do not absorb (or hardly) use s raised to kLeastX / max E: alpha stays 1 in FP32
-// and u / s = E w to FP32 rounding.
-constexpr float kLeastX = 9.094947e-13f;  // 2^-40
-
-template <int kDeg> __device__ __forceinline__ float2 absorbed(float2 x) {  // u of degree kDeg (5: Taylor)
+// phi as a polynomial in -x (all coefficients positive)
+template <int kDeg> __device__ __forceinline__ float2 phi_of(float2 nx) {  // kDeg 5: Taylor
     float2 phi;
     if (kDeg == 5) {
-        phi = __ffma2_rn(x, f2(-1.0f / 720.0f), f2(1.0f / 120.0f));
-        phi = __ffma2_rn(x, phi, f2(-1.0f / 24.0f));
-        phi = __ffma2_rn(x, phi, f2(1.0f / 6.0f));
-        phi = __ffma2_rn(x, phi, f2(-0.5f));
+        phi = __ffma2_rn(nx, f2(1.0f / 720.0f), f2(1.0f / 120.0f));
+        phi = __ffma2_rn(nx, phi, f2(1.0f / 24.0f));
+        phi = __ffma2_rn(nx, phi, f2(1.0f / 6.0f));
+        phi = __ffma2_rn(nx, phi, f2(0.5f));
+    } else if (kDeg == 4) {
+        phi = __ffma2_rn(nx, f2(0.00753017422f), f2(0.0415001325f));
+        phi = __ffma2_rn(nx, phi, f2(0.166652888f));
+        phi = __ffma2_rn(nx, phi, f2(0.499999642f));
     } else if (kDeg == 3) {
-        phi = __ffma2_rn(x, f2(-0.03859227f), f2(0.16631325f));
-        phi = __ffma2_rn(x, phi, f2(-0.49998832f));
+        phi = __ffma2_rn(nx, f2(0.0400981233f), f2(0.166576117f));
+        phi = __ffma2_rn(nx, phi, f2(0.49999851f));
     } else {
-        phi = __ffma2_rn(x, f2(0.16436407f), f2(-0.49997154f));
+        phi = __ffma2_rn(nx, f2(0.165799007f), f2(0.499995977f));
     }
-    phi = __ffma2_rn(x, phi, f2(1.0f));
-    return __fmul2_rn(x, phi);
+    return __ffma2_rn(nx, phi, f2(1.0f));
 }
 
-// One step of a pass: every lane applies its record to its 2 x 4 pixels.  kDeg 5: the
-// exponential where x is beyond kTaylorMax.
+// One step of a pass: every lane applies its record (pb: E r, g, b and s) to its 2 x 4 pixels.
+// kDeg 5: the exponential where x is beyond kDeg4Max.
 template <int kDeg>
 __device__ __forceinline__ void apply_record(const float4 &pa, const float4 &pb, const float2 (&fx)[2], const float2 &fy,
                                              float2 (&al)[3][2][2], float2 (&be)[3][2][2]) {
-    const float kx[3] = {pb.x, pb.y, pb.z};
+    const float E[3] = {pb.x, pb.y, pb.z};
+    const float inv_s = kDeg == 5 ? 1.0f / pb.w : 0.0f;
     const float2 dx[2] = {__fadd2_rn(fx[0], f2(pa.x)), __fadd2_rn(fx[1], f2(pa.x))};
     const float2 dy = __fadd2_rn(fy, f2(pa.y));
     const float2 qx[2] = {__fmul2_rn(dx[0], dx[0]), __fmul2_rn(dx[1], dx[1])};
@@ -87,22 +93,23 @@ __device__ __forceinline__ void apply_record(const float4 &pa, const float4 &pb,
         for (int cp = 0; cp < 2; ++cp) {
             const float2 d2 = __fadd2_rn(qx[cp], qr);
             const float2 g = __fmul2_rn(d2, f2(pa.w));
-            // uncovered: u = 0
+            // uncovered: e = x = 0
             const float2 w = make_float2(d2.x < pa.z ? ex2_fast(g.x) : 0.0f, d2.y < pa.z ? ex2_fast(g.y) : 0.0f);
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) {
-                const float2 x = __fmul2_rn(f2(kx[ch]), w);
-                float2 u = absorbed<kDeg>(x);
+                float2 &A = al[ch][row][cp], &B = be[ch][row][cp];
+                const float2 e = __fmul2_rn(f2(E[ch]), w), nx = __fmul2_rn(f2(-pb.w), e), phi = phi_of<kDeg>(nx);
+                float2 an = __ffma2_rn(__fmul2_rn(nx, phi), A, A);
+                float2 bn = __ffma2_rn(phi, __ffma2_rn(nx, B, e), B);
                 if (kDeg == 5) {
-                    const float2 y = __fmul2_rn(x, f2(-kLog2e));
-                    const float2 v = __fadd2_rn(f2(1.0f), make_float2(-ex2_fast(y.x), -ex2_fast(y.y)));
-                    u.x = fabsf(x.x) > kTaylorMax ? v.x : u.x;
-                    u.y = fabsf(x.y) > kTaylorMax ? v.y : u.y;
+                    const float2 y = __fmul2_rn(nx, f2(kLog2e));
+                    const float2 a = make_float2(ex2_fast(y.x), ex2_fast(y.y));
+                    const float2 fa = __fmul2_rn(a, A);
+                    const float2 fb = __ffma2_rn(a, B, __ffma2_rn(a, f2(-inv_s), f2(inv_s)));
+                    if (fabsf(nx.x) > kDeg4Max) an.x = fa.x, bn.x = fb.x;
+                    if (fabsf(nx.y) > kDeg4Max) an.y = fa.y, bn.y = fb.y;
                 }
-                const float2 nu = make_float2(-u.x, -u.y);
-                al[ch][row][cp] = __ffma2_rn(nu, al[ch][row][cp], al[ch][row][cp]);
-                const float2 t = __fadd2_rn(f2(pb.w), make_float2(-be[ch][row][cp].x, -be[ch][row][cp].y));
-                be[ch][row][cp] = __ffma2_rn(u, t, be[ch][row][cp]);
+                A = an, B = bn;
             }
         }
     }
@@ -198,10 +205,8 @@ __global__ void __launch_bounds__(kOWarps * 32, 6)
                     const int j = g * 32 + lane;
                     if (j >= nbuf) break;
                     const float R2 = __fmul_rn(rec[g].z, rec[g].z);
-                    const float emax = fmaxf(fabsf(e[g].x), fmaxf(fabsf(e[g].y), fabsf(e[g].z)));
-                    const float sa = emax > 0.0f ? fmaxf(s[g], kLeastX / emax) : 1.0f;
                     bt->pa[j] = make_float4(-rec[g].x, -rec[g].y, R2, gauss_scale(kexp, R2));
-                    bt->pb[j] = make_float4(sa * e[g].x, sa * e[g].y, sa * e[g].z, 1.0f / sa);
+                    bt->pb[j] = make_float4(e[g].x, e[g].y, e[g].z, s[g]);
                 }
             }
             int before, total;
@@ -237,12 +242,16 @@ __global__ void __launch_bounds__(kOWarps * 32, 6)
                     const float4 pb = bt->pb[idx];
                     ++lp;
                     idx = k < mine ? *lp : kOBatch;
-                    // as unsigned integers, so that a negative emission counts as the largest
-                    const uint32_t xmax = max(__float_as_uint(pb.x), max(__float_as_uint(pb.y), __float_as_uint(pb.z)));
+                    // the largest x; compared as unsigned integers, so that a negative one counts as
+                    // the largest
+                    const uint32_t emax = max(__float_as_uint(pb.x), max(__float_as_uint(pb.y), __float_as_uint(pb.z)));
+                    const uint32_t xmax = __float_as_uint(__uint_as_float(emax) * pb.w);
                     if (!__any_sync(0xffffffffu, xmax > __float_as_uint(kDeg2Max)))
                         apply_record<2>(pa, pb, fx, fy, al, be);
                     else if (!__any_sync(0xffffffffu, xmax > __float_as_uint(kDeg3Max)))
                         apply_record<3>(pa, pb, fx, fy, al, be);
+                    else if (!__any_sync(0xffffffffu, xmax > __float_as_uint(kDeg4Max)))
+                        apply_record<4>(pa, pb, fx, fy, al, be);
                     else
                         apply_record<5>(pa, pb, fx, fy, al, be);
                 }
