@@ -257,6 +257,35 @@ __device__ __forceinline__ void add_record(float4 pa, float4 pb, float2 fx0, flo
     }
 }
 
+// Records of the batch whose emission is not finite (brightness, colour and view scale are, their
+// product need not be) are added to the accumulator one by one, at the pixels they cover only:
+// add_record adds emission x 0 where a record covers nothing, which would not be 0.  Their emission
+// in the batch becomes 0.  Rare, so out of line and without regard to speed.
+__device__ __noinline__ void add_wild(WarpSmem *ws, int nbuf, int px0, int py0) {
+    const int lane = threadIdx.x & 31, x = lane & 15, y0 = 8 * (lane >> 4);
+    const float fx = (float)(px0 + x) + 0.5f;
+    for (int j = 0; j < nbuf; ++j) {
+        const float4 pa = ws->batch.pa[j], pb = ws->batch.pb[j];
+        if (isfinite(pb.x) && isfinite(pb.y) && isfinite(pb.z)) continue;
+        const float dx = __fadd_rn(fx, pa.x);
+        for (int y = y0; y < y0 + 8; ++y) {
+            const float dy = __fadd_rn((float)(py0 + y) + 0.5f, pa.y);
+            const float d2 = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
+            if (!(d2 < pa.z)) continue;
+            const float w = ex2_fast(__fmul_rn(d2, pa.w));
+            ws->acc[0][y][x] += pb.x * w;
+            ws->acc[1][y][x] += pb.y * w;
+            ws->acc[2][y][x] += pb.z * w;
+        }
+        __syncwarp();
+        if (lane == 0) ws->batch.pb[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+    __syncwarp();
+}
+
+// Finite unless a component is not (or the sum leaves the range: add_wild looks again).
+__device__ __forceinline__ float magnitude(float x, float y, float z) { return fabsf(x) + fabsf(y) + fabsf(z); }
+
 // An item of few records, into the accumulator: 32 records at a time are decoded, one per lane,
 // and evaluated one after another by the whole warp, 2 x 4 pixels per lane.  Batches, lists and
 // sorted squares cost an item about 15 us of a warp's time whatever it holds, nearly all of it
@@ -276,6 +305,7 @@ __device__ __forceinline__ void render_few(const SceneDev &sc, const FrameDev &f
     for (int c = 0; c < 3; ++c)
 #pragma unroll
         for (int k = 0; k < 4; ++k) s[c][k >> 1][k & 1] = f2(0.0f);
+    bool wild = false;  // add_wild has added to the accumulator
     for (int base = 0; base < nrec; base += 32) {
         const float4 rec[1] = {__ldcs(&recs[min(base + lane, nrec - 1)])};
         const bool live = base + lane < nrec && fmaxf(fabsf(rec[0].x - rg.xc), fabsf(rec[0].y - rg.yc)) <
@@ -300,6 +330,14 @@ __device__ __forceinline__ void render_few(const SceneDev &sc, const FrameDev &f
         }
         __syncwarp();
         const int n = __popc(bal);
+        if (kViewScale ? __any_sync(0xffffffffu, live && !isfinite(magnitude(e[0].x * vs, e[0].y * vs, e[0].z * vs)))
+                       : sc.wild) {
+            if (!wild)
+                for (int k = lane; k < 3 * kRegion * kRegion; k += 32) (&ws->acc[0][0][0])[k] = 0.0f;
+            wild = true;
+            __syncwarp();
+            add_wild(ws, n, rg.px0, rg.py0);
+        }
 #pragma unroll 2
         for (int j = 0; j < n; ++j) {
             const float4 pa = bt->pa[j], pb = bt->pb[j];
@@ -310,9 +348,12 @@ __device__ __forceinline__ void render_few(const SceneDev &sc, const FrameDev &f
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int row = 0; row < 2; ++row)
-            *reinterpret_cast<float4 *>(&ws->acc[c][y + row][x]) =
-                make_float4(s[c][row][0].x, s[c][row][0].y, s[c][row][1].x, s[c][row][1].y);
+        for (int row = 0; row < 2; ++row) {
+            float4 *p = reinterpret_cast<float4 *>(&ws->acc[c][y + row][x]);
+            float4 u = make_float4(s[c][row][0].x, s[c][row][0].y, s[c][row][1].x, s[c][row][1].y);
+            if (wild) u.x += p->x, u.y += p->y, u.z += p->z, u.w += p->w;
+            *p = u;
+        }
 }
 
 // kViewScale: multiply every record's emission by a per-view, per-species scale (plans
@@ -441,6 +482,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
             // repeat the last record
             uint32_t word[Batch<kBatch>::kWords];
             int cnt;
+            float most = 0.0f;  // kViewScale: finite if the lane's emissions are
             {
                 float4 rec[kRounds];
 #pragma unroll
@@ -477,7 +519,12 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
                     bt->pa[j] = make_float4(-rec[g].x, -rec[g].y, R2, gauss_scale(kexp, R2));
                     if constexpr (kViewScale || !kEmit)
                         bt->pb[j] = make_float4(e[g].x * vs[g], e[g].y * vs[g], e[g].z * vs[g], 0.0f);
+                    if constexpr (kViewScale) most += magnitude(e[g].x * vs[g], e[g].y * vs[g], e[g].z * vs[g]);
                 }
+            }
+            if (kViewScale ? __any_sync(0xffffffffu, !isfinite(most)) : sc.wild) {
+                __syncwarp();
+                add_wild(ws, nbuf, rg.px0, rg.py0);
             }
 
             // ---- 3. per square, the batch positions of its records; squares longest list first

@@ -379,10 +379,14 @@ static splotch_status create_scene_impl(const splotch_scene_desc *d, splotch_sce
         total += d->cmap_len[t];
     }
     std::vector<float> lut(4 * (size_t)total);
+    bool wild = false;  // entries so large that interpolating them may leave the FP32 range
     for (int t = 0; t < d->n_types; ++t)
         for (int k = 0; k < d->cmap_len[t]; ++k) {
-            for (int c = 0; c < 3; ++c)
-                lut[4 * (lut_off[t] + k) + c] = d->brightness[t] * d->cmap_rgb[t][3 * k + c];
+            for (int c = 0; c < 3; ++c) {
+                const float e = d->brightness[t] * d->cmap_rgb[t][3 * k + c];
+                lut[4 * (lut_off[t] + k) + c] = e;
+                wild |= !(std::fabs(e) <= 1e38f);
+            }
             lut[4 * (lut_off[t] + k) + 3] = 0.0f;
         }
     Carve cv;
@@ -511,6 +515,7 @@ static splotch_status create_scene_impl(const splotch_scene_desc *d, splotch_sce
     v.lut = (const float4 *)(mb + o_lut);
     v.lut_off = (const int *)(mb + o_off);
     v.lut_len = (const int *)(mb + o_len);
+    v.wild = wild;
     bool any_vec = false;
     for (int t = 0; d->col_vector && t < d->n_types; ++t) any_vec |= d->col_vector[t] != 0;
     if (any_vec) {

@@ -61,6 +61,7 @@ struct SceneDev {
     const float4 *emit;              // [n] {r, g, b, species bits}: per-particle emission
                                      // (vector colour scenes; records then carry particle
                                      // indices), or null
+    int wild;                        // an emission may not be finite (brightness times a colour)
 };
 
 // Per-frame buffers (one frame = V views).
