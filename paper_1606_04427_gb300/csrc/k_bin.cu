@@ -321,7 +321,8 @@ __global__ void __launch_bounds__(kThreads) k_count(SceneDev sc, FrameDev fr) {
     const int nt = fr.n_tiles;
     for (int k = threadIdx.x; k < g_n * nt; k += blockDim.x) s_hist[k] = 0;
     if (threadIdx.x < g_n) s_view[threadIdx.x] = fr.views[v0 + threadIdx.x];
-    // the frame's first kernel clears what the later ones count into
+    // the frame's first kernel clears what the later ones count into (each of its launches does,
+    // before any of those)
     if (b == 0 && blockIdx.y == 0) {
         for (int k = threadIdx.x; k < 2 * kOrderBins; k += blockDim.x) fr.bins[k] = 0;
         if (threadIdx.x < 4) fr.status[threadIdx.x] = 0, fr.queue[threadIdx.x] = 0;
@@ -360,13 +361,29 @@ __global__ void __launch_bounds__(kThreads) k_count(SceneDev sc, FrameDev fr) {
     }
 }
 
+// f on the frame's views, at most `most` at a time: a grid's second dimension, over views or groups
+// of views, ends at 65535.
+constexpr int64_t kGridY = 65535;
+template <class F> static cudaError_t by_views(const FrameDev &fr, int64_t most, F f) {
+    for (int64_t v0 = 0; v0 < fr.V; v0 += most) {
+        FrameDev part = fr;
+        part.V = (int)std::min<int64_t>(most, fr.V - v0);
+        part.views = fr.views + v0;
+        part.rel = fr.rel + v0 * fr.n_chunks * fr.n_tiles;
+        part.counts = fr.counts + v0 * fr.n_tiles;
+        part.offsets = fr.offsets + v0 * fr.n_tiles;
+        f(part);
+    }
+    return cudaGetLastError();
+}
+
 template <int S> static cudaError_t count_impl(const SceneDev &sc, const FrameDev &fr, cudaStream_t st) {
     const size_t smem = (size_t)fr.G * fr.n_tiles * sizeof(int);
     cudaError_t err = ensure_smem_limit((const void *)k_count<S>, kBinSmemMax);
     if (err != cudaSuccess) return err;
-    dim3 grid(fr.n_chunks, (fr.V + fr.G - 1) / fr.G);
-    k_count<S><<<grid, kThreads, smem, st>>>(sc, fr);
-    return cudaGetLastError();
+    return by_views(fr, kGridY * fr.G, [&](const FrameDev &part) {
+        k_count<S><<<dim3(part.n_chunks, (part.V + part.G - 1) / part.G), kThreads, smem, st>>>(sc, part);
+    });
 }
 
 cudaError_t launch_count(int storage, const SceneDev &sc, const FrameDev &fr, cudaStream_t st) {
@@ -597,13 +614,9 @@ __global__ void __launch_bounds__(1024) k_scan(FrameDev fr, int target_items, in
 
 cudaError_t launch_scan(const FrameDev &fr, int target_items, int kmin, cudaStream_t st) {
     const int64_t N = (int64_t)fr.V * fr.n_tiles;
-    for (int v0 = 0; v0 < fr.V; v0 += 65535) {  // the grid's second dimension holds 65535 views
-        FrameDev part = fr;
-        part.V = std::min(65535, fr.V - v0);
-        part.rel = fr.rel + (int64_t)v0 * fr.n_chunks * fr.n_tiles;
-        part.counts = fr.counts + (int64_t)v0 * fr.n_tiles;
-        k_chunk_scan<<<dim3((fr.n_tiles + 31) / 32, part.V), 32 * kChunkSegs, 0, st>>>(part);
-    }
+    by_views(fr, kGridY, [&](const FrameDev &part) {
+        k_chunk_scan<<<dim3((part.n_tiles + 31) / 32, part.V), 32 * kChunkSegs, 0, st>>>(part);
+    });
     k_scan<<<(int)((N + kScanTiles - 1) / kScanTiles), 1024, 0, st>>>(fr, target_items, kmin);
     return cudaGetLastError();
 }
@@ -752,9 +765,9 @@ template <int S> static cudaError_t scatter_impl(const SceneDev &sc, const Frame
     cudaError_t err =
         ensure_smem_limit((const void *)k_scatter<S>, kBinSmemMax);
     if (err != cudaSuccess) return err;
-    dim3 grid(fr.n_chunks, (fr.V + fr.G - 1) / fr.G);
-    k_scatter<S><<<grid, kThreads, smem, st>>>(sc, fr);
-    return cudaGetLastError();
+    return by_views(fr, kGridY * fr.G, [&](const FrameDev &part) {
+        k_scatter<S><<<dim3(part.n_chunks, (part.V + part.G - 1) / part.G), kThreads, smem, st>>>(sc, part);
+    });
 }
 
 
@@ -1005,9 +1018,9 @@ template <int S> static cudaError_t scatter_stable_impl(const SceneDev &sc, cons
     const size_t smem = (size_t)fr.G * fr.n_tiles * sizeof(int) + kStableExtra;
     cudaError_t err = ensure_smem_limit((const void *)k_scatter_stable<S>, kBinSmemMax + kStableExtra);
     if (err != cudaSuccess) return err;
-    dim3 grid(fr.n_chunks, (fr.V + fr.G - 1) / fr.G);
-    k_scatter_stable<S><<<grid, kThreads, smem, st>>>(sc, fr);
-    return cudaGetLastError();
+    return by_views(fr, kGridY * fr.G, [&](const FrameDev &part) {
+        k_scatter_stable<S><<<dim3(part.n_chunks, (part.V + part.G - 1) / part.G), kThreads, smem, st>>>(sc, part);
+    });
 }
 
 cudaError_t launch_scatter(int storage, const SceneDev &sc, const FrameDev &fr, bool stable, cudaStream_t st) {
