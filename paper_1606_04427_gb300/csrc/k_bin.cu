@@ -494,11 +494,13 @@ __global__ void __launch_bounds__(32 * kChunkSegs) k_chunk_scan(FrameDev fr) {
 // ---------------------------------------------------------------------------------------
 // k_scan: tile segment offsets (int64), work items (a tile with more than K pairs is split
 // into ceil(count / K) items), scratch slots of split tiles, and the items' size histogram
-// for k_item_order.  A CTA scans kScanTiles tiles and sums the others itself (their counts are
-// in L2), so the CTAs need no order among them: 14 us for 16384 tiles and 22 us for 65536 (30 and
-// 113 us with one CTA for all).
+// for k_item_order.  A CTA scans kScanTiles tiles, or several times as many one after another, and
+// sums those before it itself (their counts are in L2), so the CTAs need no order among them: 14 us
+// for 16384 tiles and 22 us for 65536 (30 and 113 us with one CTA for all).  At most kScanCtas of
+// them, or the sums would grow with the square of the tiles: 16 M tiles take 3.8 ms with the chunk
+// scan, 46 with a CTA for each 4096 tiles, 31 with one for all.
 
-constexpr int kScanItems = 4, kScanTiles = 1024 * kScanItems;
+constexpr int kScanItems = 4, kScanTiles = 1024 * kScanItems, kScanCtas = 152;
 
 // Sum of two values over a 1024-thread CTA, for every thread.
 __device__ __forceinline__ void block_sum2(long long &a, long long &b, long long (*s_w)[33]) {
@@ -517,11 +519,12 @@ __device__ __forceinline__ void block_sum2(long long &a, long long &b, long long
     }
 }
 
-__global__ void __launch_bounds__(1024) k_scan(FrameDev fr, int target_items, int kmin) {
+// rounds: scans of kScanTiles tiles per CTA
+__global__ void __launch_bounds__(1024) k_scan(FrameDev fr, int target_items, int kmin, int rounds) {
     __shared__ long long s_w[2][33];
     __shared__ int s_hist[kOrderBins];
     const int N = fr.V * fr.n_tiles;
-    const int base = blockIdx.x * kScanTiles;
+    const int base = blockIdx.x * rounds * kScanTiles;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x < kOrderBins) s_hist[threadIdx.x] = 0;
     // total pairs (counts is padded to a whole int4; entries past N are not added)
@@ -549,57 +552,58 @@ __global__ void __launch_bounds__(1024) k_scan(FrameDev fr, int target_items, in
     }
     if (base > 0) block_sum2(pre_p, pre_is, s_w);
 
-    const int k0 = base + threadIdx.x * kScanItems;
-    int c[kScanItems], it[kScanItems];
-    long long lp = 0, lis = 0;
+    for (int round = 0; round < rounds; ++round) {
+        const int64_t k0 = base + (int64_t)round * kScanTiles + threadIdx.x * kScanItems;
+        int c[kScanItems], it[kScanItems];
+        long long lp = 0, lis = 0;
 #pragma unroll
-    for (int q = 0; q < kScanItems; ++q) {
-        const bool in = k0 + q < N;
-        c[q] = in ? fr.counts[k0 + q] : 0;
-        it[q] = in ? items_of(c[q]) : 0;
-        lp += c[q];
-        lis += ((long long)it[q] << 32) + (c[q] > K);
-        // the tile's last slice, counted once per warp and bin, and its full ones
-        const int bin = in ? order_bin(c[q] - K * (it[q] - 1), K) : kOrderBins;
-        const uint32_t peers = warp_peers<7>((uint32_t)bin);
-        if (in && lane == __ffs(peers) - 1) atomicAdd(&s_hist[bin], __popc(peers));
-        if (it[q] > 1) atomicAdd(&s_hist[order_bin(K, K)], it[q] - 1);
-    }
-    // exclusive scan of both over the CTA
-    const long long wp = warp_incl_scan(lp), wis = warp_incl_scan(lis);
-    __syncthreads();
-    if (lane == 31) s_w[0][warp] = wp, s_w[1][warp] = wis;
-    __syncthreads();
-    const long long p_w = s_w[0][lane], is_w = s_w[1][lane];
-    const long long p_i = warp_incl_scan(p_w), is_i = warp_incl_scan(is_w);
-    const long long tp = __shfl_sync(0xffffffffu, p_i, 31), tis = __shfl_sync(0xffffffffu, is_i, 31);
-    long long ep = pre_p + wp - lp + __shfl_sync(0xffffffffu, p_i - p_w, warp);
-    long long eis = pre_is + wis - lis + __shfl_sync(0xffffffffu, is_i - is_w, warp);
-#pragma unroll
-    for (int q = 0; q < kScanItems; ++q) {
-        const int k = k0 + q;
-        if (k < N) {
-            fr.offsets[k] = ep;
-            fr.item_off[k] = (int)(eis >> 32);
-            fr.split_slot[k] = c[q] > K ? (int)(eis & 0xffffffffll) : -1;
+        for (int q = 0; q < kScanItems; ++q) {
+            const bool in = k0 + q < N;
+            c[q] = in ? fr.counts[k0 + q] : 0;
+            it[q] = in ? items_of(c[q]) : 0;
+            lp += c[q];
+            lis += ((long long)it[q] << 32) + (c[q] > K);
+            // the tile's last slice, counted once per warp and bin, and its full ones
+            const int bin = in ? order_bin(c[q] - K * (it[q] - 1), K) : kOrderBins;
+            const uint32_t peers = warp_peers<7>((uint32_t)bin);
+            if (in && lane == __ffs(peers) - 1) atomicAdd(&s_hist[bin], __popc(peers));
+            if (it[q] > 1) atomicAdd(&s_hist[order_bin(K, K)], it[q] - 1);
         }
-        ep += c[q];
-        eis += ((long long)it[q] << 32) + (c[q] > K);
+        // exclusive scan of both over the CTA
+        const long long wp = warp_incl_scan(lp), wis = warp_incl_scan(lis);
+        __syncthreads();
+        if (lane == 31) s_w[0][warp] = wp, s_w[1][warp] = wis;
+        __syncthreads();
+        const long long p_w = s_w[0][lane], is_w = s_w[1][lane];
+        const long long p_i = warp_incl_scan(p_w), is_i = warp_incl_scan(is_w);
+        long long ep = pre_p + wp - lp + __shfl_sync(0xffffffffu, p_i - p_w, warp);
+        long long eis = pre_is + wis - lis + __shfl_sync(0xffffffffu, is_i - is_w, warp);
+#pragma unroll
+        for (int q = 0; q < kScanItems; ++q) {
+            if (k0 + q < N) {
+                fr.offsets[k0 + q] = ep;
+                fr.item_off[k0 + q] = (int)(eis >> 32);
+                fr.split_slot[k0 + q] = c[q] > K ? (int)(eis & 0xffffffffll) : -1;
+            }
+            ep += c[q];
+            eis += ((long long)it[q] << 32) + (c[q] > K);
+        }
+        pre_p += __shfl_sync(0xffffffffu, p_i, 31), pre_is += __shfl_sync(0xffffffffu, is_i, 31);
     }
     if (threadIdx.x < kOrderBins && s_hist[threadIdx.x]) atomicAdd(&fr.bins[threadIdx.x], s_hist[threadIdx.x]);
     if (blockIdx.x != gridDim.x - 1) return;
     // the scatter's cursors are 32-bit within a view
     int big = 0;
     if (tot > (long long)INT32_MAX)
-        for (int v = threadIdx.x; v < fr.V; v += blockDim.x) {
+        for (int v = warp; v < fr.V; v += 32) {
             long long sum = 0;
-            for (int t = 0; t < fr.n_tiles; ++t) sum += fr.counts[(int64_t)v * fr.n_tiles + t];
+            for (int t = lane; t < fr.n_tiles; t += 32) sum += fr.counts[(int64_t)v * fr.n_tiles + t];
+            for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
             big |= sum > (long long)INT32_MAX;
         }
     big = __syncthreads_or(big);
     if (threadIdx.x == 0) {
-        const long long is = pre_is + tis;
-        const int items = (int)(is >> 32), splits = (int)(is & 0xffffffffll);
+        const int items = (int)(pre_is >> 32), splits = (int)(pre_is & 0xffffffffll);
         fr.offsets[N] = tot;
         fr.item_off[N] = items;
         fr.sizes[kSizePairs] = tot;
@@ -617,7 +621,8 @@ cudaError_t launch_scan(const FrameDev &fr, int target_items, int kmin, cudaStre
     by_views(fr, kGridY, [&](const FrameDev &part) {
         k_chunk_scan<<<dim3((part.n_tiles + 31) / 32, part.V), 32 * kChunkSegs, 0, st>>>(part);
     });
-    k_scan<<<(int)((N + kScanTiles - 1) / kScanTiles), 1024, 0, st>>>(fr, target_items, kmin);
+    const int blocks = (int)((N + kScanTiles - 1) / kScanTiles), rounds = (blocks + kScanCtas - 1) / kScanCtas;
+    k_scan<<<(blocks + rounds - 1) / rounds, 1024, 0, st>>>(fr, target_items, kmin, rounds);
     return cudaGetLastError();
 }
 
