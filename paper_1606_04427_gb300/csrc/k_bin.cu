@@ -1263,6 +1263,9 @@ __global__ void __launch_bounds__(256) k_expand(const ViewParams *__restrict__ v
             n1 = poff[q + 1] + sums[(q + 1) / kScanChunk];
         }
     };
+    // every slot of the P has to be written: the counts add up to them
+    if (blockIdx.x == 0 && threadIdx.x == 0 && (int64_t)poff[n] + sums[n / kScanChunk] != P)
+        atomicExch(&status[kStatOverflow], 1);
     ahead(base0 + lane);
     for (int64_t base = base0; base < n; base += wstride) {
         const int64_t q = base + lane;
@@ -1272,11 +1275,12 @@ __global__ void __launch_bounds__(256) k_expand(const ViewParams *__restrict__ v
         int tx0 = 0, tx1 = -1, ty0 = 0, ty1 = -1;
         if (c) tile_box(s_v, rec.x, rec.y, rec.z, tx0, tx1, ty0, ty1);
         const bool small = c && tx1 >= tx0 && tx1 - tx0 <= 1 && ty1 - ty0 <= 1;
+        if (c && (tx1 < tx0 || ty1 < ty0)) atomicExch(&status[kStatOverflow], 1);
         if (small) {
             const uint32_t m = tile_mask2(s_v, rec.x, rec.y, rec.z, tx0, tx1, ty0, ty1);
             const uint32_t t00 = (uint32_t)(ty0 * s_v.ntx + tx0);
             uint32_t pos = o0;
-            if ((uint32_t)__popc(m) > c || (int64_t)o0 + __popc(m) > P) {
+            if ((uint32_t)__popc(m) != c || (int64_t)o0 + c > P) {
                 atomicExch(&status[kStatOverflow], 1);
             } else {
 #pragma unroll
@@ -1315,6 +1319,7 @@ __global__ void __launch_bounds__(256) k_expand(const ViewParams *__restrict__ v
                     }
                     k += (uint32_t)__popc(bal);
                 }
+            if (lane == 0 && k != bc) atomicExch(&status[kStatOverflow], 1);
         }
     }
 }

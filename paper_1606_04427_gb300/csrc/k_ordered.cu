@@ -375,17 +375,18 @@ __global__ void __launch_bounds__(kComposeThreads) k_compose_slices(FrameDev fr,
     }
 }
 
-__global__ void k_gather_records(const float4 *__restrict__ src, const uint32_t *__restrict__ idx, int64_t n,
-                                 float4 *dst) {
+__global__ void k_gather_records(const float4 *__restrict__ src, const uint32_t *__restrict__ idx, uint32_t last,
+                                 int64_t n, float4 *dst) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        dst[i] = src[idx[i]];
+        dst[i] = src[min(idx[i], last)];
 }
 
 static int grid_for(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 32)); }
 
-cudaError_t launch_gather_records(const float4 *src, const uint32_t *idx, int64_t n, float4 *dst, cudaStream_t st) {
+cudaError_t launch_gather_records(const float4 *src, const uint32_t *idx, uint32_t last, int64_t n, float4 *dst,
+                                  cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_gather_records<<<grid_for(n), 256, 0, st>>>(src, idx, n, dst);
+    k_gather_records<<<grid_for(n), 256, 0, st>>>(src, idx, last, n, dst);
     return cudaGetLastError();
 }
 

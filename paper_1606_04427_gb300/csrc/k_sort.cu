@@ -134,7 +134,8 @@ __global__ void __launch_bounds__(1024) k_scan_chunks(uint32_t *a, int64_t n, ui
 }
 
 // kGather: the last pass of a sort whose values index a payload: instead of the keys and
-// values, write payload[value] to each element's slot (payload_out).
+// values, write payload[value] to each element's slot (payload_out).  A value past payload_last
+// reads that one.
 template <typename K, bool kGather>
 __global__ void __launch_bounds__(kSortThreads, 3) k_digit_scatter(const K *__restrict__ keys,
                                                                const uint32_t *__restrict__ vals, int64_t n,
@@ -144,6 +145,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_digit_scatter(const K *__re
                                                                K *__restrict__ keys_out,
                                                                uint32_t *__restrict__ vals_out,
                                                                const float4 *__restrict__ payload,
+                                                               uint32_t payload_last,
                                                                float4 *__restrict__ payload_out) {
     __shared__ uint32_t s_wc[kSortWarps][256];  // per warp: running count, then warp base
     __shared__ uint32_t s_off[256];             // output start of this CTA's digit d
@@ -242,7 +244,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_digit_scatter(const K *__re
         const uint32_t d = s_dig[l];
         const uint32_t g = s_off[d] + (uint32_t)l - s_loc[d];
         if (kGather)
-            payload_out[g] = payload[s_val[l]];
+            payload_out[g] = payload[min(s_val[l], payload_last)];
         else
             vals_out[g] = s_val[l];
     }
@@ -261,10 +263,11 @@ size_t sort_temp_bytes(int64_t n) {
 template <typename K>
 static cudaError_t sort_impl(K *keys, K *keys_alt, uint32_t *vals, uint32_t *vals_alt, int64_t n, int bit_lo,
                              int bit_hi, void *temp, cudaStream_t st, bool *in_alt, KeyRange range,
-                             const float4 *payload = nullptr, float4 *payload_out = nullptr) {
+                             const float4 *payload = nullptr, uint32_t payload_last = 0,
+                             float4 *payload_out = nullptr) {
     *in_alt = false;
     if (n <= 1 || bit_lo >= bit_hi) {
-        if (payload && n > 0) return launch_gather_records(payload, vals, n, payload_out, st);
+        if (payload && n > 0) return launch_gather_records(payload, vals, payload_last, n, payload_out, st);
         return cudaSuccess;
     }
     const int nb = sort_blocks(n);
@@ -279,10 +282,10 @@ static cudaError_t sort_impl(K *keys, K *keys_alt, uint32_t *vals, uint32_t *val
         k_scan_chunks<<<chunks, 1024, 0, st>>>(hist, h, sums, arrivals);
         if (payload && shift + 8 >= bit_hi)
             k_digit_scatter<K, true><<<nb, kSortThreads, 0, st>>>(ka, va, n, shift, range, nb, hist, sums, kb, vb,
-                                                                 payload, payload_out);
+                                                                 payload, payload_last, payload_out);
         else
             k_digit_scatter<K, false><<<nb, kSortThreads, 0, st>>>(ka, va, n, shift, range, nb, hist, sums, kb, vb,
-                                                                  nullptr, nullptr);
+                                                                  nullptr, 0, nullptr);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         range = KeyRange{};
@@ -304,11 +307,11 @@ cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *keys_alt, uint32_t *vals,
 }
 
 cudaError_t radix_sort_gather(uint32_t *keys, uint32_t *keys_alt, uint32_t *vals, uint32_t *vals_alt, int64_t n,
-                              int bit_lo, int bit_hi, void *temp, const float4 *payload, float4 *payload_out,
-                              cudaStream_t st) {
+                              int bit_lo, int bit_hi, void *temp, const float4 *payload, int64_t payload_n,
+                              float4 *payload_out, cudaStream_t st) {
     bool alt = false;
     return sort_impl<uint32_t>(keys, keys_alt, vals, vals_alt, n, bit_lo, bit_hi, temp, st, &alt, KeyRange{},
-                               payload, payload_out);
+                               payload, (uint32_t)(payload_n - 1), payload_out);
 }
 
 size_t scan_temp_bytes(int64_t n) {

@@ -1861,7 +1861,8 @@ extern "C" splotch_status splotch_render_ordered(splotch_scene *sc, const splotc
     int tbits = 8;
     while (tbits < 32 && ((int64_t)(rs.views[0].n_tiles - 1) >> tbits) > 0) tbits += 8;
     if (e == cudaSuccess)
-        e = radix_sort_gather(tka, tkb, tva, tvb, P, 0, tbits, ex + o_tmp, (const float4 *)(ex + o_srec), fr.lists, st);
+        e = radix_sort_gather(tka, tkb, tva, tvb, P, 0, tbits, ex + o_tmp, (const float4 *)(ex + o_srec), n, fr.lists,
+                              st);
     const int64_t squares = (int64_t)std::max(1, items) * split * split;
     const int per_cta = std::max(1, ordered_workers_per_sm() / ordered_ctas_per_sm());
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count(sc->dev) * ordered_ctas_per_sm(),

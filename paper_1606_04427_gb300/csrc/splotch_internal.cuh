@@ -434,11 +434,12 @@ cudaError_t radix_sort_pairs(uint64_t *keys, uint64_t *keys_alt, uint32_t *vals,
 cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *keys_alt, uint32_t *vals, uint32_t *vals_alt, int64_t n,
                              int bit_lo, int bit_hi, void *temp, cudaStream_t st, bool *in_alt,
                              KeyRange range = KeyRange{});
-// Sort by key bits [bit_lo, bit_hi) whose values index `payload`, and write the payload in
-// sorted order to payload_out (the last pass gathers; keys and values end up undefined).
+// Sort by key bits [bit_lo, bit_hi) whose values index `payload` (payload_n > 0 entries; a value
+// past them reads the last), and write the payload in sorted order to payload_out (the last pass
+// gathers; keys and values end up undefined).
 cudaError_t radix_sort_gather(uint32_t *keys, uint32_t *keys_alt, uint32_t *vals, uint32_t *vals_alt, int64_t n,
-                              int bit_lo, int bit_hi, void *temp, const float4 *payload, float4 *payload_out,
-                              cudaStream_t st);
+                              int bit_lo, int bit_hi, void *temp, const float4 *payload, int64_t payload_n,
+                              float4 *payload_out, cudaStream_t st);
 // Exclusive scan of 32-bit counts whose total stays below 2^32, in two parts: entry i is
 // a[i] + temp[i / kScanChunk].  *scan_arrivals(n, temp) must be 0 before.
 constexpr int kScanChunk = 4096;  // entries per CTA
@@ -450,7 +451,7 @@ cudaError_t exclusive_scan_u32(uint32_t *a, int64_t n, void *temp, cudaStream_t 
 // the range of the active keys), the records and counts in sorted order (cnt has n + 1 entries,
 // the last set to 0; *arrivals is set to 0 for the scan of cnt), and the expansion into pairs
 // (tile id, place in sorted order) at the scanned offsets poff, sums; k_expand flags
-// kStatOverflow in `status` if a particle's tiles disagree with its count.
+// kStatOverflow in `status` if a particle's tiles disagree with its count, or the counts with P.
 cudaError_t launch_depth_records(int storage, const SceneDev &sc, const ViewParams *views, float4 *prec,
                                  uint32_t *dkey, uint32_t *pid, uint32_t *krange, cudaStream_t st);
 cudaError_t launch_sorted_counts(const ViewParams *views, const float4 *prec, const uint32_t *skey,
@@ -461,7 +462,8 @@ cudaError_t launch_expand(const ViewParams *views, const float4 *srec, const uin
 
 // Depth-ordered render: record gather by sorted index and the ordered splat (tiles up to
 // 32 px; squares of up to 16 px, split when T > 16).
-cudaError_t launch_gather_records(const float4 *src, const uint32_t *idx, int64_t n, float4 *dst, cudaStream_t st);
+cudaError_t launch_gather_records(const float4 *src, const uint32_t *idx, uint32_t last, int64_t n, float4 *dst,
+                                  cudaStream_t st);
 int ordered_split(int T);
 int ordered_ctas_per_sm();
 int ordered_workers_per_sm();
