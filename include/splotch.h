@@ -49,7 +49,7 @@ typedef enum {
     SPLOTCH_ERR_OOM = 2,         /* an allocation (callback or default) returned NULL */
     SPLOTCH_ERR_CUDA = 3,        /* a CUDA runtime call failed */
     SPLOTCH_ERR_CAPACITY = 4,    /* a plan's pre-sized buffers were too small for this frame */
-    SPLOTCH_ERR_TIMEOUT = 5,     /* a bounded device wait ran out (the kernel returned early) */
+    SPLOTCH_ERR_TIMEOUT = 5,     /* a bounded device wait ran out (the self-test's; no render waits) */
     SPLOTCH_ERR_UNSUPPORTED = 6  /* valid request outside this build's limits (e.g. tile count) */
 } splotch_status;
 
@@ -142,14 +142,14 @@ typedef struct {
  *   sigma_over_R  Gaussian sigma as a fraction of the support, > 0 (0.5)
  *   r_min_px      smallest support radius in pixels, >= 0 (0.75)
  *   block_particles  particles each CTA of the raster / count / scatter kernels streams,
- *                 rounded up to a multiple of 1024 (FP32) or 2048 (FP16 / BF16);
+ *                 rounded up to a multiple of 4096 (FP32) or 8192 (FP16 / BF16);
  *                 0 = about four CTAs per SM.  A tuning knob with no effect on results.
  *   flags         SPLOTCH_OUT_ACCUM: write the accumulation a instead of 1 - exp(-a);
  *                 SPLOTCH_OUT_ADD: add the accumulation a to what `out` holds (several
  *                 renders, e.g. particle subsets, summed in one image; the final transform
  *                 is then applied once with splotch_final_transform);
- *                 SPLOTCH_SYNC: splotch_render waits for the frame and reports a device-side
- *                 TIMEOUT before returning; SPLOTCH_PLAN_GRAPH: a plan captures its launch
+ *                 SPLOTCH_SYNC: splotch_render waits for the frame and reports its errors
+ *                 before returning; SPLOTCH_PLAN_GRAPH: a plan captures its launch
  *                 sequence into a CUDA graph on first launch and replays it afterwards;
  *                 SPLOTCH_TIMING: splotch_render records CUDA events around each kernel on
  *                 `stream`, waits for the frame and keeps the durations for
@@ -208,7 +208,7 @@ splotch_status splotch_camera_params(const splotch_camera *cam, float m[12], flo
  *   out = 1 - exp(-a) (or a with SPLOTCH_OUT_ACCUM).
  * The call blocks until the particle-tile pair count of each view is known (to size the
  * tile lists), then enqueues the rest on `stream` and returns; out is ready when `stream`
- * reaches that point.  Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA, TIMEOUT. */
+ * reaches that point.  Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA. */
 splotch_status splotch_render(splotch_scene *scene, const splotch_camera *cams, int32_t n_views,
                               const splotch_render_params *params, float *out, void *stream);
 
@@ -227,8 +227,8 @@ splotch_status splotch_render(splotch_scene *scene, const splotch_camera *cams, 
  * to 32 px (larger: UNSUPPORTED); other output flags are ignored.  The particles are sorted by
  * depth (stable radix sort from index order) and their tile entries, written out in that
  * order, grouped by a stable sort on tile id; device memory besides the tile lists: about 52
- * bytes per particle, 16 per particle-tile pair and 24 T^2 per slice of a tile list.  Synchronous.  Errors: INVALID_ARG,
- * UNSUPPORTED, OOM, CUDA, TIMEOUT. */
+ * bytes per particle, 16 per particle-tile pair and 24 T^2 per slice of a tile list.
+ * Synchronous.  Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA. */
 splotch_status splotch_render_ordered(splotch_scene *scene, const splotch_camera *cam,
                                       const splotch_render_params *params, const float *absorb, float *out,
                                       void *stream);
@@ -323,8 +323,8 @@ splotch_status splotch_plan_set_colormaps(splotch_plan *plan, const float *const
 /* Enqueue one batch render into out (device, n_views x H x W x 3 FP32). */
 splotch_status splotch_plan_launch(splotch_plan *plan, float *out, void *stream);
 
-/* Synchronise `stream` and report the last launch: OK, CAPACITY (pairs_needed set), or
- * TIMEOUT.  pairs_needed may be NULL. */
+/* Synchronise `stream` and report the last launch: OK or CAPACITY (pairs_needed set).
+ * pairs_needed may be NULL. */
 splotch_status splotch_plan_check(splotch_plan *plan, void *stream, int64_t *pairs_needed);
 
 /* Device bytes a plan holds (its workspace), and its tile size. */
@@ -365,8 +365,8 @@ splotch_status splotch_frame_prepare(splotch_scene *scene, const splotch_camera 
 splotch_status splotch_frame_render(splotch_frame *frame, float *out, void *stream);
 splotch_status splotch_frame_destroy(splotch_frame *frame);
 
-/* Self-test of the bounded device wait every kernel uses: one CTA waits on a shared-memory
- * mbarrier that nothing completes, gives up after ~limit_cycles SM cycles (1e3..1e10) and
+/* Self-test of a bounded device wait (the render kernels wait on nothing but their own warps and
+ * copies): one CTA waits on a shared-memory mbarrier that nothing completes, gives up after ~limit_cycles SM cycles (1e3..1e10) and
  * reports it.  Returns SPLOTCH_ERR_TIMEOUT when the wait ran out as designed, SPLOTCH_OK
  * if the barrier completed (it cannot), INVALID_ARG / CUDA otherwise.  Synchronous. */
 splotch_status splotch_selftest_bounded_wait(int64_t limit_cycles, void *stream);

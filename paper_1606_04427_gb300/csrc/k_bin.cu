@@ -43,7 +43,6 @@ cudaError_t ensure_smem_limit(const void *kernel, size_t bytes) {
 // largest tile histogram: G x n_tiles <= kMaxTiles counters
 constexpr size_t kBinSmemMax = sizeof(int) * (size_t)kMaxTiles;
 
-
 // ---------------------------------------------------------------------------------------
 // Scene preparation (Section 2.1: ranging, normalisation, optional logarithm).
 
@@ -1172,10 +1171,8 @@ __global__ void __launch_bounds__(256) k_depth_records(SceneDev sc, const ViewPa
     }
 }
 
-// Depth keys relative to the smallest active one (active: key - base in [0, span];
-// inactive: span + 1, sorted last).
-// Tiles of a rasterised particle, in row-major order over its tile box: the first
-// `small` boxes (up to 2 x 2) by one lane, larger ones by the whole warp.
+// Candidate tiles of a rasterised particle (up to 2 x 2 are tested by one lane, more by the whole
+// warp).
 __device__ __forceinline__ void tile_box(const ViewParams &v, float X, float Y, float R, int &tx0, int &tx1,
                                          int &ty0, int &ty1) {
     int i0, i1, j0, j1;

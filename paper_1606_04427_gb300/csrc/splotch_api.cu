@@ -925,20 +925,12 @@ static splotch_status render_frame(splotch_scene *sc, const RenderSetup &rs, flo
                               st, ev);
         if (s != SPLOTCH_OK) break;
         if (sync) {
-            int64_t *box = host_box();
-            if (!box) {
-                s = fail(SPLOTCH_ERR_OOM, "pinned host buffer");
-                break;
-            }
-            cudaError_t e = cudaMemcpyAsync(box, fixed + fh.o_status, sizeof(int) * 4, cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            const cudaError_t e = cudaStreamSynchronize(st);
             if (e != cudaSuccess) {
                 s = fail(SPLOTCH_ERR_CUDA, "render: %s", cudaGetErrorString(e));
                 break;
             }
-            const int *stat = (const int *)box;
-            if (stat[kStatTimeout]) s = fail(SPLOTCH_ERR_TIMEOUT, "splat stage wait timed out");
-            if (timed && s == SPLOTCH_OK) {
+            if (timed) {
                 float t[4] = {0, 0, 0, 0};
                 cudaEventElapsedTime(&t[0], ev[0], ev[1]);
                 cudaEventElapsedTime(&t[1], ev[1], ev[2]);
@@ -1107,12 +1099,8 @@ extern "C" splotch_status splotch_frame_render(splotch_frame *f, float *out, voi
     splotch_status s = frame_scatter(f, st);
     if (s == SPLOTCH_OK) s = frame_splat(f, out, st);
     if (s != SPLOTCH_OK || !(f->rs.pr.flags & SPLOTCH_SYNC)) return s;
-    int64_t *box = host_box();
-    if (!box) return fail(SPLOTCH_ERR_OOM, "pinned host buffer");
-    cudaError_t e = cudaMemcpyAsync(box, f->fixed + f->fh.o_status, sizeof(int) * 4, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    const cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return fail(SPLOTCH_ERR_CUDA, "render: %s", cudaGetErrorString(e));
-    if (((const int *)box)[kStatTimeout]) return fail(SPLOTCH_ERR_TIMEOUT, "splat stage wait timed out");
     return SPLOTCH_OK;
 }
 
@@ -1397,7 +1385,6 @@ extern "C" splotch_status splotch_plan_check(splotch_plan *pl, void *stream, int
     const int64_t *sizes = pl->box;
     const int *stat = (const int *)(pl->box + 8);
     if (pairs_needed) *pairs_needed = sizes[kSizePairs];
-    if (stat[kStatTimeout]) return fail(SPLOTCH_ERR_TIMEOUT, "splat stage wait timed out");
     if (stat[kStatOverflow])
         return fail(SPLOTCH_ERR_CAPACITY, "frame needs %lld pairs / %lld items / %lld split tiles, plan holds %lld / %d / %d",
                     (long long)sizes[kSizePairs], (long long)sizes[kSizeItems], (long long)sizes[kSizeSplits],
@@ -1529,7 +1516,7 @@ extern "C" splotch_status splotch_render_noalloc(splotch_scene *sc, const splotc
     char *var = base + fixed;
     FrameDev fr = frame_dev(fh, base, var);
 
-    // every call shares the array: zero what the kernels count into before they start
+    // every call shares the array: the accumulators of split tiles start at zero
     cudaStream_t st = (cudaStream_t)stream;
     CUDA_TRY(cudaMemcpyAsync(base + fh.o_views, &vp, sizeof(ViewParams), cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaMemsetAsync(var + fh.o_scratch, 0, fh.var_bytes - fh.o_scratch, st));
@@ -1542,7 +1529,6 @@ extern "C" splotch_status splotch_render_noalloc(splotch_scene *sc, const splotc
     CUDA_TRY(cudaMemcpyAsync(sizes, base + fh.o_sizes, sizeof(sizes), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaMemcpyAsync(stat, base + fh.o_status, sizeof(stat), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
-    if (stat[kStatTimeout]) return fail(SPLOTCH_ERR_TIMEOUT, "splat stage wait timed out");
     if (stat[kStatOverflow])
         return fail(SPLOTCH_ERR_CAPACITY,
                     "frame needs %lld particle-tile pairs and %lld split tiles; the fixed %zu-byte workspace holds %lld and %d",
@@ -1878,6 +1864,5 @@ extern "C" splotch_status splotch_render_ordered(splotch_scene *sc, const splotc
     sc->mem.release(fixed, st);
     if (e != cudaSuccess) return fail(SPLOTCH_ERR_CUDA, "ordered render: %s", cudaGetErrorString(e));
     if (stat[kStatOverflow]) return fail(SPLOTCH_ERR_CUDA, "depth-ordered binning: tile counts disagree");
-    if (stat[kStatTimeout]) return fail(SPLOTCH_ERR_TIMEOUT, "splat stage wait timed out");
     return SPLOTCH_OK;
 }

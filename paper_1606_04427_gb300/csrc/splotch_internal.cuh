@@ -78,7 +78,7 @@ struct FrameDev {
     int *item_off;            // [V * n_tiles + 1] first work item of each tile
     int *split_slot;          // [V * n_tiles] scratch slot of tiles split over items, else -1
     int64_t *sizes;           // [8] pairs, items, splits, K
-    int *status;              // [4] 0: capacity overflow, 1: timeout
+    int *status;              // [4] 0: capacity overflow
     int *bins;                // [2 * kOrderBins] work items per size bin, and k_item_order's cursors
     int *queue;               // [4] the splat's work queue
     float4 *lists;            // [pair capacity] tile records (X, Y, R, code)
@@ -97,7 +97,7 @@ struct FrameDev {
 };
 
 enum { kSizePairs = 0, kSizeItems = 1, kSizeSplits = 2, kSizeK = 3 };
-enum { kStatOverflow = 0, kStatTimeout = 1 };
+enum { kStatOverflow = 0 };
 
 // Size bin of a work item of `size` <= K records, for the splat's largest-first order.
 constexpr int kOrderBins = 64;
@@ -111,7 +111,6 @@ __device__ __forceinline__ int order_bin(int size, int K) {
 template <int S> struct Store;
 template <> struct Store<0> {
     static constexpr int VEC = 4;
-    static constexpr int BYTES = 4;
     __device__ __forceinline__ static void load(const void *p, int64_t i, float *v) {
         float4 a = __ldg(reinterpret_cast<const float4 *>(static_cast<const float *>(p) + i));
         v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
@@ -119,7 +118,6 @@ template <> struct Store<0> {
 };
 template <> struct Store<1> {
     static constexpr int VEC = 8;
-    static constexpr int BYTES = 2;
     __device__ __forceinline__ static void load(const void *p, int64_t i, float *v) {
         uint4 a = __ldg(reinterpret_cast<const uint4 *>(static_cast<const __half *>(p) + i));
         const __half2 *q = reinterpret_cast<const __half2 *>(&a);
@@ -132,7 +130,6 @@ template <> struct Store<1> {
 };
 template <> struct Store<2> {
     static constexpr int VEC = 8;
-    static constexpr int BYTES = 2;
     __device__ __forceinline__ static void load(const void *p, int64_t i, float *v) {
         uint4 a = __ldg(reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(p) + i));
         const __nv_bfloat162 *q = reinterpret_cast<const __nv_bfloat162 *>(&a);
@@ -263,19 +260,8 @@ template <int NB> __device__ __forceinline__ uint32_t warp_peers(uint32_t key) {
     return peers;
 }
 
-// Inclusive warp scan of an int.
-__device__ __forceinline__ int warp_incl_scan_i(int v) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += u;
-    }
-    return v;
-}
-
 // ------------------------------------------------------------------------------------
-// Bulk-copy (TMA, non-tensor) and mbarrier helpers.
+// mbarrier helpers (of the self-test of a bounded wait; no render kernel waits on one).
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -286,39 +272,10 @@ __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
 __device__ __forceinline__ void mbar_fence_init() {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
-__device__ __forceinline__ void fence_proxy_async_smem() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-// Plain arrival (release semantics at CTA scope: this thread's earlier shared-memory
-// writes are visible to a thread whose wait observes the phase completing).
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Non-blocking test of a phase's completion.
-__device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(ok)
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
@@ -333,8 +290,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     }
     return true;
 }
-
-constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz
 
 // ------------------------------------------------------------------------------------
 // Exact, order-independent merge of FP32 partial sums (slices of a split tile).  A value

@@ -22,7 +22,7 @@ class RenderParams:
     """Tile edge (0 = library default), support factor, sigma / support, minimum
     support in pixels; ``accum`` returns the accumulation a instead of 1 - exp(-a);
     ``add`` adds the accumulation to what the output holds; ``sync`` waits for the frame
-    and reports device-side timeouts; ``map`` makes the depth-ordered render write the
+    and reports its errors; ``map`` makes the depth-ordered render write the
     per-pixel affine map (alpha, beta) instead of I; ``stable`` builds every tile list in
     ascending particle index, which makes the image bitwise reproducible (the binning
     takes longer)."""
