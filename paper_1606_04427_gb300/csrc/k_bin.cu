@@ -617,9 +617,10 @@ __global__ void __launch_bounds__(1024) k_scan(FrameDev fr, int target_items, in
 
 cudaError_t launch_scan(const FrameDev &fr, int target_items, int kmin, cudaStream_t st) {
     const int64_t N = (int64_t)fr.V * fr.n_tiles;
-    by_views(fr, kGridY, [&](const FrameDev &part) {
+    const cudaError_t err = by_views(fr, kGridY, [&](const FrameDev &part) {
         k_chunk_scan<<<dim3((part.n_tiles + 31) / 32, part.V), 32 * kChunkSegs, 0, st>>>(part);
     });
+    if (err != cudaSuccess) return err;
     const int blocks = (int)((N + kScanTiles - 1) / kScanTiles), rounds = (blocks + kScanCtas - 1) / kScanCtas;
     k_scan<<<(blocks + rounds - 1) / rounds, 1024, 0, st>>>(fr, target_items, kmin, rounds);
     return cudaGetLastError();
