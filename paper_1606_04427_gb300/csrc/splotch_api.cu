@@ -1652,6 +1652,7 @@ extern "C" splotch_status splotch_render_streamed(const splotch_scene_desc *d, i
         if (!sc) return;
         sc->mem.release(sc->attr, st);
         sc->mem.release(sc->meta, st);
+        sc->mem.release(sc->emit, st);
         delete sc;
     };
     const float *src[5] = {d->x, d->y, d->z, d->h, d->intensity};
