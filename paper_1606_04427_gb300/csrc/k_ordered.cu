@@ -20,7 +20,7 @@
 // is not split writes beta; the slices of a split tile store their maps, which k_compose_slices
 // composes far to near.
 //
-// What bounds it: the FP32 pipe.  Hence the short polynomials (8 to 10 packed operations per channel
+// What bounds it: the FP32 pipe.  Hence the short polynomials (9 or 10 packed operations per channel
 // and two pixels, 15 with the exponential) and squares of 4 x 4 pixels: 6.7 squares, 107 pixel
 // evaluations per particle, against 235 in the 8 x 8 units of a warp per record.  10 M particles at
 // 2048^2: frame 4.97 ms with a warp per record, 3.22 now (3.03 with the cheaper and less accurate
@@ -47,15 +47,16 @@ struct __align__(16) OWarpSmem {
 // where s = 0 stood for 2^-40 / E.  Emulated against 64 bits for 1 to 200 records, x from 0.001 to 2,
 // the present form is nowhere less accurate than a beta + b with a and b rounded apart.)
 // phi is a polynomial whose degree follows the step's largest x (w <= 1, so a record's x is at most
-// its s E): degree 2 up to kDeg2Max, 3 up to kDeg3Max, 4 up to kDeg4Max, minimax with phi(0) = 1
-// (fitted here by iteratively reweighted least squares against expm1 in 64 bits; largest relative
-// errors 5.4e-9, 8.0e-9 and 3.0e-9).  Beyond, and for negative emissions, the Taylor polynomial of
-// degree 5 where |x| <= kDeg4Max (next term x^6 / 7! <= 5e-8) and the exponential itself elsewhere:
-// alpha <- a alpha, beta <- a beta + (1 - a) / s, a = exp(-x).
-constexpr float kDeg2Max = 0.015f, kDeg3Max = 0.1f, kDeg4Max = 0.25f;
+// its s E): degree 3 up to kDeg3Max and 4 up to kDeg4Max, minimax with phi(0) = 1 (fitted here by
+// iteratively reweighted least squares against expm1 in 64 bits; largest relative errors 8.0e-9 and
+// 3.0e-9).  Beyond, and for negative emissions, the Taylor polynomial of degree 5 where
+// |x| <= kDeg4Max (next term x^6 / 7! <= 5e-8) and the exponential itself elsewhere:
+// alpha <- a alpha, beta <- a beta + (1 - a) / s, a = exp(-x).  (A degree 2 up to 0.015 as well: 10 M
+// particles at 2048^2 in 3.15 instead of 3.11 ms, a step's 16 records are rarely all below.)
+constexpr float kDeg3Max = 0.1f, kDeg4Max = 0.25f;
 
 // phi as a polynomial in -x (all coefficients positive)
-template <int kDeg> __device__ __forceinline__ float2 phi_of(float2 nx) {  // kDeg 5: Taylor
+template <int kDeg> __device__ __forceinline__ float2 phi_of(float2 nx) {  // degree 3, 4 or 5 (Taylor)
     float2 phi;
     if (kDeg == 5) {
         phi = __ffma2_rn(nx, f2(1.0f / 720.0f), f2(1.0f / 120.0f));
@@ -66,11 +67,9 @@ template <int kDeg> __device__ __forceinline__ float2 phi_of(float2 nx) {  // kD
         phi = __ffma2_rn(nx, f2(0.00753017422f), f2(0.0415001325f));
         phi = __ffma2_rn(nx, phi, f2(0.166652888f));
         phi = __ffma2_rn(nx, phi, f2(0.499999642f));
-    } else if (kDeg == 3) {
+    } else {
         phi = __ffma2_rn(nx, f2(0.0400981233f), f2(0.166576117f));
         phi = __ffma2_rn(nx, phi, f2(0.49999851f));
-    } else {
-        phi = __ffma2_rn(nx, f2(0.165799007f), f2(0.499995977f));
     }
     return __ffma2_rn(nx, phi, f2(1.0f));
 }
@@ -246,11 +245,10 @@ __global__ void __launch_bounds__(kOWarps * 32, 6)
                     // the largest
                     const uint32_t emax = max(__float_as_uint(pb.x), max(__float_as_uint(pb.y), __float_as_uint(pb.z)));
                     const uint32_t xmax = __float_as_uint(__uint_as_float(emax) * pb.w);
-                    if (!__any_sync(0xffffffffu, xmax > __float_as_uint(kDeg2Max)))
-                        apply_record<2>(pa, pb, fx, fy, al, be);
-                    else if (!__any_sync(0xffffffffu, xmax > __float_as_uint(kDeg3Max)))
+                    const uint32_t most = __reduce_max_sync(0xffffffffu, xmax);
+                    if (most <= __float_as_uint(kDeg3Max))
                         apply_record<3>(pa, pb, fx, fy, al, be);
-                    else if (!__any_sync(0xffffffffu, xmax > __float_as_uint(kDeg4Max)))
+                    else if (most <= __float_as_uint(kDeg4Max))
                         apply_record<4>(pa, pb, fx, fy, al, be);
                     else
                         apply_record<5>(pa, pb, fx, fy, al, be);
