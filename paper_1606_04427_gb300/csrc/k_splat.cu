@@ -292,7 +292,7 @@ __device__ __forceinline__ float magnitude(float x, float y, float z) { return f
 // latency: 50 k particles at 4096^2 take 142 us instead of 213.  The limit: with 32 / 64 / 96
 // records, 300 k clustered particles at 4096^2 take 253 / 232 / 232 us; 1 M at 256^2 (teams of 4)
 // 76 / 85 / 85.
-template <bool kViewScale, bool kEmit>
+template <bool kViewScale, bool kEmit, bool kWild>
 __device__ __forceinline__ void render_few(const SceneDev &sc, const FrameDev &fr, WarpSmem *ws, const Region &rg,
                                            const float4 *recs, int nrec, int v, float kexp) {
     const int lane = threadIdx.x & 31, x = 4 * (lane & 3), y = 2 * (lane >> 2);
@@ -330,8 +330,7 @@ __device__ __forceinline__ void render_few(const SceneDev &sc, const FrameDev &f
         }
         __syncwarp();
         const int n = __popc(bal);
-        if (kViewScale ? __any_sync(0xffffffffu, live && !isfinite(magnitude(e[0].x * vs, e[0].y * vs, e[0].z * vs)))
-                       : sc.wild) {
+        if (kWild && __any_sync(0xffffffffu, live && !isfinite(magnitude(e[0].x * vs, e[0].y * vs, e[0].z * vs)))) {
             if (!wild)
                 for (int k = lane; k < 3 * kRegion * kRegion; k += 32) (&ws->acc[0][0][0])[k] = 0.0f;
             wild = true;
@@ -351,14 +350,16 @@ __device__ __forceinline__ void render_few(const SceneDev &sc, const FrameDev &f
         for (int row = 0; row < 2; ++row) {
             float4 *p = reinterpret_cast<float4 *>(&ws->acc[c][y + row][x]);
             float4 u = make_float4(s[c][row][0].x, s[c][row][0].y, s[c][row][1].x, s[c][row][1].y);
-            if (wild) u.x += p->x, u.y += p->y, u.z += p->z, u.w += p->w;
+            if (kWild && wild) u.x += p->x, u.y += p->y, u.z += p->z, u.w += p->w;
             *p = u;
         }
 }
 
 // kViewScale: multiply every record's emission by a per-view, per-species scale (plans
 // with a brightness sequence); a separate instance, so plain renders carry no extra code.
-template <bool kViewScale, bool kEmit>
+// kWild: an emission may not be finite (add_wild): scenes that say so, and all plans, whose scales
+// change between replays.  The branch cost plain frames 0.4 to 0.8 % when they had it as well.
+template <bool kViewScale, bool kEmit, bool kWild>
 __global__ void __launch_bounds__(kWarps * 32, 2)
     k_splat(SceneDev sc, FrameDev fr, int *queue, float *out, int out_accum, int split) {
     if (fr.status[kStatOverflow]) return;  // no complete tile lists
@@ -463,7 +464,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
         }
 
         if (nrec <= few) {
-            render_few<kViewScale, kEmit>(sc, fr, ws, rg, recs, nrec, v, kexp);
+            render_few<kViewScale, kEmit, kWild>(sc, fr, ws, rg, recs, nrec, v, kexp);
             nrec = 0;
         } else {
             float *acc = &ws->acc[0][0][0];
@@ -482,7 +483,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
             // repeat the last record
             uint32_t word[Batch<kBatch>::kWords];
             int cnt;
-            float most = 0.0f;  // kViewScale: finite if the lane's emissions are
+            float most = 0.0f;  // finite if the lane's emissions are
             {
                 float4 rec[kRounds];
 #pragma unroll
@@ -519,10 +520,11 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
                     bt->pa[j] = make_float4(-rec[g].x, -rec[g].y, R2, gauss_scale(kexp, R2));
                     if constexpr (kViewScale || !kEmit)
                         bt->pb[j] = make_float4(e[g].x * vs[g], e[g].y * vs[g], e[g].z * vs[g], 0.0f);
-                    if constexpr (kViewScale) most += magnitude(e[g].x * vs[g], e[g].y * vs[g], e[g].z * vs[g]);
+                    if constexpr (kWild && kViewScale)
+                        most += magnitude(e[g].x * vs[g], e[g].y * vs[g], e[g].z * vs[g]);
                 }
             }
-            if (kViewScale ? __any_sync(0xffffffffu, !isfinite(most)) : sc.wild) {
+            if (kWild && (!kViewScale || __any_sync(0xffffffffu, !isfinite(most)))) {
                 __syncwarp();
                 add_wild(ws, nbuf, rg.px0, rg.py0);
             }
@@ -562,7 +564,6 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
 #pragma unroll 3
                 for (int k = 2; k < steps + 2; ++k) {
                     const float4 pa = na, pb = nb;
-                    const float R2 = pa.z;
                     na = bt->pa[idx];
                     nb = bt->pb[idx];
                     lp += 1 << a;
@@ -614,15 +615,16 @@ typedef void (*SplatFn)(SceneDev, FrameDev, int *, float *, int, int);
 // pixels) 8.72 against 32.2 ms, 200 k at 5000^2 (40 pixels) 0.44 against 0.43.
 int splat_split(int T) { return (T + kRegion - 1) / kRegion; }
 
-static SplatFn splat_fn(bool scaled, bool emit) {
-    if (emit) return scaled ? k_splat<true, true> : k_splat<false, true>;
-    return scaled ? k_splat<true, false> : k_splat<false, false>;
+static SplatFn splat_fn(bool scaled, bool emit, bool wild) {
+    if (scaled) return emit ? k_splat<true, true, true> : k_splat<true, false, true>;
+    if (wild) return emit ? k_splat<false, true, true> : k_splat<false, false, true>;
+    return emit ? k_splat<false, true, false> : k_splat<false, false, false>;
 }
 
 static size_t splat_smem() { return sizeof(WarpSmem) * kWarps; }
 
 int splat_blocks_per_sm() {
-    const void *fn = (const void *)splat_fn(false, false);
+    const void *fn = (const void *)splat_fn(false, false, false);
     if (ensure_smem_limit(fn, splat_smem()) != cudaSuccess) return 0;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kWarps * 32, splat_smem()) != cudaSuccess) return 0;
@@ -695,7 +697,7 @@ cudaError_t launch_splat(const SceneDev &sc, const FrameDev &fr, float *out, int
                          cudaStream_t st) {
     cudaError_t e = launch_item_order(fr, st);
     if (e != cudaSuccess) return e;
-    const SplatFn fn = splat_fn(fr.vscale != nullptr, sc.emit != nullptr);
+    const SplatFn fn = splat_fn(fr.vscale != nullptr, sc.emit != nullptr, sc.wild != 0);
     e = ensure_smem_limit((const void *)fn, splat_smem());
     if (e != cudaSuccess) return e;
     fn<<<grid, kWarps * 32, splat_smem(), st>>>(sc, fr, fr.queue, out, out_accum, splat_split(fr.T));
