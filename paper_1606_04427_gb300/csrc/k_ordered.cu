@@ -20,12 +20,14 @@
 // is not split writes beta; the slices of a split tile store their maps, which k_compose_slices
 // composes far to near.
 //
-// What bounds it: the FP32 pipe.  Hence the short polynomials (9 or 10 packed operations per channel
-// and two pixels, 15 with the exponential) and squares of 4 x 4 pixels: 6.7 squares, 107 pixel
+// What bounds it: the FP32 pipe (68 % of its cycles on the 10 M-particle two-species frame; a packed
+// operation holds it two).  Hence the short polynomials (9 or 10 packed operations per channel and
+// two pixels, 15 with the exponential) and squares of 4 x 4 pixels: 6.7 squares, 107 pixel
 // evaluations per particle, against 235 in the 8 x 8 units of a warp per record.  10 M particles at
-// 2048^2: frame 4.97 ms with a warp per record, 3.22 now (3.03 with the cheaper and less accurate
-// update that apply_record's comment names); a 1 M-particle map at 1000 x 757: 1.21 -> 0.58 ms
-// (0.54).  Batches of 192 (12 warps per SM): 128 on 16 warps took 2.47 ms where 192 took 2.21.
+// 2048^2: 3.33 ms with a warp per record, 1.64 and 0.05 for the composition now (1.52 with the
+// cheaper and less accurate update named below); a frame of 1 M particles as maps at 1000 x 757:
+// 1.22 -> 0.59 ms (0.55).  Batches of 192 (12 warps per SM): 128 on 16 warps took 2.47 ms where 192
+// took 2.21.
 #include "splat_batch.cuh"
 
 namespace spl {
@@ -327,7 +329,8 @@ __global__ void __launch_bounds__(kOWarps * 32, 6)
 // neighbouring crowded tiles go to different CTAs.  Bound by the latency of the loads: 41 us on
 // the 10 M-particle frame at 2048^2 (crowded tiles of some 350 slices), 109 with the loads left to
 // the compiler.  The last warp to finish a tile used to compose it, which held the splat up: 1.90
-// ms, now 1.53 and these 41 us; 4 M particles at 1024^2: 0.89 ms, now 0.40 + 0.09.
+// ms against 1.53 and these 41 us; 4 M particles at 1024^2: 0.89 ms against 0.40 + 0.09 (with the
+// cheaper update).
 constexpr int kComposeThreads = 256;
 constexpr int kAtOnce = 16;  // slices loaded together
 
