@@ -12,9 +12,9 @@
 // result.  In frames of few records teams of 2, 4 or 8 warps of a CTA take the long items
 // together (team_of): each warp renders a consecutive part of the list and the parts' sums are
 // added in order, so a frame of 256 tiles occupies 2048 warps instead of 256.  The items come
-// longest first; at the first short one a team parts and its warps go on alone.  (Without that
-// order the short items are the team's first warp's.)  How an item's sums are formed depends on the
-// item and the frame alone, never on which team or warp meets it.  Teams never wait on one another.
+// longest first; at the first short one a team parts and its warps go on alone.  How an item's sums
+// are formed depends on the item and the frame alone, never on which team or warp meets it.  Teams
+// never wait on one another.
 //
 // What a warp does with an item.  The kernel is bound by instruction issue and the latency
 // between its phases (the records are read once, DRAM is nearly idle), so the layout is
@@ -48,15 +48,6 @@
 #include "splat_batch.cuh"
 
 namespace spl {
-
-__device__ __forceinline__ int find_tile(const int *__restrict__ item_off, int N, int item) {
-    int a = 0, b = N - 1;  // last gt with item_off[gt] <= item
-    while (a < b) {
-        const int m = (a + b + 1) >> 1;
-        if (__ldg(&item_off[m]) <= item) a = m; else b = m - 1;
-    }
-    return a;
-}
 
 // Output of a pixel's accumulation a: mode 0 gives 1 - exp(-a) (final transform), 1 gives a,
 // 2 adds a to what the pixel held (several renders summed in one image).
@@ -373,7 +364,6 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
     constexpr int kRounds = Batch<kBatch>::kRounds;
     const int lane = threadIdx.x & 31;
     const int nt = fr.n_tiles;
-    const int N = fr.V * nt;
     const int S2 = split * split;
     const int64_t K = fr.sizes[kSizeK];
     const int pair = lane >> 1;  // lane pair: the unit that evaluates a square
@@ -410,14 +400,8 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
         // item = (slice of a tile list, region of the tile); the regions of a slice are
         // consecutive items, so they run at once and share the slice's records in L2
         const int qs = item / S2, q = item - qs * S2;
-        int gt, chunk;  // the slice's tile and its place in the tile's list
-        if (fr.order) {
-            const int2 o = __ldg(&fr.order[qs]);
-            gt = o.x, chunk = o.y;
-        } else {
-            gt = find_tile(fr.item_off, N, qs);
-            chunk = qs - fr.item_off[gt];
-        }
+        const int2 ord = __ldg(&fr.order[qs]);
+        const int gt = ord.x, chunk = ord.y;  // the slice's tile and its place in the tile's list
         const int v = gt / nt, t = gt - v * nt;
         const float kexp = fr.views[v].kexp;
         Region rg;
@@ -444,12 +428,15 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
         const float4 *recs = fr.lists + e0;
         int few = kFew;
         if (kn.team > 1) {
-            int part = nrec;  // the first warp's alone
             // by the slice's length: that of the order, also where the region has no pixel
             if (order_bin(len, (int)K) >= shared_from(kn.team)) {
-                part = ((nrec + kn.team - 1) / kn.team + 31) & ~31;
+                // this warp's consecutive part of the slice
+                const int part = ((nrec + kn.team - 1) / kn.team + 31) & ~31;
+                const int first = min(nrec, (me >> 5) * part);
+                recs += first;
+                nrec = min(part, nrec - first);
                 few = kFew / 2;
-            } else if (fr.order) {  // all later items are a warp's alone as well: the team parts
+            } else {  // the first warp's alone, and so are all later items: the team parts
                 if (lane == 0) s_known[threadIdx.x >> 5].team = 1;
                 __syncwarp();
                 if (me >= 32) {
@@ -457,10 +444,6 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
                     continue;
                 }
             }
-            // this warp's consecutive part of the slice
-            const int first = min(nrec, (me >> 5) * part);
-            recs += first;
-            nrec = min(part, nrec - first);
         }
 
         if (nrec <= few) {
@@ -687,7 +670,6 @@ __global__ void __launch_bounds__(1024) k_item_order(FrameDev fr) {
 }
 
 cudaError_t launch_item_order(const FrameDev &fr, cudaStream_t st) {
-    if (!fr.order) return cudaSuccess;
     const int64_t N = (int64_t)fr.V * fr.n_tiles;
     k_item_order<<<(int)((N + 1023) / 1024), 1024, 0, st>>>(fr);
     return cudaGetLastError();

@@ -733,8 +733,8 @@ static void layout_fixed(FrameHost &fh, const splotch_scene *sc, int V, int n_ti
 // Exact accumulators of one split tile: 3 channels x T x T pixels, 16 bytes each.
 static size_t split_scratch_bytes(int T) { return sizeof(unsigned long long) * 2 * 3 * (size_t)T * T; }
 
-// order: room for the splat's item order (one int2 per work item; the fixed-array render
-// takes its items in tile order).
+// order: room for the splat's item order (one int2 per work item; the fixed-array render has its
+// own).
 static void layout_var(FrameHost &fh, int64_t pairs, int items, int splits, bool pids, bool order = true) {
     fh.pair_cap = pairs;
     fh.item_cap = items;
@@ -1448,12 +1448,15 @@ extern "C" splotch_status splotch_compose_maps(const float *maps, int32_t n_maps
 // process exits.
 
 static constexpr size_t kStaticBytes = size_t(32) << 20;          // 32 MiB per GPU
+// and, behind them, the splat's work order: an entry per tile and per full slice of the most pairs
+// that fit
+static constexpr int kStaticItems = kMaxTiles + (int)(kStaticBytes / sizeof(float4)) / kMinItemPairs;
 static constexpr int64_t kStaticRelBudget = int64_t(2) << 20;      // chunk bases: 2 MiB of it
 static constexpr int kStaticSplits = 256;                          // split-tile scratch slots
 static constexpr size_t kStaticSplitBytes = size_t(8) << 20;       // and at most 8 MiB for them
 static constexpr int kMaxDevices = 64;
 
-static __device__ __align__(256) unsigned char g_static_ws[kStaticBytes];
+static __device__ __align__(256) unsigned char g_static_ws[kStaticBytes + sizeof(int2) * kStaticItems];
 
 static std::mutex g_static_mu;
 static void *g_static_addr[kMaxDevices];  // device address of g_static_ws, per device
@@ -1510,11 +1513,12 @@ extern "C" splotch_status splotch_render_noalloc(splotch_scene *sc, const splotc
         return fail(SPLOTCH_ERR_UNSUPPORTED, "%d tiles of %d px need %zu bytes of tables, more than the %zu-byte fixed workspace",
                     vp.n_tiles, T, fixed + scratch, kStaticBytes);
     const int64_t pairs = (int64_t)((kStaticBytes - fixed - scratch - 1024) / sizeof(float4));
-    layout_var(fh, pairs, INT32_MAX, splits, false, false);
+    layout_var(fh, pairs, kStaticItems, splits, false, false);
     if (fixed + fh.var_bytes > kStaticBytes)
         return fail(SPLOTCH_ERR_UNSUPPORTED, "fixed workspace layout overflow");
     char *var = base + fixed;
     FrameDev fr = frame_dev(fh, base, var);
+    fr.order = (int2 *)(base + kStaticBytes);
 
     // every call shares the array: the accumulators of split tiles start at zero
     cudaStream_t st = (cudaStream_t)stream;

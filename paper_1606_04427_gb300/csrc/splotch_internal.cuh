@@ -86,7 +86,7 @@ struct FrameDev {
     unsigned long long *scratch;  // [split capacity][3][T][T][2] exact accumulators (fix_add)
     int *tickets;                 // [split capacity]
     int2 *order;                  // [item capacity] work items (tile, slice of its list), largest
-                                  // first (k_item_order), or null: items in tile order
+                                  // first (k_item_order)
     int64_t pair_cap;
     int item_cap, split_cap;
     const float *vscale;      // [V * n_types] emission scale per view and species, or null
@@ -422,8 +422,7 @@ cudaError_t launch_gather_records(const float4 *src, const uint32_t *idx, uint32
 int ordered_split(int T);
 int ordered_ctas_per_sm();
 int ordered_workers_per_sm();
-// Work items of the frame ordered largest first into fr.order (k_item_order; no-op when
-// fr.order is null).
+// Work items of the frame ordered largest first into fr.order (k_item_order).
 cudaError_t launch_item_order(const FrameDev &fr, cudaStream_t st);
 cudaError_t launch_splat_ordered(const SceneDev &sc, const FrameDev &fr, float *out, const float *absorb,
                                  float *ord_scratch, int map_out, int grid, int splits, cudaStream_t st);
