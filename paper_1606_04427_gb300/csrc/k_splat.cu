@@ -80,8 +80,12 @@ __device__ __forceinline__ int team_of(int64_t records, int64_t K, int64_t warps
 
 // Size bin from which a team shares an item: an eighth of K, 256 records (from a quarter, 50 k
 // particles at 256^2 take 48 us instead of 35), for teams of 2 a quarter (from an eighth, 1 M uniform
-// particles at 2048^2 take 167 us against 151).
-__device__ __forceinline__ int shared_from(int team) { return team > 2 ? kOrderBins / 8 : kOrderBins / 4; }
+// particles at 2048^2 take 167 us against 151).  Twice that where a region is a part of its tile and
+// keeps a part of the list: 1 M single-pixel particles at 2501^2 (tiles of 24) take 122 us instead of
+// 218, and tiles of 64 at 256^2 lose what sharing gives 50 k clustered ones if it is four times.
+__device__ __forceinline__ int shared_from(int team, int split) {
+    return (team > 2 ? kOrderBins / 8 : kOrderBins / 4) * min(split, 2);
+}
 
 // Barrier of one team's warps (`team` of them, a power of two).
 __device__ __forceinline__ void team_sync(int team) {
@@ -441,7 +445,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
         int few = kFew;
         if (kn.team > 1) {
             // by the slice's length: that of the order, also where the region has no pixel
-            if (order_bin(len, (int)K) >= shared_from(kn.team)) {
+            if (order_bin(len, (int)K) >= shared_from(kn.team, split)) {
                 // this warp's consecutive part of the slice
                 const int part = ((nrec + kn.team - 1) / kn.team + 31) & ~31;
                 const int first = min(nrec, (me >> 5) * part);

@@ -75,3 +75,9 @@ def test_regions_of_14_pixels_take_no_longer_per_pixel():
     """Nor are the rows of regions of 14 pixels aligned: per pixel, a frame of 10 k particles took 1.4
     times as long at 5000^2 (tiles of 40) as at 4096^2 (tiles of 32)."""
     assert _frame_ms(5000, 10_000) / 5000 ** 2 < 1.2 * _frame_ms(4096, 10_000) / 4096 ** 2
+
+
+def test_more_particles_are_not_faster():
+    """Lists of 300 records in tiles of 24 pixels: shared by teams of four, whose parts then hold a few
+    records of a region, 1 M particles took 1.4 times as long as 1.2 M in teams of two."""
+    assert _frame_ms(2501, 1_000_000, 0.6) < 1.15 * _frame_ms(2501, 1_200_000, 0.6)
