@@ -144,9 +144,26 @@ __device__ __forceinline__ void finish_item(const FrameDev &fr, float *out, int 
         // together (read one by one, a warp's 24 trips to memory: 485 instead of 338 us for 400 k
         // clustered particles added to an image of 3958 x 4096).
         const int lane = threadIdx.x & 31;
+        if (kAlone && blank) {  // a = 0
+            if (out_accum == 2) return;
+            if (wide) {
+                for (int k = lane; k < th * 12; k += 32) {
+                    const int r = k / 12;
+                    *reinterpret_cast<float4 *>(reg + (int64_t)r * W * 3 + 4 * (k - 12 * r)) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                }
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < 3; ++j) {
+                    const int odd = 32 * j + lane >= 3 * kRegion, c = 32 * j + lane - 3 * kRegion * odd;
+                    float *to = reg + (int64_t)odd * W * 3 + c;
+                    if (c / 3 < tw)
+                        for (int p = 0; 2 * p + odd < th; ++p) to[(int64_t)p * 6 * W] = 0.0f;
+                }
+            }
+            return;
+        }
         float *held = reinterpret_cast<float *>(ws->batch.pa) + (wide ? 4 : 1) * lane;
         static_assert(sizeof(ws->batch.pa) >= 3 * kRegion * kRegion * sizeof(float), "a region's values");
-        if (kAlone && blank && out_accum == 2) return;  // adds nothing
         if (out_accum == 2) {
             if (wide) {
                 for (int k = me, i = 0; k < th * 12; k += unit, i += 128)
@@ -165,14 +182,11 @@ __device__ __forceinline__ void finish_item(const FrameDev &fr, float *out, int 
         if (wide) {
             for (int k = me, i = 0; k < th * 12; k += unit, i += 128) {
                 const int r = k / 12, c = 4 * (k - 12 * r);
-                float4 u = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (!kAlone || !blank) {
-                    u = *reinterpret_cast<float4 *>(held + i);
-                    u.x = pixel(u.x, sums[(c + 0) % 3][r][(c + 0) / 3], out_accum);
-                    u.y = pixel(u.y, sums[(c + 1) % 3][r][(c + 1) / 3], out_accum);
-                    u.z = pixel(u.z, sums[(c + 2) % 3][r][(c + 2) / 3], out_accum);
-                    u.w = pixel(u.w, sums[(c + 3) % 3][r][(c + 3) / 3], out_accum);
-                }
+                float4 u = *reinterpret_cast<float4 *>(held + i);
+                u.x = pixel(u.x, sums[(c + 0) % 3][r][(c + 0) / 3], out_accum);
+                u.y = pixel(u.y, sums[(c + 1) % 3][r][(c + 1) / 3], out_accum);
+                u.z = pixel(u.z, sums[(c + 2) % 3][r][(c + 2) / 3], out_accum);
+                u.w = pixel(u.w, sums[(c + 3) % 3][r][(c + 3) / 3], out_accum);
                 *reinterpret_cast<float4 *>(reg + (int64_t)r * W * 3 + c) = u;
             }
         } else {
@@ -185,11 +199,6 @@ __device__ __forceinline__ void finish_item(const FrameDev &fr, float *out, int 
                 if (col >= tw) continue;
                 const float *from = &sums[c - 3 * col][odd][col];
                 float *to = reg + (int64_t)odd * W * 3 + c;
-                if (kAlone && blank) {
-#pragma unroll 4
-                    for (int p = 0; 2 * p + odd < th; ++p) to[(int64_t)p * 6 * W] = 0.0f;
-                    continue;
-                }
 #pragma unroll 4
                 for (int p = me >> 5; 2 * p + odd < th; p += team)
                     to[(int64_t)p * 6 * W] = pixel(held[32 * (kRegion / 2 * j + p)], from[2 * kRegion * p], out_accum);
