@@ -21,8 +21,8 @@
 // composes far to near.
 //
 // What bounds it: the FP32 pipe (68 % of its cycles on the 10 M-particle two-species frame; a packed
-// operation holds it two).  Hence the short polynomials (9 or 10 packed operations per channel and
-// two pixels, 15 with the exponential) and squares of 4 x 4 pixels: 6.7 squares, 107 pixel
+// operation holds it two).  Hence the short polynomials (9, 10 or 12 packed operations per channel
+// and two pixels, 15 with the exponential) and squares of 4 x 4 pixels: 6.7 squares, 107 pixel
 // evaluations per particle, against 235 in the 8 x 8 units of a warp per record.  10 M particles at
 // 2048^2: 3.33 ms with a warp per record, 1.64 and 0.05 for the composition now (1.52 with the
 // cheaper and less accurate update named below); a frame of 1 M particles as maps at 1000 x 757:
@@ -49,22 +49,28 @@ struct __align__(16) OWarpSmem {
 // where s = 0 stood for 2^-40 / E.  Emulated against 64 bits for 1 to 200 records, x from 0.001 to 2,
 // the present form is nowhere less accurate than a beta + b with a and b rounded apart.)
 // phi is a polynomial whose degree follows the step's largest x (w <= 1, so a record's x is at most
-// its s E): degree 3 up to kDeg3Max and 4 up to kDeg4Max, minimax with phi(0) = 1 (fitted here by
-// iteratively reweighted least squares against expm1 in 64 bits; largest relative errors 8.0e-9 and
-// 3.0e-9).  Beyond, and for negative emissions, the Taylor polynomial of degree 5 where
-// |x| <= kDeg4Max (next term x^6 / 7! <= 5e-8) and the exponential itself elsewhere:
+// its s E): degree 3 up to kDeg3Max, 4 up to kDeg4Max and 6 up to kDeg6Max, minimax with phi(0) = 1
+// (fitted here by iteratively reweighted least squares against expm1 in 64 bits; largest relative
+// errors 8.0e-9, 3.0e-9 and 9.3e-9).  Beyond, and for negative emissions, the Taylor polynomial of
+// degree 5 where |x| <= kDeg4Max (next term x^6 / 7! <= 5e-8) and the exponential itself elsewhere:
 // alpha <- a alpha, beta <- a beta + (1 - a) / s, a = exp(-x).  (A degree 2 up to 0.015 as well: 10 M
 // particles at 2048^2 in 3.15 instead of 3.11 ms, a step's 16 records are rarely all below.)
-constexpr float kDeg3Max = 0.1f, kDeg4Max = 0.25f;
+constexpr float kDeg3Max = 0.1f, kDeg4Max = 0.25f, kDeg6Max = 1.0f;
 
 // phi as a polynomial in -x (all coefficients positive)
-template <int kDeg> __device__ __forceinline__ float2 phi_of(float2 nx) {  // degree 3, 4 or 5 (Taylor)
+template <int kDeg> __device__ __forceinline__ float2 phi_of(float2 nx) {  // degree 3, 4, 6 or 5 (Taylor)
     float2 phi;
     if (kDeg == 5) {
         phi = __ffma2_rn(nx, f2(1.0f / 720.0f), f2(1.0f / 120.0f));
         phi = __ffma2_rn(nx, phi, f2(1.0f / 24.0f));
         phi = __ffma2_rn(nx, phi, f2(1.0f / 6.0f));
         phi = __ffma2_rn(nx, phi, f2(0.5f));
+    } else if (kDeg == 6) {
+        phi = __ffma2_rn(nx, f2(0.000129130945f), f2(0.00130112655f));
+        phi = __ffma2_rn(nx, phi, f2(0.00827620924f));
+        phi = __ffma2_rn(nx, phi, f2(0.0416474678f));
+        phi = __ffma2_rn(nx, phi, f2(0.166663662f));
+        phi = __ffma2_rn(nx, phi, f2(0.499999851f));
     } else if (kDeg == 4) {
         phi = __ffma2_rn(nx, f2(0.00753017422f), f2(0.0415001325f));
         phi = __ffma2_rn(nx, phi, f2(0.166652888f));
@@ -252,6 +258,8 @@ __global__ void __launch_bounds__(kOWarps * 32, 6)
                         apply_record<3>(pa, pb, fx, fy, al, be);
                     else if (most <= __float_as_uint(kDeg4Max))
                         apply_record<4>(pa, pb, fx, fy, al, be);
+                    else if (most <= __float_as_uint(kDeg6Max))
+                        apply_record<6>(pa, pb, fx, fy, al, be);
                     else
                         apply_record<5>(pa, pb, fx, fy, al, be);
                 }

@@ -38,9 +38,12 @@ def _apart(beta):
 # x's own rounding moves phi by at most x / 2 x 2^-24 = 7.4e-9, the rounding of phi's inner terms by
 # 4e-9, and the polynomial is off by 8e-9: 1.2e-7 in all.  Roundings have no sign: over 240000
 # values their mean is below 1e-9, and a polynomial's mean error is below its largest.
+# For x up to 1, phi is above 0.63 and the inner terms count more: 6.0e-8 for the product, 4.8e-8
+# for phi, 3.6e-8 for its inner terms, 2.5e-8 for x's rounding, 9.3e-9 for the polynomial.
 @pytest.mark.parametrize("s", [0.3, 1.5, 7.0])
-@pytest.mark.parametrize("xmax", [0.0148, 0.04, 0.099, 0.2, 0.249])
-def test_one_record_rounds_without_bias(xmax, s):
+@pytest.mark.parametrize("xmax,tol", [(0.0148, 1.2e-7), (0.04, 1.2e-7), (0.099, 1.2e-7), (0.2, 1.2e-7), (0.249, 1.2e-7),
+                                      (0.26, 1.8e-7), (0.99, 1.8e-7)])
+def test_one_record_rounds_without_bias(xmax, tol, s):
     sc, cam, e = _apart(xmax / s)
     got = sc.render_ordered(cam, [s]).cpu().numpy().astype(np.float64)
     assert (got[e == 0] == 0).all()
@@ -48,7 +51,7 @@ def test_one_record_rounds_without_bias(xmax, s):
     s = float(np.float32(s))
     rel = got[on] * s / -np.expm1(-s * e[on].astype(np.float64)) - 1.0
     assert on.sum() > 200_000
-    assert np.abs(rel).max() <= 1.2e-7
+    assert np.abs(rel).max() <= tol
     assert abs(rel.mean()) <= 9e-9
 
 
