@@ -381,8 +381,9 @@ splotch_status splotch_last_timing(double ms[4], int64_t counts[3]);
  * this serves callers that cannot allocate while they render (a host application that
  * owns all device memory through its own manager, a real-time loop that forbids
  * allocation after start-up, since an allocation can block on the device).  The frame
- * workspace lives in a fixed 32 MiB device array inside this library, present on every
- * GPU that loads the library until the process exits.  The caller passes the scene
+ * workspace lives in a fixed 32 MiB device array inside this library (and 136 KiB behind it
+ * for the splat's work order), present on every GPU that loads the library until the process
+ * exits.  The caller passes the scene
  * (created earlier with splotch_create_scene, on the device that is current for this
  * call: INVALID_ARG otherwise), the camera, the parameters and `out` (device, H x W x 3
  * FP32), as for splotch_render.  The first call on a device looks up that device's copy

@@ -20,13 +20,13 @@
 // is not split writes beta; the slices of a split tile store their maps, which k_compose_slices
 // composes far to near.
 //
-// What bounds it: the FP32 pipe (68 % of its cycles on the 10 M-particle two-species frame; a packed
+// What bounds it: the FP32 pipe (67 % of its cycles on the 10 M-particle two-species frame; a packed
 // operation holds it two).  Hence the short polynomials (9, 10 or 12 packed operations per channel
 // and two pixels, 15 with the exponential) and squares of 4 x 4 pixels: 6.7 squares, 107 pixel
 // evaluations per particle, against 235 in the 8 x 8 units of a warp per record.  10 M particles at
-// 2048^2: 3.33 ms with a warp per record, 1.64 and 0.05 for the composition now (1.52 with the
+// 2048^2: 3.33 ms with a warp per record, 1.66 and 0.05 for the composition now (1.52 with the
 // cheaper and less accurate update named below); a frame of 1 M particles as maps at 1000 x 757:
-// 1.22 -> 0.59 ms (0.55).  Batches of 192 (12 warps per SM): 128 on 16 warps took 2.47 ms where 192
+// 1.24 -> 0.55 ms (0.55).  Batches of 192 (12 warps per SM): 128 on 16 warps took 2.47 ms where 192
 // took 2.21.
 #include "splat_batch.cuh"
 

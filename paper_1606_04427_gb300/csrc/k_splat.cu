@@ -637,9 +637,9 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
 typedef void (*SplatFn)(SceneDev, FrameDev, int *, float *, int, int);
 
 // Regions per tile edge.  Each reads its tile's whole list and keeps a part of it.  At tiles of 32 /
-// 40 / 48 / 64 pixels (10 M particles at 2048^2) the splat takes 0.86 / 1.03 / 1.00 / 1.24 ms, where a
-// CTA per tile above 32 pixels that read the list once took 3.81 / 4.50 / 4.95; 20 M at 8192^2 (64
-// pixels) 8.72 against 32.2 ms, 200 k at 5000^2 (40 pixels) 0.44 against 0.43.
+// 40 / 48 / 64 pixels (10 M particles at 2048^2) the splat takes 0.85 / 1.03 / 1.02 / 1.30 ms, where a
+// CTA per tile above 32 pixels that read the list once took 3.80 / 4.52 / 4.91; 20 M at 8192^2 (64
+// pixels) 8.75 against 32.3 ms, 200 k at 5000^2 (40 pixels) 0.27 against 0.43.
 int splat_split(int T) { return (T + kRegion - 1) / kRegion; }
 
 static SplatFn splat_fn(bool scaled, bool emit, bool wild) {
